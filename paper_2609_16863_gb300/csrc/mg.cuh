@@ -1169,44 +1169,93 @@ static __global__ void k_dense_level(FineDesc fd, double* Adense) {
     }
 }
 
-// In-place Gauss--Jordan inverse (SPD input, no pivoting needed), one block.
-static __global__ void __launch_bounds__(1024) k_gauss_jordan(double* A, double* Inv, int n, int* fail) {
+// Gauss--Jordan inverses (SPD input, no pivoting needed) of the coarsest level's matrices, one cluster
+// of kGjCtas CTAs per matrix.  Bound by FP64 arithmetic: n^3 multiply-adds at about two per cycle and
+// SM, so one CTA needs 9.0 ms for n = 256 while the rest of the chip idles.  Here CTA r keeps rows
+// r, r + kGjCtas, ... in shared memory (in place: column k of the inverse replaces column k of A, half
+// the arithmetic of an augmented matrix); the owner of pivot row k + 1 updates and scales that row
+// first and stores it into every CTA's buffer, then all CTAs eliminate their rows with pivot row k,
+// so one cluster barrier per pivot is left.  The same pivots and products as elimination of [A | I].
+constexpr int kGjCtas = 16;
+constexpr int kGjThreads = 512;
+
+inline size_t gj_smem(int n) {
+    return ((size_t)((n + kGjCtas - 1) / kGjCtas) * n + 2 * (size_t)n) * sizeof(double);
+}
+
+static __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan(const double* Ain, double* Inv, int n, int* fail) {
     pdl_prologue();
-    // one CTA; warps take rows, lanes take columns; the scaled pivot rows live in shared memory
-    __shared__ double prow[kMaxCoarsest], pinvrow[kMaxCoarsest];
-    __shared__ double piv;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = w; i < n; i += nw)
-        for (int j = lane; j < n; j += 32) Inv[i * n + j] = i == j ? 1.0 : 0.0;
+    extern __shared__ __align__(16) double gj_sm[];
+    unsigned rank, mat;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(mat));
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = kGjThreads / 32;
+    const int nr = n > (int)rank ? (n - (int)rank + kGjCtas - 1) / kGjCtas : 0;   // own rows
+    double* prow = gj_sm;                       // two pivot rows, scaled by 1 / pivot
+    double* R = gj_sm + 2 * n;
+    const double* A = Ain + (long long)mat * n * n;
+    for (int i = w; i < nr; i += nw)
+        for (int j = lane; j < n; j += 32) R[i * n + j] = A[(long long)(rank + i * kGjCtas) * n + j];
     __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            piv = A[k * n + k];
-            if (!(piv > 0.0)) *fail = 1;
-        }
-        __syncthreads();
+    // row i minus its column k times pivot row k; the pivot's own entry becomes 1 / pivot there, so
+    // column k of every other row becomes -f / pivot
+    auto eliminate = [&](double* row, const double* pr, int k) {
+        const double f = row[k];
+        __syncwarp();
+        for (int j = lane; j < n; j += 32) row[j] = j == k ? -f * pr[j] : row[j] - f * pr[j];
+    };
+    auto publish = [&](int k) {                 // the owner: scale row k, store it into every CTA
+        double* row = R + (k / kGjCtas) * n;
+        const double piv = row[k];
+        if (tid == 0 && !(piv > 0.0)) *fail = 1;
         const double pinv = 1.0 / piv;
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            const double a = A[k * n + j] * pinv, v = Inv[k * n + j] * pinv;
-            A[k * n + j] = a;
-            Inv[k * n + j] = v;
-            prow[j] = a;
-            pinvrow[j] = v;
-        }
         __syncthreads();
-        for (int i = w; i < n; i += nw) {
-            if (i == k) continue;
-            const double f = A[i * n + k];
-            for (int j = lane; j < n; j += 32) {
-                if (j != k) A[i * n + j] -= f * prow[j];
-                Inv[i * n + j] -= f * pinvrow[j];
+        for (int j = tid; j < n; j += kGjThreads) {
+            const double v = j == k ? pinv : row[j] * pinv;
+            row[j] = v;
+            double* dst = prow + (k & 1) * n + j;
+            for (unsigned c = 0; c < kGjCtas; ++c) {
+                unsigned long long q;
+                asm volatile("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"(dst), "r"(c));
+                *reinterpret_cast<double*>(q) = v;
             }
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            if (i != k) A[i * n + k] = 0.0;
-        __syncthreads();
+    };
+    auto cluster_barrier = [] {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    };
+    cluster_barrier();                          // every CTA has started before the first remote store
+    if (rank == 0) publish(0);
+    cluster_barrier();
+    for (int k = 0; k < n; ++k) {
+        const double* pr = prow + (k & 1) * n;
+        const bool ahead = k + 1 < n && (k + 1) % kGjCtas == (int)rank;
+        const int ia = (k + 1) / kGjCtas;
+        if (ahead) {
+            if (w == 0) eliminate(R + ia * n, pr, k);
+            __syncthreads();
+            publish(k + 1);                     // buffer (k + 1) & 1: last read before the previous barrier
+        }
+        for (int i = w; i < nr; i += nw) {
+            if ((int)rank + i * kGjCtas == k || (ahead && i == ia)) continue;
+            eliminate(R + i * n, pr, k);
+        }
+        cluster_barrier();
     }
+    double* O = Inv + (long long)mat * n * n;
+    for (int i = w; i < nr; i += nw)
+        for (int j = lane; j < n; j += 32) O[(long long)(rank + i * kGjCtas) * n + j] = R[i * n + j];
+}
+
+// Invert nmat consecutive n x n matrices; *fail is set when a pivot is not positive.
+inline aao_status launch_gauss_jordan(const double* A, double* Inv, int n, int nmat, int* fail, cudaStream_t st) {
+    AAO_CUDA_TRY(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)gj_smem(kMaxCoarsest)));
+    AAO_CUDA_TRY(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    launch_cluster(k_gauss_jordan, dim3(kGjCtas * nmat), dim3(kGjThreads), gj_smem(n), st, kGjCtas, A, Inv, n, fail);
+    AAO_LAUNCH_CHECK();
+    return AAO_OK;
 }
 
 // Per-component max |coef| (one block per component) and conversion to S.

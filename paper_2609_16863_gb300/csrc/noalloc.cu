@@ -194,8 +194,7 @@ extern "C" aao_status aao_rk_shifted_solve_noalloc(const aao_grid* grid, double 
     launch(k_dense_level, (unsigned)((nc + 127) / 128), 128, 0, st, fd, dense);
     // the scratch keeps the previous call's contents: the breakdown flag must start at zero
     AAO_CUDA_TRY(cudaMemsetAsync(fail, 0, sizeof(int), st));
-    launch(k_gauss_jordan, 1, 1024, 0, st, dense, dinv, nc, fail);
-    AAO_LAUNCH_CHECK();
+    AAO_TRY(launch_gauss_jordan(dense, dinv, nc, 1, fail, st));
     LevelOp<double> ops[kMaxLevels];
     for (int l = 0; l < L; ++l) {
         LevelOp<double>& op = ops[l];

@@ -242,8 +242,9 @@ class Precond : public PrecondBase {
         const int ncst = (int)gcst.nx;
         double *dense, *dinv64;
         int* fail;
-        AAO_TRY(ar.alloc(&dense, (size_t)ncst * ncst));
-        AAO_TRY(ar.alloc(&dinv64, (size_t)ncst * ncst));
+        const long long nn = (long long)ncst * ncst;
+        AAO_TRY(ar.alloc(&dense, (size_t)(s * nn)));
+        AAO_TRY(ar.alloc(&dinv64, (size_t)(s * nn)));
         AAO_TRY(ar.alloc(&fail, 1));
         AAO_CUDA_TRY(cudaMemsetAsync(fail, 0, sizeof(int), st()));
         for (int i = 0; i < s; ++i) {
@@ -292,12 +293,15 @@ class Precond : public PrecondBase {
                 cd.c = 0;
                 cd.sten = sten64[L - 1];
             }
-            launch(k_dense_level, (unsigned)((ncst + 127) / 128), 128, 0, st(), cd, dense);
-            launch(k_gauss_jordan, 1, 1024, 0, st(), dense, dinv64, ncst, fail);
+            launch(k_dense_level, (unsigned)((ncst + 127) / 128), 128, 0, st(), cd, dense + i * nn);
             AAO_LAUNCH_CHECK();
-            AAO_TRY(ar.alloc(&Dinv[i], (size_t)ncst * ncst));
-            launch(k_convert_dense<A>, (unsigned)(((long long)ncst * ncst + 255) / 256), 256, 0, st(), 
-                dinv64, Dinv[i], (long long)ncst * ncst);
+        }
+        // the stages' coarsest inverses in one launch, a cluster each
+        AAO_TRY(launch_gauss_jordan(dense, dinv64, ncst, s, fail, st()));
+        for (int i = 0; i < s; ++i) {
+            AAO_TRY(ar.alloc(&Dinv[i], (size_t)nn));
+            launch(k_convert_dense<A>, (unsigned)((nn + 255) / 256), 256, 0, st(), (const double*)(dinv64 + i * nn),
+                   Dinv[i], nn);
             AAO_LAUNCH_CHECK();
         }
         int hfail = 0;
