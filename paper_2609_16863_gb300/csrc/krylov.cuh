@@ -118,19 +118,30 @@ __global__ void __launch_bounds__(kBlock) k_mgs(int n0, long long rows, int B, c
     block_finish((double)acc, b, red, out + (long long)b * hstride, dot ? 0 : 1);
 }
 
-// out_b = src_b / denom[b * dstride]  (any storage); inactive items skipped.
+// Per-step state of the Schur substitution, in device memory so that one
+// captured step can be replayed for every n: z (output vector), r (input
+// vector) and the step index n.
+struct StepPtrs {
+    double* z;
+    const double* r;
+    int n;
+};
+
+// out_b = src_b / denom[b * dstride]  (any storage); inactive items skipped.  rep > 0: the source
+// has rep rows per item, which repeat.  sp: also advance the recurrence's step index.
 template <class SO, class SR>
 __global__ void __launch_bounds__(kPtMaxThreads) k_scale_store(PtMap pm, int rows, int B, const int* active, const SR* src,
                                                       long long sbs, const double* denom, long long dstride,
-                                                      Vec<SO> out) {
+                                                      Vec<SO> out, int rep, StepPtrs* sp) {
     pdl_prologue();
+    if (sp && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) sp->n += 1;
     using A = typename PT<SO>::A;
     PtPos q = pt_pos(pm, B, rows, active);
     if constexpr (!PT<SO>::scaled) {
         if (!q.valid) return;
     }
     const int n0 = pm.n0;
-    const SR* x = src + (long long)q.b * sbs + q.row * n0;
+    const SR* x = src + (long long)q.b * sbs + (rep ? q.row % rep : q.row) * n0;
     // the reciprocal in the arithmetic type: an FP64 division per thread is slow on this GPU
     A inv = (denom && q.valid) ? A(1) / A(denom[(long long)q.b * dstride]) : A(1);
     SO* o; float* osc;
@@ -195,32 +206,6 @@ static __global__ void k_givens(int B, int k, int kmax, double* H, long long hs,
     if (res <= tol * beta_ref[b] || hk1 == 0.0 || k == kmax - 1) active[b] = 0;
 }
 
-// Start of a batched inner solve: items with beta == 0 are done at once (z = 0).
-static __global__ void k_inner_init(int B, int kmax, const double* beta, int* active, int* its, double* g, int* nonfinite) {
-    pdl_prologue();
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    double bt = beta[b];
-    if (!isfinite(bt)) atomicExch(nonfinite, 1);
-    active[b] = (bt > 0.0 && isfinite(bt)) ? 1 : 0;
-    its[b] = 0;
-    for (int i = 0; i <= kmax; ++i) g[(long long)b * (kmax + 1) + i] = i == 0 ? bt : 0.0;
-}
-
-static __global__ void k_count_its(int B, const int* its, long long* count) {
-    pdl_prologue();
-    __shared__ long long sh[128];
-    long long t = 0;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) t += its[b];
-    sh[threadIdx.x] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long a = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) a += sh[i];
-        *count += a;
-    }
-}
-
 // y = R^{-1} g (R the rotated upper triangle, its[b] columns), per item.
 static __global__ void k_hess_solve(int B, int kmax, const double* H, long long hs, const double* g, const int* its,
                              double* y, int* breakdown) {
@@ -267,41 +252,6 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_combine(PtMap pm, int rows, i
             acc += (A)y[(long long)q.b * kmax + k] * z.at(q.row, c);
         }
         o[c] = (SO)acc;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Theta_hat z (Eq. discretized_system_stages with M = I):
-//   w_i = z_i + tau sum_j coef[i*s + j] K z_j,  coef = A_RK (or A_RK^T).
-// One warp per (item, spatial row); every stage of the row at once.
-// ---------------------------------------------------------------------------
-template <class SZ, class A>
-__global__ void __launch_bounds__(kPtMaxThreads) k_theta(Geo g, PtMap pm, int B, const int* active, Vec<SZ> Z, A* wv,
-                                                long long wbs, int s, const double* coef, A tau, SpaceOp<A> sop) {
-    pdl_prologue();
-    // tau a_ij in the arithmetic type, once per block (the products the per-point sum uses)
-    __shared__ A tc[kMaxS * kMaxS];
-    for (int t = threadIdx.y * blockDim.x + threadIdx.x; t < s * s; t += blockDim.x * blockDim.y)
-        tc[t] = tau * (A)coef[t];
-    __syncthreads();
-    PtPos q = pt_pos(pm, B, g.R, active);
-    if (!q.valid) return;
-    const long long row = q.row;
-    int j, k;
-    row_jk(g, row, j, k);
-    A* out = wv + (long long)q.b * wbs + row * g.n0;
-    for (int c = q.c0; c < g.n0; c += pm.n0p) {
-        A kz[kMaxS];
-        for (int i = 0; i < s; ++i) {
-            View<SZ> zi = view_of(Z, q.b, (long long)i * g.nx, g.n0);
-            kz[i] = (A)op_K(zi, g, sop, row, j, k, c);
-        }
-        for (int i = 0; i < s; ++i) {
-            View<SZ> zi = view_of(Z, q.b, (long long)i * g.nx, g.n0);
-            A acc = (A)op_M(zi, g, sop, row, j, k, c);
-            for (int jj = 0; jj < s; ++jj) acc += tc[i * s + jj] * kz[jj];
-            out[(long long)i * g.nx + c] = acc;
-        }
     }
 }
 
@@ -390,15 +340,6 @@ __global__ void k_schur_g(long long nx, int nt, int s, const double* r, const do
     wbuf[i] = v;
 }
 
-// Per-step state of the Schur substitution, in device memory so that one
-// captured step can be replayed for every n: z (output vector), r (input
-// vector) and the step index n.
-struct StepPtrs {
-    double* z;
-    const double* r;
-    int n;
-};
-
 static __global__ void k_step_set(StepPtrs* sp, double* z, const double* r, int n) {
     pdl_prologue();
     sp->z = z;
@@ -408,54 +349,6 @@ static __global__ void k_step_set(StepPtrs* sp, double* z, const double* r, int 
 
 static __global__ void k_step_add(StepPtrs* sp, int d) {
     pdl_prologue(); sp->n += d; }
-
-// t_i = K z_{v,n} for every stage i (the e (x) K z_{v,n} right-hand side).
-template <class A>
-__global__ void __launch_bounds__(kBlock) k_schur_rhs(Geo g, int s, const StepPtrs* sp, A* t, SpaceOp<A> sop) {
-    pdl_prologue();
-    long long row = gwarp();
-    if (row >= g.R) return;
-    int j, k;
-    row_jk(g, row, j, k);
-    View<double> z{sp->z + (long long)sp->n * g.nx, nullptr, g.n0};
-    for (int c = lane_id(); c < g.n0; c += kWarp) {
-        A v = (A)op_K(z, g, sop, row, j, k, c);
-        for (int i = 0; i < s; ++i) t[(long long)i * g.nx + row * g.n0 + c] = v;
-    }
-}
-
-// z_{v,n+1} = w_{n+1} + z_{v,n} - tau sum_i b_i q_i,  q = sum_k y_k Z_k (item 0).
-template <class SZ, class A>
-__global__ void __launch_bounds__(kBlock) k_schur_update(Geo g, int s, const A* wbuf, const StepPtrs* sp,
-                                                         Vec<SZ> Z0, long long zstride, const double* y,
-                                                         int kmax, const int* its, const double* bw,
-                                                         double tau) {
-    pdl_prologue();
-    long long row = gwarp();
-    if (row >= g.R) return;
-    const int n = sp->n;
-    const A* wn1 = wbuf + (long long)(n + 1) * g.nx;
-    const double* zvn = sp->z + (long long)n * g.nx;
-    double* zvn1 = sp->z + (long long)(n + 1) * g.nx;
-    int m = its[0];
-    A coef[kMaxInner * kMaxS];
-    for (int k = 0; k < m; ++k)
-        for (int i = 0; i < s; ++i) coef[k * s + i] = (A)(tau * bw[i] * y[k]);
-    for (int c = lane_id(); c < g.n0; c += kWarp) {
-        long long p = row * g.n0 + c;
-        A acc = wn1[p] + (A)zvn[p];
-        for (int k = 0; k < m; ++k) {
-            Vec<SZ> Zk = Z0;
-            Zk.d += k * zstride;
-            if constexpr (PT<SZ>::scaled) Zk.sc += (k * zstride) / g.n0;
-            for (int i = 0; i < s; ++i) {
-                View<SZ> z = view_of(Zk, 0, (long long)i * g.nx, g.n0);
-                acc -= coef[k * s + i] * z.at(row, c);
-            }
-        }
-        zvn1[p] = (double)acc;
-    }
-}
 
 // Transposed substitution: t_i = b_i u_{n+1}.
 template <class A>
@@ -498,57 +391,6 @@ __global__ void __launch_bounds__(kBlock) k_schurT_update(Geo g, int s, const St
 // the C-point residual w_{n+1} + Phi(z_n) - z_{n+1} of item b into block b + 1 of
 // res (transposed: block nres - 1 - b) instead of updating the recurrence.
 // ---------------------------------------------------------------------------
-template <class A>
-__global__ void __launch_bounds__(kBlock) k_schur_rhs_b(Geo g, int s, const StepPtrs* sp, int stride, A* t,
-                                                        SpaceOp<A> sop) {
-    pdl_prologue();
-    long long row = gwarp();
-    if (row >= g.R) return;
-    const int b = blockIdx.y;
-    int j, k;
-    row_jk(g, row, j, k);
-    View<double> z{sp->z + (long long)(sp->n + b * stride) * g.nx, nullptr, g.n0};
-    A* tb = t + (long long)b * s * g.nx;
-    for (int c = lane_id(); c < g.n0; c += kWarp) {
-        A v = (A)op_K(z, g, sop, row, j, k, c);
-        for (int i = 0; i < s; ++i) tb[(long long)i * g.nx + row * g.n0 + c] = v;
-    }
-}
-
-template <class SZ, class A>
-__global__ void __launch_bounds__(kBlock) k_schur_update_b(Geo g, int s, const A* wbuf, const StepPtrs* sp,
-                                                           int stride, Vec<SZ> Z0, long long zstride,
-                                                           const double* y, int kmax, const int* its,
-                                                           const double* bw, double tau, A* res) {
-    pdl_prologue();
-    long long row = gwarp();
-    if (row >= g.R) return;
-    const int b = blockIdx.y;
-    const int n = sp->n + b * stride;
-    const A* wn1 = wbuf + (long long)(n + 1) * g.nx;
-    const double* zvn = sp->z + (long long)n * g.nx;
-    double* zvn1 = sp->z + (long long)(n + 1) * g.nx;
-    const int m = its[b];
-    A coef[kMaxInner * kMaxS];
-    for (int k = 0; k < m; ++k)
-        for (int i = 0; i < s; ++i) coef[k * s + i] = (A)(tau * bw[i] * y[(long long)b * kmax + k]);
-    for (int c = lane_id(); c < g.n0; c += kWarp) {
-        long long p = row * g.n0 + c;
-        A acc = wn1[p] + (A)zvn[p];
-        for (int k = 0; k < m; ++k) {
-            Vec<SZ> Zk = Z0;
-            Zk.d += k * zstride;
-            if constexpr (PT<SZ>::scaled) Zk.sc += (k * zstride) / g.n0;
-            for (int i = 0; i < s; ++i) {
-                View<SZ> z = view_of(Zk, b, (long long)i * g.nx, g.n0);
-                acc -= coef[k * s + i] * z.at(row, c);
-            }
-        }
-        if (res) res[(long long)(b + 1) * g.nx + p] = acc - (A)zvn1[p];
-        else zvn1[p] = (double)acc;
-    }
-}
-
 // Transposed: t_{b,i} = b_i u_{n_b + 1}.
 template <class A>
 __global__ void k_schurT_rhs_b(long long nx, int s, const StepPtrs* sp, int stride, const double* bw, A* t) {

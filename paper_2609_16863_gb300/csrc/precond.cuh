@@ -17,6 +17,7 @@
 #include <memory>
 #include <type_traits>
 
+#include "arnoldi.cuh"
 #include "cluster_mg.cuh"
 #include "handle.cuh"
 #include "mg.cuh"
@@ -59,6 +60,9 @@ class Precond : public PrecondBase {
     double *Hh = nullptr, *csh = nullptr, *snh = nullptr, *gh = nullptr, *yh = nullptr, *betah = nullptr;
     int *activeh = nullptr, *itsh = nullptr, *nonfin = nullptr, *brk = nullptr;
     long long* itcount = nullptr;  // running total of inner iterations (device)
+    double* gramh = nullptr;       // products of the basis vectors, kin*kin per item
+    double* ar_part = nullptr;     // partial sums of the Arnoldi kernels
+    unsigned int* ar_count = nullptr;   // their arrival counters, Bmax, zero between launches
     // Schur state
     A* wbuf = nullptr;             // (nt+1)*nx
     A* tbuf = nullptr;             // s*nx
@@ -351,6 +355,10 @@ class Precond : public PrecondBase {
         AAO_TRY(ar.alloc(&gh, (size_t)Bmax * (kin + 1)));
         AAO_TRY(ar.alloc(&yh, (size_t)Bmax * kin));
         AAO_TRY(ar.alloc(&betah, (size_t)Bmax));
+        AAO_TRY(ar.alloc(&gramh, (size_t)Bmax * kin * kin));
+        AAO_TRY(ar.alloc(&ar_part, (size_t)(kArBlocks + Bmax) * (2 * (kin <= kArSmallK ? kArSmallK : kMaxInner) - 1)));
+        AAO_TRY(ar.alloc(&ar_count, (size_t)Bmax));
+        AAO_CUDA_TRY(cudaMemsetAsync(ar_count, 0, sizeof(unsigned int) * Bmax, st()));
         AAO_TRY(ar.alloc(&activeh, (size_t)Bmax));
         AAO_TRY(ar.alloc(&itsh, (size_t)Bmax));
         AAO_TRY(ar.alloc(&nonfin, 2));
@@ -944,6 +952,13 @@ class Precond : public PrecondBase {
                 }
             }
             bytes_hint(1.0 * nact * g.nx * (sizeof(SP) + (transpose ? s - 1 - i : i) * sizeof(SI) + sizeof(SI)));
+            if constexpr (!PT<SI>::scaled) {
+                if (!h->q1) {
+                    launch_rana_vec(B, act, V, i, Z, transpose);
+                    AAO_TRY(mg_solve(i, B, act, mgb, Zi));
+                    continue;
+                }
+            }
             launch(k_rana_rhs<SP, SI>, pt_grid(pm0, g.R, B), pt_block(pm0), 0, st(), g, pm0, B, act, V, i, Z, s,
                    coef, (A)h->tau, sopA, mgb);
             AAO_LAUNCH_CHECK();
@@ -953,65 +968,184 @@ class Precond : public PrecondBase {
     }
 
     // ------------------------------------------------------- inner GMRES
+    static constexpr int kVN = (int)(16 / sizeof(A));    // points per thread where rows are whole vectors
+    bool rows_vec() const { return h->g.n0 % kVN == 0 && !h->q1; }
+    template <class F> static void with_int(bool big, F&& f) {     // f(std::true_type) or f(std::false_type)
+        if (big) f(std::true_type{});
+        else f(std::false_type{});
+    }
+    static bool aligned16(const void* p) { return (reinterpret_cast<unsigned long long>(p) & 15ULL) == 0; }
+
+    // Blocks per item of the Arnoldi kernels: one position per thread while that gives fewer than kArBlocks
+    // blocks (eight per SM) over the batch, else the blocks stride over the item.
+    ArRed ar_red(int B, long long positions) const {
+        const long long full = (positions + kArThreads - 1) / kArThreads, cap = (kArBlocks + B - 1) / B;
+        ArRed r;
+        r.part = ar_part;
+        r.count = ar_count;
+        r.nchunk = (int)std::max<long long>(1, std::min(full, cap));
+        return r;
+    }
+    ArItems ar_items() const {
+        ArItems it;
+        it.kin = kin;
+        it.H = Hh;
+        it.cs = csh;
+        it.sn = snh;
+        it.g = gh;
+        it.beta = betah;
+        it.y = yh;
+        it.gram = gramh;
+        it.active = activeh;
+        it.its = itsh;
+        it.nonfinite = nonfin;
+        it.breakdown = brk;
+        it.count = itcount;
+        it.tol = itol;
+        return it;
+    }
+    template <class S> Basis<S> basis_of(const Vec<S>& v, long long stride) const {
+        return Basis<S>{v, stride, (long long)h->s * h->g.R, stride / h->g.n0};
+    }
+
+    // v = src / denom per item of s*n_x values (rep: src is one stage of n_x, used for every stage).
+    template <class SR>
+    void scale_basis(int B, const SR* src, long long sbs, const double* denom, long long dstride, Vec<SP> v, int rep,
+                     StepPtrs* sp) {
+        const Geo& g = h->g;
+        const long long item = (long long)h->s * g.nx;
+        if constexpr (PT<SP>::scaled) {
+            const PtMap pm = ptmap(g.n0);
+            const int rows = h->s * g.R;
+            launch(k_scale_store<SP, SR>, pt_grid(pm, rows, B), pt_block(pm), 0, st(), pm, rows, B,
+                   (const int*)activeh, src, sbs, denom, dstride, v, rep ? g.R : 0, sp);
+        } else {
+            constexpr int U = 2;
+            const bool vec = g.n0 % kVN == 0 && (sizeof(SR) != sizeof(SP) || aligned16(src));
+            with_int(vec, [&](auto big) {
+                constexpr int N = decltype(big)::value ? kVN : 1;
+                const long long per = (long long)U * kArThreads * N, n = rep ? g.nx : item;
+                launch(k_scale_vec<SP, SR, N, U>, dim3((unsigned)((n + per - 1) / per), (unsigned)B), kArThreads, 0,
+                       st(), item, g.nx, rep ? h->s : 0, (const int*)activeh, src, sbs, denom, dstride, v, sp);
+            });
+        }
+    }
+
+    void launch_rana_vec(int B, const int* act, Vec<SP> V, int i, Vec<SI> Z, int transpose) {
+        const Geo& g = h->g;
+        const int s = h->s;
+        StageCoef<A> cf{};
+        cf.j0 = transpose ? i + 1 : 0;
+        cf.j1 = transpose ? s : i;
+        for (int j = cf.j0; j < cf.j1; ++j)
+            cf.c[j] = (A)h->tau * (A)(transpose ? h->L[j * s + i] * h->D[i] : h->L[i * s + j] * h->D[j]);
+        with_int(rows_vec(), [&](auto big) {
+            constexpr int N = decltype(big)::value ? kVN : 1;
+            const long long pos = (long long)(g.n0 / N) * g.R;
+            const dim3 grid((unsigned)((pos + kArThreads - 1) / kArThreads), (unsigned)B);
+            with_int(s > 3, [&](auto many) {
+                constexpr int TS = decltype(many)::value ? kMaxS : 3;
+                launch(k_rana_vec<SP, SI, N, TS>, grid, kArThreads, 0, st(), g, inv_h2<A>(g), act, V, i, Z, cf, facesA,
+                       mgb);
+            });
+        });
+    }
+
+    // The Krylov steps of B items whose v_0 is in place (ar_init has run): on exit Z0 / yh / itsh hold
+    // every item's solution.
+    aao_status arnoldi(int B, int transpose) {
+        const Geo& g = h->g;
+        const int s = h->s;
+        const long long item = (long long)s * g.nx;
+        const unsigned rows = (unsigned)s * (unsigned)g.R;
+        const Basis<SP> V = basis_of(V0, vstride);
+        const ArItems it = ar_items();
+        refresh_nact(B);
+        for (int k = 0; k < kin; ++k) {
+            Vec<SP> Vk = shift_vec(V0, k * vstride, g.n0);
+            Vec<SI> Zk = shift_vec(Z0, k * zstride, g.n0);
+            AAO_TRY(rana(B, activeh, Vk, Zk, transpose));
+            with_int(rows_vec(), [&](auto big) {
+                constexpr int N = decltype(big)::value ? kVN : 1;
+                const long long pos = (long long)(g.n0 / N) * g.R;
+                const ArRed rt = ar_red(B, pos), ru = ar_red(B, s * pos);
+                with_int(kin > kArSmallK, [&](auto deep) {
+                    constexpr int MK = decltype(deep)::value ? kMaxInner : kArSmallK;
+                    with_int(s > 3, [&](auto many) {
+                        constexpr int TS = decltype(many)::value ? kMaxS : 3;
+                        bytes_hint(1.0 * nact * item * (sizeof(SI) + sizeof(A) + (k + 1) * sizeof(SP)));
+                        launch(k_theta_dots<SI, SP, A, N, TS, MK>, dim3((unsigned)rt.nchunk, (unsigned)B), kArThreads,
+                               0, st(), g, inv_h2<A>(g), (const int*)activeh, Zk, (long long)rows, wv, item, s,
+                               (const double*)(transpose ? h->d_AT : h->d_A), (A)h->tau, sopA, V, k, rt, it);
+                    });
+                    bytes_hint(1.0 * nact * item * (2 * sizeof(A) + (k + 1) * sizeof(SP)));
+                    launch(k_arnoldi_upd<SP, A, N, MK>, dim3((unsigned)ru.nchunk, (unsigned)B), kArThreads, 0, st(),
+                           g.n0, rows, (const int*)activeh, wv, item, V, k, ru, it);
+                });
+            });
+            AAO_LAUNCH_CHECK();
+            refresh_nact(B);
+            if (k + 1 < kin)
+                scale_basis<A>(B, wv, item, Hh + (k + 1) * kin + k, (long long)(kin + 1) * kin,
+                               shift_vec(V0, (k + 1) * vstride, g.n0), 0, nullptr);
+            AAO_LAUNCH_CHECK();
+        }
+        return AAO_OK;
+    }
+
+    // out_b = sum_k y_k Z_k of every item.
+    template <class SO> void combine(int B, SO* out, long long obs) {
+        const Geo& g = h->g;
+        const unsigned rows = (unsigned)h->s * (unsigned)g.R;
+        with_int(g.n0 % kVN == 0 && (!std::is_same<SO, double>::value || std::is_same<A, float>::value || aligned16(out)),
+                 [&](auto big) {
+            constexpr int N = decltype(big)::value ? kVN : 1;
+            const long long pos = (long long)(g.n0 / N) * rows;
+            launch(k_combine_vec<SI, SO, N>, dim3((unsigned)((pos + kArThreads - 1) / kArThreads), (unsigned)B),
+                   kArThreads, 0, st(), g.n0, rows, basis_of(Z0, zstride), (const double*)yh, kin, (const int*)itsh, out,
+                   obs);
+        });
+    }
+
     // Batched GMRES(kin) on Theta_hat (or Theta_hat^T) for B items of s*nx;
     // rhs item b at src + b*sbs (type SR, unscaled).  On exit Z0/yh/itsh hold the
     // Krylov solution of every item; out (if given) receives sum_k y_k Z_k.
     template <class SR>
     aao_status inner(int B, const SR* src, long long sbs, double* out, long long obs, int transpose) {
+        const long long item = (long long)h->s * h->g.nx;
+        const ArRed red = ar_red(B, item / 4 + 1);
+        launch(k_ar_start<SR>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), item, src, sbs, red,
+               ar_items());
+        scale_basis<SR>(B, src, sbs, (const double*)betah, 1LL, V0, 0, nullptr);
+        AAO_LAUNCH_CHECK();
+        AAO_TRY(arnoldi(B, transpose));
+        if (out) combine<double>(B, out, obs);
+        AAO_LAUNCH_CHECK();
+        return AAO_OK;
+    }
+
+    // One forward step of S_tilde's recurrence for B items, time index sp->n + b * stride (advanced by
+    // one): t = K z_n, Theta_tilde^{-1} (e (x) t), and z_{n+1} or its C-point residual.
+    aao_status forward_step(int B, int stride, const A* w, A* res) {
         const Geo& g = h->g;
         const int s = h->s;
-        const long long item = (long long)s * g.nx;
-        const long long rows = (long long)s * g.R;
-        const PtMap pm0 = ptmap(g.n0);
-        const dim3 nbp = pt_grid(pm0, rows, B), ntp = pt_block(pm0);
-        Red red = h->red;
-        red.nchunk = h->nchunk_for(B, rows * ((g.n0 + kWarp - 1) / kWarp));
-        dim3 rgrid(red.nchunk, B);
-        launch(k_norm<SR>, rgrid, kBlock, 0, st(), g.n0, rows, B, nullptr, src, sbs, red, betah, 1);
-        launch(k_inner_init, (B + 127) / 128, 128, 0, st(), B, kin, betah, activeh, itsh, gh, nonfin);
-        refresh_nact(B);
-        launch(k_scale_store<SP, SR>, nbp, ntp, 0, st(), pm0, (int)rows, B, activeh, src, sbs, (const double*)betah, 1LL, V0);
+        const H2FF h2{to_ff(g.hx2), to_ff(g.hy2), to_ff(g.hz2)};
+        with_int(rows_vec(), [&](auto big) {
+            constexpr int N = decltype(big)::value ? kVN : 1;
+            const ArRed red = ar_red(B, (long long)(g.n0 / N) * g.R);
+            launch(k_schur_start<A, N>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g, h2, s,
+                   (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
+        });
+        scale_basis<A>(B, tbuf, g.nx, (const double*)betah, 1LL, V0, 1, stepp);
         AAO_LAUNCH_CHECK();
-        const long long HS = (long long)(kin + 1) * kin;
-        for (int k = 0; k < kin; ++k) {
-            Vec<SP> Vk = shift_vec(V0, k * vstride, g.n0);
-            Vec<SI> Zk = shift_vec(Z0, k * zstride, g.n0);
-            AAO_TRY(rana(B, activeh, Vk, Zk, transpose));
-            bytes_hint(1.0 * nact * item * (sizeof(SI) + sizeof(A)));
-            launch(k_theta<SI, A>, pt_grid(pm0, g.R, B), pt_block(pm0), 0, st(), g, pm0, B, (const int*)activeh, Zk,
-                   wv, item, s, transpose ? h->d_AT : h->d_A,
-                                                     (A)h->tau, sopA);
-            AAO_LAUNCH_CHECK();
-            // modified Gram--Schmidt: h_{0,k} = V_0.w; then w -= h_{i-1,k} V_{i-1}, h_{i,k} = V_i.w
-            Vec<SP> none{};
-            bytes_hint(1.0 * nact * item * (sizeof(A) + sizeof(SP)));
-            launch(k_mgs<SP, A>, rgrid, kBlock, 0, st(), g.n0, rows, B, activeh, wv, item, none, nullptr, V0, HS,
-                                                     red, Hh + k);
-            for (int i = 1; i <= k + 1; ++i) {
-                Vec<SP> Vp = shift_vec(V0, (i - 1) * vstride, g.n0);
-                Vec<SP> Vn = i <= k ? shift_vec(V0, i * vstride, g.n0) : none;
-                bytes_hint(1.0 * nact * item * (2 * sizeof(A) + (i <= k ? 2 : 1) * sizeof(SP)));
-                launch(k_mgs<SP, A>, rgrid, kBlock, 0, st(), g.n0, rows, B, activeh, wv, item, Vp,
-                                                         Hh + (i - 1) * kin + k, Vn, HS, red, Hh + i * kin + k);
-            }
-            launch(k_givens, (B + 127) / 128, 128, 0, st(), B, k, kin, Hh, HS, csh, snh, gh, betah, itol, activeh, itsh,
-                                                        nonfin, nullptr);
-            AAO_LAUNCH_CHECK();
-            refresh_nact(B);
-            if (k + 1 < kin) {
-                Vec<SP> Vn = shift_vec(V0, (k + 1) * vstride, g.n0);
-                launch(k_scale_store<SP, A>, nbp, ntp, 0, st(), pm0, (int)rows, B, (const int*)activeh, (const A*)wv, item,
-                                                              Hh + (k + 1) * kin + k, HS, Vn);
-                AAO_LAUNCH_CHECK();
-            }
-        }
-        launch(k_hess_solve, (B + 127) / 128, 128, 0, st(), B, kin, Hh, HS, gh, itsh, yh, brk);
-        launch(k_count_its, 1, 128, 0, st(), B, itsh, itcount);
-        if (out) {
-            Vec<SI> Zc = Z0;
-            launch(k_combine<SI, double>, nbp, ntp, 0, st(), pm0, (int)rows, B, Zc, zstride, (const double*)yh, kin,
-                   (const int*)itsh, out, obs, 0);
-        }
+        AAO_TRY(arnoldi(B, 0));
+        with_int(g.n0 % kVN == 0, [&](auto big) {
+            constexpr int N = decltype(big)::value ? kVN : 1;
+            const long long pos = (long long)(g.n0 / N) * g.R;
+            launch(k_schur_finish<SI, A, N>, dim3((unsigned)((pos + kArThreads - 1) / kArThreads), (unsigned)B),
+                   kArThreads, 0, st(), g, s, w, (const StepPtrs*)stepp, stride, basis_of(Z0, zstride), (const double*)yh,
+                   kin, (const int*)itsh, (const double*)h->d_b, h->tau, res);
+        });
         AAO_LAUNCH_CHECK();
         return AAO_OK;
     }
@@ -1025,20 +1159,12 @@ class Precond : public PrecondBase {
         const long long item = (long long)s * g.nx;
         const unsigned nbr = blocks_for_rows(g.R);
         if (!transpose) {
-            launch(k_schur_rhs<A>, nbr, kBlock, 0, st(), g, s, (const StepPtrs*)stepp, tbuf, sopA);
-            AAO_TRY(inner<A>(1, tbuf, item, nullptr, 0, 0));
-            launch(k_schur_update<SI, A>, nbr, kBlock, 0, st(), g, s, wsrc ? wsrc : (const A*)wbuf,
-                   (const StepPtrs*)stepp, Z0,
-                   zstride, (const double*)yh, kin, (const int*)itsh, (const double*)h->d_b, h->tau);
-            launch(k_step_add, 1, 1, 0, st(), stepp, 1);
+            AAO_TRY(forward_step(1, 0, wsrc ? wsrc : (const A*)wbuf, nullptr));
         } else {
             launch(k_schurT_rhs<A>, (unsigned)((item + 255) / 256), 256, 0, st(), g.nx, s, (const StepPtrs*)stepp,
                    (const double*)h->d_b, tbuf);
             AAO_TRY(inner<A>(1, tbuf, item, nullptr, 0, 1));
-            Vec<SI> Zc = Z0;
-            launch(k_combine<SI, A>, pt_grid(ptmap(g.n0), (long long)s * g.R, 1), pt_block(ptmap(g.n0)), 0, st(), ptmap(g.n0),
-                   s * g.R, 1,
-                   Zc, zstride, (const double*)yh, kin, (const int*)itsh, qbuf, item, 0);
+            combine<A>(1, qbuf, item);
             launch(k_schurT_update<A>, nbr, kBlock, 0, st(), g, s, (const StepPtrs*)stepp, (const A*)qbuf, h->tau,
                    sopA);
             launch(k_step_add, 1, 1, 0, st(), stepp, -1);
@@ -1056,21 +1182,12 @@ class Precond : public PrecondBase {
         const long long item = (long long)s * g.nx;
         const unsigned nbr = blocks_for_rows(g.R);
         if (!transpose) {
-            launch(k_schur_rhs_b<A>, dim3(nbr, (unsigned)B), kBlock, 0, st(), g, s, (const StepPtrs*)stepp, stride, tbuf,
-                   sopA);
-            AAO_TRY(inner<A>(B, tbuf, item, nullptr, 0, 0));
-            launch(k_schur_update_b<SI, A>, dim3(nbr, (unsigned)B), kBlock, 0, st(), g, s, (const A*)wbuf,
-                   (const StepPtrs*)stepp, stride, Z0, zstride, (const double*)yh, kin, (const int*)itsh,
-                   (const double*)h->d_b, h->tau, residual ? coarse->wbuf : (A*)nullptr);
-            launch(k_step_add, 1, 1, 0, st(), stepp, 1);
+            AAO_TRY(forward_step(B, stride, wbuf, residual ? coarse->wbuf : (A*)nullptr));
         } else {
             launch(k_schurT_rhs_b<A>, dim3((unsigned)((item + 255) / 256), (unsigned)B), 256, 0, st(), g.nx, s,
                    (const StepPtrs*)stepp, stride, (const double*)h->d_b, tbuf);
             AAO_TRY(inner<A>(B, tbuf, item, nullptr, 0, 1));
-            const PtMap pm = ptmap(g.n0);
-            Vec<SI> Zc = Z0;
-            launch(k_combine<SI, A>, pt_grid(pm, (long long)s * g.R, B), pt_block(pm), 0, st(), pm, s * g.R, B, Zc,
-                   zstride, (const double*)yh, kin, (const int*)itsh, qbuf, item, 0);
+            combine<A>(B, qbuf, item);
             launch(k_schurT_update_b<A>, dim3(nbr, (unsigned)B), kBlock, 0, st(), g, s, (const StepPtrs*)stepp, stride,
                    (const A*)qbuf, h->tau, sopA, residual ? rbufT : (double*)nullptr, B);
             launch(k_step_add, 1, 1, 0, st(), stepp, -1);
@@ -1393,7 +1510,8 @@ class Precond : public PrecondBase {
         nact = 1;
         launch(k_scale_store<SI, double>, pt_grid(ptmap(g.n0), g.R, 1), pt_block(ptmap(g.n0)), 0, st(), ptmap(g.n0), g.R, 1,
                (const int*)nullptr, b, g.nx,
-                                                                             nullptr, 0, mgb);
+                                                                             nullptr, 0, mgb, 0,
+               (StepPtrs*)nullptr);
         AAO_LAUNCH_CHECK();
         Vec<SI> out = Z0;   // item 0, stage 0 of the first Z basis
         AAO_TRY(mg_solve(stage, 1, nullptr, mgb, out));
@@ -1409,7 +1527,7 @@ class Precond : public PrecondBase {
         const long long rows = (long long)h->s * g.R;
         launch(k_scale_store<SP, double>, pt_grid(ptmap(g.n0), rows, 1), pt_block(ptmap(g.n0)), 0, st(), ptmap(g.n0),
                (int)rows, 1, (const int*)nullptr, r,
-                                                                              (long long)h->s * g.nx, nullptr, 0, V0);
+                                                                              (long long)h->s * g.nx, nullptr, 0, V0, 0, (StepPtrs*)nullptr);
         AAO_LAUNCH_CHECK();
         AAO_TRY(rana(1, nullptr, V0, Z0, transpose));
         launch(k_load<SI, double>, pt_grid(ptmap(g.n0), rows, 1), pt_block(ptmap(g.n0)), 0, st(), ptmap(g.n0), (int)rows, 1,

@@ -565,7 +565,7 @@ static aao_status fgmres(Handle* h, const double* b, double* x, int x0_given, in
             if (total >= h->opt.maxit) break;
             Vec<double> V0{h->V, nullptr, nst};
             launch(k_scale_store<double, double>, nbp, ntp, 0, st, pmo, (int)rows, 1, (const int*)nullptr, (const double*)h->r, nst,
-                   (const double*)h->beta, 0LL, V0);
+                   (const double*)h->beta, 0LL, V0, 0, (StepPtrs*)nullptr);
             launch(k_outer_init, 1, 32, 0, st, h->gv, m, h->beta, h->flags);
             AAO_LAUNCH_CHECK();
             bool stop = false;
@@ -605,7 +605,7 @@ static aao_status fgmres(Handle* h, const double* b, double* x, int x0_given, in
                 if (!h->hsmall->active || total >= h->opt.maxit) break;
                 Vec<double> Vn{h->V + (long long)(k + 1) * nst, nullptr, nst};
                 launch(k_scale_store<double, double>, nbp, ntp, 0, st, pmo, (int)rows, 1, (const int*)nullptr, (const double*)h->w, nst,
-                                                                     h->H + (k + 1) * m + k, 0, Vn);
+                                                                     h->H + (k + 1) * m + k, 0, Vn, 0, (StepPtrs*)nullptr);
                 AAO_LAUNCH_CHECK();
             }
             if (stop) break;
@@ -707,7 +707,7 @@ static aao_status fgmres_left(Handle* h, const double* b, double* x, int x0_give
             if (total >= h->opt.maxit) break;
             Vec<double> V0{h->V, nullptr, nst};
             launch(k_scale_store<double, double>, nbp, ntp, 0, st, pmo, (int)rows, 1, (const int*)nullptr,
-                   (const double*)h->w, nst, (const double*)h->beta, 0LL, V0);
+                   (const double*)h->w, nst, (const double*)h->beta, 0LL, V0, 0, (StepPtrs*)nullptr);
             launch(k_outer_init, 1, 32, 0, st, h->gv, m, h->beta, h->flags);
             AAO_LAUNCH_CHECK();
             bool stop = false;
@@ -745,7 +745,7 @@ static aao_status fgmres_left(Handle* h, const double* b, double* x, int x0_give
                 if (!h->hsmall->active || total >= h->opt.maxit) break;
                 Vec<double> Vn{h->V + (long long)(k + 1) * nst, nullptr, nst};
                 launch(k_scale_store<double, double>, nbp, ntp, 0, st, pmo, (int)rows, 1, (const int*)nullptr,
-                       (const double*)h->w, nst, h->H + (k + 1) * m + k, 0, Vn);
+                       (const double*)h->w, nst, h->H + (k + 1) * m + k, 0, Vn, 0, (StepPtrs*)nullptr);
                 AAO_LAUNCH_CHECK();
             }
             if (stop) break;
