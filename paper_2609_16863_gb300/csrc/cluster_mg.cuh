@@ -1,36 +1,47 @@
-// Cluster-resident multigrid for one 2D item (the Schur sweep's shifted
-// solves (M + c_i K) x = b, Sec. 5: three V-cycles per stage solve).
+// Cluster-resident multigrid for 2D items (the Schur sweep's shifted solves (M + c_i K) x = b, Sec. 5:
+// three V-cycles per stage solve).
 //
-// The V-cycles of one shifted solve are a chain of ~30 dependent grid-wide
-// steps per cycle; as separate launches each step costs a launch latency.
-// Here one thread-block cluster (up to 16 CTAs, one per SM) runs all cycles:
-//   * every level above the coarsest is split by grid rows over the CTAs; a
-//     CTA keeps its rows of x (two ping-pong buffers), b, the stored stencil
-//     and the Jacobi weights in shared memory;
-//   * x / b rows are stored with a zero column on each side and a ghost row
-//     above and below the CTA's range, so stencils, restriction and
-//     interpolation read without bounds tests (the zeros stand for the
-//     Dirichlet boundary and add exact zeros);
-//   * a step that writes a CTA's first or last row also stores that row into
-//     the neighbouring CTA's ghost row (distributed shared memory, generic
-//     addresses from `mapa`), so after the cluster barrier that ends the step
-//     every read is local;
-//   * the level-l partition follows the finest one: coarse row J belongs to
-//     the CTA owning fine row 2J+1, so restriction and interpolation only ever
-//     touch one row beyond a CTA's range;
-//   * the coarsest level (at most a few hundred unknowns) is held whole by
-//     every CTA: each CTA restricts its right-hand side from all CTAs'
-//     residual rows, applies its own slice of rows of the dense inverse
-//     (staged once per launch) and gathers the other slices after a cluster
-//     barrier;
-//   * the Jacobi weights omega / a_PP are staged once per launch, so a sweep
-//     is x + w (b - A x) without a division.
-// Operator applications, residuals, restriction and interpolation follow the
-// level kernels in mg.cuh (same formulas and summation order); intermediate
-// vectors stay on chip in the arithmetic type.
+// The V-cycles of one shifted solve are a chain of about 30 dependent grid-wide steps per cycle.  One
+// thread-block cluster per item (16 CTAs for single items, 8 for batches) runs the chain on chip:
+//   * every level above the coarsest is split by grid rows over the CTAs; a CTA keeps its rows of x (two
+//     ping-pong buffers), b, the stored stencil and the Jacobi weights in shared memory, with H ghost
+//     rows on each side and zero columns beside the grid (the Dirichlet boundary);
+//   * the level-l partition follows the finest one: coarse row J belongs to the CTA owning fine row
+//     2J+1, so restriction and interpolation touch at most one row beyond what they produce for;
+//   * the coarsest level (at most a few hundred unknowns) is held whole by every CTA: each CTA
+//     restricts its rows into every CTA's copy of b, applies its slice of rows of the dense inverse and
+//     stores the results into every CTA's copy of x.
+//
+// What bounds it is latency and instruction supply.  Measured on 16 CTAs of 512 threads (2.07 GHz): a
+// block barrier costs 45 cycles, a cluster barrier 137 without and 521 with its release fence, an exchange
+// of edge rows (remote stores, barrier) 790 cycles; a step's own work was 850 cycles even for two
+// rows, most of it call and index overhead and instruction fetches.  So:
+//   * a step's result is computed on as many ghost rows as its inputs reach (`ext`), and rows are
+//     exchanged only when a step has none left: with H = 3 (4 on the finest level, whose iterate
+//     enters a cycle nonzero) a level needs two exchanges per cycle, of b after the restriction and of x
+//     after the last sweep, instead of five; the redundant rows fit the threads that a step leaves
+//     idle.  H = 1 exchanges after every sweep; levels fall back to it where shared memory is short and
+//     everywhere in FP64, whose rate (two operations per cycle and SM) makes redundant rows dearer;
+//   * the cycle is a program of 8-byte operations laid out by the host (cl_program), run by one loop
+//     in which every kind of step is instantiated once: sweeps, zero-guess sweeps and residuals are the
+//     same instructions with other coefficients;
+//   * what does not change between launches (stencils, weights, faces, the slice of the coarsest
+//     inverse) is laid out once per handle as each CTA's shared-memory image, padded rows included, and
+//     copied linearly;
+//   * a thread keeps one 16-byte vector of columns and walks down consecutive rows with the rows around
+//     it in registers; on the finest level (FD, kappa = 1) the sweep's constants are folded, x + w (b - A x)
+//     = k0 P + kx (W + E) + ky (S + N) + w b, six operations per point instead of ten.  Rows are padded
+//     to whole vectors with zeros, so odd widths take the same path.
+//
+// One launch of three V(2,2)-cycles, one item on 16 CTAs (event-timed, before -> now): FP32 256^2 77.9 -> 69.3 us,
+// 128^2 53.7 -> 47.9, 127 x 95 57.5 -> 47.7, 64^2 39.2 -> 34.5, Q1 80 x 72 53.4 -> 50.1; FP64 256^2 332 -> 270
+// (FP64-bound), 64^2 69.2 -> 60.7, 32^2 45.1 -> 37.0; eight to fifteen items of 256^2 on 8 CTAs each 97 -> 93.
+// Deep ghost regions against single ghost rows on the new kernel: 256^2 68 against 82, 64^2 FP64 60.1 against 60.3.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "mg.cuh"
 
@@ -40,91 +51,100 @@ constexpr int kClMax = 16;            // CTAs per cluster (16 needs the non-port
 constexpr int kClThreads = 512;
 constexpr int kClMaxBatch = 32;       // batches of at most this many items run one cluster per item
 constexpr int kClBatch8 = 8;          // batches of at least this many items take the 8-CTA plan
-constexpr int kClPad = 4;             // columns before a row's first point (column -1 is the last of them) and
-                                      // after its last (column n0 the first): rows start 16-byte aligned
+constexpr int kClPad = 4;             // columns before a row's first point and after its last vector: rows
+                                      // start 16-byte aligned, the columns beside the grid are zero
+constexpr int kClReach = 3;           // CTAs on either side whose ghost rows may hold a CTA's rows
+constexpr int kClMaxLevels = 10;      // 2D levels of grids that fit a cluster
 
+// Columns per thread: one 16-byte vector in FP32.  FP64 takes single columns: a step's chain of FP64 operations
+// is long, and twice the warps hide twice as much of it.
+template <class A> struct ClVec;
+template <> struct ClVec<float> {
+    using T = float4;
+    static constexpr int n = 4;
+};
+template <> struct ClVec<double> {
+    using T = double;
+    static constexpr int n = 1;
+};
+
+// Plan of one shift (a kernel parameter: every field is read through the constant bank).
 template <class SI> struct ClCtx {
     using A = typename PT<SI>::A;
     int C, L, T;                          // cluster size, levels, T = L-1 (the replicated coarsest level)
     int cycles, nu1, nu2;
-    A omega;
+    int fine0, has_faces;                 // level 0 is the FD operator; with faces of a kappa field
     A sigma, c;                           // level 0 (FD): sigma I + c K
-    int fine0, has_faces;
-    Geo g[kMaxLevels];
-    unsigned magic[kMaxLevels];           // ceil(2^32 / n0_l): p / n0_l = umulhi(p, magic) for p*n0_l < 2^32
-    int rlo[kMaxLevels][kClMax + 1];      // distributed level l: CTA r owns rows [rlo[l][r], rlo[l][r+1])
-    int maxr[kMaxLevels];                 // rows per CTA in the shared-memory layout (n1 for l >= T)
-    int off[kMaxLevels];                  // A-element offset of level l's X0 | X1 | B, each (maxr+2) x (n0+2)
-    int soff[kMaxLevels];                 // A-element offset of level l's staged stencil (9 x maxr*n0; -1: none)
-    int woff[kMaxLevels];                 // A-element offset of omega / a_PP (maxr*n0; -1: coarsest)
-    int fxoff, fyoff;                     // level 0 faces: maxr rows of n0+1 | maxr+1 rows of n0
+    A hx2, hy2;
+    A w0, k0, kx, ky;                     // FD, kappa = 1: omega / a_PP; the folded sweep
+    A d0, ex, ey;                         // FD, kappa = 1: A u = d0 P - ex (W + E) - ey (S + N)
+    int fuse0;                            // 1: level 0 takes two zero-guess sweeps at once (mode 3)
+    int n0[kClMaxLevels], n1[kClMaxLevels];
+    int nvp[kClMaxLevels];                // vectors per padded row
+    unsigned magicv[kClMaxLevels];        // ceil(2^32 / nvp): tid / nvp = umulhi(tid, magicv)
+    unsigned magic[kClMaxLevels];         // ceil(2^32 / n0)
+    int per[kClMaxLevels];                // rows per thread
+    int H[kClMaxLevels];                  // ghost rows
+    int ix[kClMaxLevels];                 // rows of the x inbox per side
+    int maxr[kClMaxLevels];               // own rows in the shared-memory layout
+    int rlo[kClMaxLevels][kClMax + 1];    // CTA r owns rows [rlo[l][r], rlo[l][r+1]) (the coarsest: computes them)
+    int off[kClMaxLevels];                // A-element offset of level l's X0 | X1 | B, each (maxr + 2H) x ld
+    int ioff[kClMaxLevels];               // x inbox: 2 ix rows of ld
+    int soff[kClMaxLevels];               // staged stencil, 9 x (maxr + 2(H-1)) x padded row (-1: none)
+    int woff[kClMaxLevels];               // omega / a_PP, (maxr + 2H) x padded row (-1: the scalar w0)
+    int sten_global[kClMaxLevels];        // 1: level l's stencil is read from global memory (L2), not staged
+    int fxoff, fyoff;                     // level 0 faces: rows of ld | rows of the padded width
+    int dinv_global;                      // 1: the rows of A_c^{-1} are read from global memory
+    int dinv_off, boff;                   // this CTA's rows of A_c^{-1}, each padded to ncp; the coarsest b (ncp)
+    int ncp;                              // unknowns of the coarsest level, rounded up to vectors
     int cs[kClMax + 1];                   // coarsest rows [cs[r], cs[r+1]) of A_c^{-1} b are computed by CTA r
-    int dinv_off;                         // A-element offset of this CTA's rows of A_c^{-1} (max rows * nc)
-    int rowtab_off;                       // A-element offset (8-byte aligned) of the row table of level T-1
+    int img_off, img_len;                 // the staged constants: A elements [img_off, img_off + img_len)
+    int prog_off;                         // byte offset of the program in shared memory (part of the image)
+    int pc[4];                            // operations of the first cycle, of odd and of even later cycles
+    int kfin;                             // buffer of x_0 after the last cycle
+    const A* img;                         // C images
     const A* fx;
     const A* fy;
-    const SI* sten[kMaxLevels];
-    const float* sten_sc[kMaxLevels];
-    const A* Dinv;
-    // lean plans (a cluster of 8 for batches, where the full layout does not fit shared memory):
-    int sten_global[kMaxLevels];          // 1: level l's stencil is read from global memory (L2), not staged
-    int dinv_global;                      // 1: the rows of A_c^{-1} are read from global memory
-    int w0_const;                         // 1: level 0's omega / a_PP is one scalar (FD, kappa = 1)
-    int vec[kMaxLevels];                  // 1: level l's sweeps and residual take 16-byte vectors of points
-    unsigned magicv[kMaxLevels];          // ceil(2^32 / (n0_l / points per vector))
+    const SI* sten[kClMaxLevels];
+    const float* sten_sc[kClMaxLevels];
+    const A* W[kClMaxLevels];             // omega / a_PP of every point (null: w0)
+    const A* Dinv;                        // rows of ncp values (dinv_global and the image's source: nc)
 };
 
-// This CTA's share of a distributed level.
-template <class A> struct ClLev {
-    int a, nr;                // own rows [a, a + nr)
-    A* pu[3];                 // ghost row below the range of the previous non-empty CTA (buffers X0, X1, B;
-                              // first interior column), or nullptr
-    A* pd[3];                 // ghost row above the range of the next non-empty CTA
+// One operation of the cycle's program.
+enum ClKind { kClStep, kClRestrict, kClRestrictLast, kClSolve, kClProlong, kClInbox, kClClear };
+struct ClOp {
+    unsigned char kind, lev;
+    unsigned char mode;                   // step: 0 sweep, 1 sweep of a zero guess, 2 residual, 3 two sweeps of a
+                                          // zero guess at once; restriction: also the first sweep (1)
+    unsigned char kin;                    // buffer read (prolong: x_f's)
+    unsigned char kc;                     // prolong: buffer of x_c; step: buffer written; restriction: of the sweep
+    unsigned char ext;                    // ghost rows computed
+    unsigned char depth;                  // ghost rows stored into the other CTAs (0: none)
+    unsigned char flags;                  // 1: into the x inboxes; 2: cluster barrier
 };
+static_assert(sizeof(ClOp) == 8, "one 8-byte load");
 
-// One level as a step sees it (built once per launch in shared memory; a step copies it to
-// registers only in warps that have points of the level).
-template <class A> struct ClL {
-    int n0, n1, nr, a, ld, xs, cs;
-    unsigned magic;
-    int vec;                  // sweeps and residual by 16-byte vectors of points (cl_step_v)
+// One distributed level as a step sees it (shared memory, built once per launch).  Positions are indices
+// into the dynamic shared memory: accesses stay in the shared address space with 32-bit arithmetic (as
+// pointers held in memory they would be generic, with 64-bit arithmetic and longer latency).
+template <class A> struct alignas(16) ClL {
+    int nr, a, rest, n0;                  // own rows, the first one, rows from it to the grid's end; columns
+    int nvp, per;                         // vectors per row; rows per thread, of the own and ghost rows
     unsigned magicv;
-    A* X;                     // buffer 0 at (row -1, column -1); buffer k at X + k*xs; (lr, c) at (lr+1)*ld + c+1
-    const A* S;               // stored stencil (component stride cs = maxr*n0); nullptr: FD level 0 (or Sg)
-    const void* Sg;           // stencil in global memory in the storage type (16-bit: times Ssc[k]), read by
-    const float* Ssc;         //   the vector steps only; nullptr: S
-    const A* W;               // omega / a_PP (index lr*n0 + c); nullptr: the scalar w0
-    A w0;
-    A *pu0, *pu1, *pu2;       // neighbours' ghost rows (see ClLev)
-    A *pd0, *pd1, *pd2;
-    A sigma, c, hx2, hy2;
-    const A* fx;              // staged faces of the FD level (nullptr: kappa = 1)
-    const A* fy;
-    __device__ __forceinline__ A* pu(int k) const { return k == 0 ? pu0 : (k == 1 ? pu1 : pu2); }
-    __device__ __forceinline__ A* pd(int k) const { return k == 0 ? pd0 : (k == 1 ? pd1 : pd2); }
-    __device__ __forceinline__ A* el(int k, int lr, int col) const {
-        return X + k * xs + (lr + 1) * ld + col + kClPad;
-    }
-    // store v at (lr, c) of buffer k and mirror the CTA's first / last row into the neighbours' ghost rows
-    __device__ __forceinline__ void put(int k, int lr, int col, A v) const {
-        *el(k, lr, col) = v;
-        if (lr == 0) {
-            A* q = pu(k);
-            if (q) q[col] = v;
-        }
-        if (lr == nr - 1) {
-            A* q = pd(k);
-            if (q) q[col] = v;
-        }
-    }
-};
-
-template <class SI> struct ClShared {
-    ClCtx<SI> t;
-    ClLev<typename PT<SI>::A> lv[kMaxLevels];
-    ClL<typename PT<SI>::A> lev[kMaxLevels];
-    typename PT<SI>::A w0;    // level 0's omega / a_PP where it is one scalar (w0_const)
-    int rank;
+    int H;                                // ghost rows
+    int X, xs, ld, kind;                  // (own row 0, column 0) of buffer 0, buffer stride, row stride;
+                                          // 0: stored stencil, 1: FD with kappa = 1, 2: FD with faces
+    int W, ix, in, cs;                    // weights at (own row 0, column 0) with row stride nvp * VN; x inbox, rows
+                                          // per side; stencil's component stride
+    int S, fx, fy, far;                   // stencil at (own row 0, column 0), row stride nvp * VN; faces likewise (rows
+                                          // of ld | of nvp * VN); 1: ghost rows reach beyond the next CTA
+    int prev[kClReach], next[kClReach];   // rows of the CTAs before and after, nearest first (0: none)
+    A cf[4][4];                           // kind 1, per mode (cl_fd)
+    A mP[4];                              // kind 1, per mode: factor of P
+    A sigma, c, hx2, hy2;                 // kind 2 (and kind 1 in 16-bit storage): sigma I + c K
+    const void* Sg;                       // stencil in global memory at (own row 0, column 0), component stride cs,
+    const float* Ssc;                     // row stride n0 (16-bit: times Ssc[k])
 };
 
 __device__ __forceinline__ unsigned cl_rank() {
@@ -144,157 +164,41 @@ __device__ __forceinline__ void cl_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Barrier after a step: the cluster for distributed levels, the CTA for replicated ones.
-__device__ __forceinline__ void cl_step_sync(bool dist) {
-    if (dist) cl_sync();
+// Barrier after a step: the cluster's where rows were stored into other CTAs, else the block's.
+__device__ __forceinline__ void cl_step_sync(bool remote) {
+    if (remote) cl_sync();
     else __syncthreads();
 }
 
-// Generic address of the same shared-memory location in CTA `rank` of the cluster.
-template <class T> __device__ __forceinline__ T* cl_map(T* p, unsigned rank) {
-    unsigned long long out;
-    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"(p), "r"(rank));
-    return reinterpret_cast<T*>(out);
+template <class A> __device__ __forceinline__ A* cl_sm() {
+    extern __shared__ __align__(16) unsigned char cl_smem[];
+    return reinterpret_cast<A*>(cl_smem);
 }
 
+// Stores into CTA `rank` of the cluster at index p of its dynamic shared memory: one value, one vector.
+template <class A> __device__ __forceinline__ unsigned cl_remote(int p, int rank) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(cl_sm<A>() + p);
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(d), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cl_rstore(int p, int rank, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cl_remote<float>(p, rank)), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cl_rstore(int p, int rank, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cl_remote<double>(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cl_rvstore(int p, int rank, const float* v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cl_remote<float>(p, rank)), "f"(v[0]),
+                 "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+}
+__device__ __forceinline__ void cl_rvstore(int p, int rank, const double* v) {
+    cl_rstore(p, rank, v[0]);
+}
+
+// p / d for magic = ceil(2^32 / d), d >= 2
 __device__ __forceinline__ int cl_div(int p, unsigned magic) { return (int)__umulhi((unsigned)p, magic); }
-
-template <class SI>
-__device__ __forceinline__ ClL<typename PT<SI>::A> cl_level(const ClShared<SI>& S, typename PT<SI>::A* sm, int l) {
-    using A = typename PT<SI>::A;
-    const ClCtx<SI>& t = S.t;
-    ClL<A> v;
-    v.n0 = t.g[l].n0;
-    v.n1 = t.g[l].n1;
-    v.ld = v.n0 + 2 * kClPad;
-    v.xs = (t.maxr[l] + 2) * v.ld;
-    v.cs = t.maxr[l] * v.n0;
-    v.magic = t.magic[l];
-    v.vec = t.vec[l];
-    v.magicv = t.magicv[l];
-    const bool dist = l < t.T;
-    v.a = dist ? S.lv[l].a : 0;
-    v.nr = dist ? S.lv[l].nr : v.n1;
-    v.X = sm + t.off[l];
-    v.Sg = nullptr;
-    v.Ssc = nullptr;
-    if ((l == 0 && t.fine0) || (t.soff[l] < 0 && !t.sten_global[l])) {
-        v.S = nullptr;
-    } else if (t.sten_global[l]) {
-        // the level's stencil in global memory: component stride n_x, rows from this CTA's first
-        v.cs = (int)t.g[l].nx;
-        if constexpr (std::is_same<SI, A>::value) {
-            v.S = reinterpret_cast<const A*>(t.sten[l]) + (long long)v.a * v.n0;
-        } else {
-            v.S = nullptr;
-            v.Sg = t.sten[l] + (long long)v.a * v.n0;
-            v.Ssc = t.sten_sc[l];
-        }
-    } else {
-        v.S = sm + t.soff[l];
-    }
-    v.W = t.woff[l] < 0 ? nullptr : sm + t.woff[l];
-    v.w0 = S.w0;
-    v.pu0 = dist ? S.lv[l].pu[0] : nullptr;
-    v.pu1 = dist ? S.lv[l].pu[1] : nullptr;
-    v.pu2 = dist ? S.lv[l].pu[2] : nullptr;
-    v.pd0 = dist ? S.lv[l].pd[0] : nullptr;
-    v.pd1 = dist ? S.lv[l].pd[1] : nullptr;
-    v.pd2 = dist ? S.lv[l].pd[2] : nullptr;
-    v.sigma = t.sigma;
-    v.c = t.c;
-    v.hx2 = A(t.g[0].hx2);
-    v.hy2 = A(t.g[0].hy2);
-    v.fx = t.has_faces ? sm + t.fxoff : nullptr;
-    v.fy = t.has_faces ? sm + t.fyoff : nullptr;
-    return v;
-}
-
-// (A x)_P at own point p = (lr, c); xm points at x(lr, c) in the padded layout.
-template <class A>
-__device__ __forceinline__ A cl_apply(const ClL<A>& v, int p, int lr, int c, const A* xm) {
-    const int ld = v.ld;
-    if (v.S == nullptr) {
-        const A uP = xm[0], uW = xm[-1], uE = xm[1], uS = xm[-ld], uN = xm[ld];
-        A K;
-        if (v.fx == nullptr) {
-            K = v.hx2 * (A(2) * uP - uW - uE) + v.hy2 * (A(2) * uP - uS - uN);
-        } else {
-            const A* fxr = v.fx + lr * (v.n0 + 1);
-            const A* fyr = v.fy + lr * v.n0;
-            K = fxr[c] * (uP - uW) + fxr[c + 1] * (uP - uE) + fyr[c] * (uP - uS) + fyr[c + v.n0] * (uP - uN);
-        }
-        return v.sigma * uP + v.c * K;
-    }
-    const A* Sp = v.S + p;
-    const int cs = v.cs;
-    A acc = A(0);
-    acc += Sp[0 * cs] * xm[-ld - 1];
-    acc += Sp[1 * cs] * xm[-ld];
-    acc += Sp[2 * cs] * xm[-ld + 1];
-    acc += Sp[3 * cs] * xm[-1];
-    acc += Sp[4 * cs] * xm[0];
-    acc += Sp[5 * cs] * xm[1];
-    acc += Sp[6 * cs] * xm[ld - 1];
-    acc += Sp[7 * cs] * xm[ld];
-    acc += Sp[8 * cs] * xm[ld + 1];
-    return acc;
-}
-
-// Damped Jacobi into buffer 1-kin: zero ? w b : x + w (b - A x), x = buffer kin.
-template <class A>
-__device__ __forceinline__ void cl_sweep(const ClL<A>& vin, int kin, bool zero, int tid, int nthr) {
-    if (tid >= vin.nr * vin.n0) return;
-    const ClL<A> v = vin;
-    const int n0 = v.n0;
-    const int np = v.nr * n0;
-    for (int p = tid; p < np; p += nthr) {
-        const int lr = cl_div(p, v.magic);
-        const int c = p - lr * n0;
-        const A bp = *v.el(2, lr, c);
-        A val;
-        const A wp = v.W ? v.W[p] : v.w0;
-        if (zero) {
-            val = wp * bp;
-        } else {
-            const A* xm = v.el(kin, lr, c);
-            val = xm[0] + wp * (bp - cl_apply(v, p, lr, c, xm));
-        }
-        v.put(1 - kin, lr, c, val);
-    }
-}
-
-// Residual b - A x of buffer kin into buffer 1 - kin.
-template <class A>
-__device__ __forceinline__ void cl_residual(const ClL<A>& vin, int kin, int tid, int nthr) {
-    if (tid >= vin.nr * vin.n0) return;
-    const ClL<A> v = vin;
-    const int n0 = v.n0;
-    const int np = v.nr * n0;
-    for (int p = tid; p < np; p += nthr) {
-        const int lr = cl_div(p, v.magic);
-        const int c = p - lr * n0;
-        const A* xm = v.el(kin, lr, c);
-        v.put(1 - kin, lr, c, *v.el(2, lr, c) - cl_apply(v, p, lr, c, xm));
-    }
-}
-
-// The points of a CTA's rows as 16-byte vectors (4 FP32 or 2 FP64 consecutive points of a row, rows
-// 16-byte aligned by kClPad): one vector load per neighbouring row, scalar loads of the two points
-// beside the vector, one vector store.  MODE 0: damped Jacobi into buffer 1 - kin; MODE 1: the same
-// from x = 0 (w b); MODE 2: the residual b - A x into buffer 1 - kin.  Per point the operations of
-// cl_sweep / cl_residual / cl_apply in the same order: the same values.  Levels planned with
-// `vec`: n0 a multiple of the vector width, and a 9-point stored stencil or the FD level with
-// kappa = 1.
-template <class A> struct ClVec;
-template <> struct ClVec<float> {
-    using T = float4;
-    static constexpr int n = 4;
-};
-template <> struct ClVec<double> {
-    using T = double2;
-    static constexpr int n = 2;
-};
 
 template <class A>
 __device__ __forceinline__ void cl_vload(const A* p, A* out) {
@@ -315,149 +219,334 @@ __device__ __forceinline__ void cl_vstore(A* p, const A* in) {
     *reinterpret_cast<VT*>(p) = v;
 }
 
-template <int MODE, class SI, class A>
-__device__ __forceinline__ void cl_step_v(const ClL<A>& vin, int kin, int tid, int nthr) {
-    constexpr int VN = ClVec<A>::n;
-    const int nv = vin.n0 / VN;
-    if (tid >= vin.nr * nv) return;
-    const ClL<A> v = vin;
-    const int np = v.nr * nv, ld = v.ld, kout = 1 - kin;
-    for (int q = tid; q < np; q += nthr) {
-        const int lr = cl_div(q, v.magicv);
-        const int c = (q - lr * nv) * VN;
-        const int p = lr * v.n0 + c;
-        A b[VN], w[VN], out[VN];
-        cl_vload(v.el(2, lr, c), b);
-        if (MODE != 2) {
-            if (v.W) {
-                cl_vload(v.W + p, w);
-            } else {
-#pragma unroll
-                for (int t = 0; t < VN; ++t) w[t] = v.w0;
-            }
-        }
-        if (MODE == 1) {
-#pragma unroll
-            for (int t = 0; t < VN; ++t) out[t] = w[t] * b[t];
-        } else {
-            const A* xm = v.el(kin, lr, c);
-            A xc[VN], xs[VN], xn[VN];
-            cl_vload(xm, xc);
-            cl_vload(xm - ld, xs);
-            cl_vload(xm + ld, xn);
-            const A xl = xm[-1], xr = xm[VN];
-            A Au[VN];
-            if (v.S == nullptr && v.Sg == nullptr) {
-#pragma unroll
-                for (int t = 0; t < VN; ++t) {
-                    const A uP = xc[t], uW = t == 0 ? xl : xc[t - 1], uE = t == VN - 1 ? xr : xc[t + 1];
-                    const A K = v.hx2 * (A(2) * uP - uW - uE) + v.hy2 * (A(2) * uP - xs[t] - xn[t]);
-                    Au[t] = v.sigma * uP + v.c * K;
-                }
-            } else {
-                const A sl = xm[-ld - 1], sr = xm[-ld + VN], nl = xm[ld - 1], nrt = xm[ld + VN];
-                A S[9][VN];
-                if constexpr (!std::is_same<SI, A>::value) {
-                    if (v.Sg) {
-                        // 16-bit storage in global memory: VN values (8 bytes) per component, times its scale
-                        const SI* g = reinterpret_cast<const SI*>(v.Sg) + p;
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) {
-                            const uint2 raw = *reinterpret_cast<const uint2*>(g + (long long)k * v.cs);
-                            const SI* e = reinterpret_cast<const SI*>(&raw);
-#pragma unroll
-                            for (int t = 0; t < VN; ++t) S[k][t] = PT<SI>::ld(e[t]) * v.Ssc[k];
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) cl_vload(v.S + (long long)k * v.cs + p, S[k]);
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 9; ++k) cl_vload(v.S + (long long)k * v.cs + p, S[k]);
-                }
-#pragma unroll
-                for (int t = 0; t < VN; ++t) {
-                    const A sW = t == 0 ? sl : xs[t - 1], sE = t == VN - 1 ? sr : xs[t + 1];
-                    const A uW = t == 0 ? xl : xc[t - 1], uE = t == VN - 1 ? xr : xc[t + 1];
-                    const A nW = t == 0 ? nl : xn[t - 1], nE = t == VN - 1 ? nrt : xn[t + 1];
-                    A acc = A(0);
-                    acc += S[0][t] * sW;
-                    acc += S[1][t] * xs[t];
-                    acc += S[2][t] * sE;
-                    acc += S[3][t] * uW;
-                    acc += S[4][t] * xc[t];
-                    acc += S[5][t] * uE;
-                    acc += S[6][t] * nW;
-                    acc += S[7][t] * xn[t];
-                    acc += S[8][t] * nE;
-                    Au[t] = acc;
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < VN; ++t) out[t] = MODE == 0 ? xc[t] + w[t] * (b[t] - Au[t]) : b[t] - Au[t];
-        }
-        cl_vstore(v.el(kout, lr, c), out);
-        if (lr == 0) {
-            A* u = v.pu(kout);
-            if (u) cl_vstore(u + c, out);
-        }
-        if (lr == v.nr - 1) {
-            A* d = v.pd(kout);
-            if (d) cl_vstore(d + c, out);
-        }
-    }
-}
-
-// Sweep or residual of one level: vectors where planned, else point by point.
-template <class SI, class A>
-__device__ __forceinline__ void cl_sweep_any(const ClL<A>& v, int kin, bool zero, int tid, int nthr) {
-    if (v.vec) {
-        if (zero) cl_step_v<1, SI>(v, kin, tid, nthr);
-        else cl_step_v<0, SI>(v, kin, tid, nthr);
-    } else {
-        cl_sweep(v, kin, zero, tid, nthr);
-    }
-}
-
-template <class SI, class A>
-__device__ __forceinline__ void cl_residual_any(const ClL<A>& v, int kin, int tid, int nthr) {
-    if (v.vec) cl_step_v<2, SI>(v, kin, tid, nthr);
-    else cl_residual(v, kin, tid, nthr);
-}
-
-// b_c = P^T r (r = buffer kr of the fine level f) on the coarse rows this CTA computes.
-// any_row: the coarse level is the replicated coarsest; fine rows come from rowtab (row i of
-// buffer 0, first interior column, in the CTA that owns it).
+// Store the vector at (own row lr, column c) into the ghost rows (depth rows) of the CTAs that need it:
+// into buffer k, or (inbox) into their x inbox.
 template <class A>
-__device__ __forceinline__ void cl_restrict(const ClL<A>& fin, const ClL<A>& cvin, int kr, bool any_row,
-                                            const A* const* rowtab, int tid, int nthr) {
-    if (tid >= cvin.nr * cvin.n0) return;
-    const ClL<A> f = fin, cv = cvin;
-    const int n0c = cv.n0;
-    const int np = cv.nr * n0c;
-    for (int p = tid; p < np; p += nthr) {
-        const int lr = cl_div(p, cv.magic);
-        const int I = p - lr * n0c;
-        const int J = cv.a + lr;
-        A acc = A(0);
+__device__ __forceinline__ void cl_push(const ClL<A>& v, int rank, int k, int lr, int c, const A* out, int depth,
+                                        bool inbox) {
+    const int at = (inbox ? v.in + v.ix * v.ld : v.X + k * v.xs) + lr * v.ld + c, ld = v.ld;
+    if (lr < depth && v.prev[0] > 0) {
+        // beyond the end of the CTA before
+        cl_rvstore(at + (inbox ? 0 : v.prev[0] * ld), rank - 1, out);
+        if (v.far) {
+            int between = v.prev[0];
 #pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int fj = 2 * J + 1 + dy;
-            const A wy = dy == 0 ? A(1) : A(0.5);
-            const A* row;
-            if (any_row) {
-                if (fj < 0 || fj >= f.n1) continue;
-                row = rowtab[fj] + kr * f.xs;
-            } else {
-                row = f.el(kr, fj - f.a, 0);          // own or ghost row (zero beyond the boundary)
+            for (int q = 1; q < kClReach; ++q) {
+                if (lr >= depth - between || v.prev[q] == 0) break;
+                cl_rvstore(at + (inbox ? between : between + v.prev[q]) * ld, rank - 1 - q, out);
+                between += v.prev[q];
             }
-            const int fi = 2 * I + 1;
-            acc += A(0.5) * wy * row[fi - 1];
-            acc += A(1) * wy * row[fi];
-            acc += A(0.5) * wy * row[fi + 1];        // the zero column when fi + 1 == n0
         }
-        cv.put(2, lr, I, acc);
+    }
+    if (lr >= v.nr - depth && v.next[0] > 0) {
+        // before the first row of the CTA after
+        cl_rvstore(at - v.nr * ld, rank + 1, out);
+        if (v.far) {
+            int between = v.next[0];
+#pragma unroll
+            for (int q = 1; q < kClReach; ++q) {
+                if (lr < v.nr - depth + between || v.next[q] == 0) break;
+                cl_rvstore(at - (v.nr + between) * ld, rank + 1 + q, out);
+                between += v.next[q];
+            }
+        }
+    }
+}
+
+// This thread's column vector of the level and its consecutive rows of [lo, hi): own and ghost rows are dealt
+// out once per level, per rows to a thread.
+struct ClRows {
+    int c, r0, r1;
+};
+template <class A>
+__device__ __forceinline__ ClRows cl_rows(const ClL<A>& v, int lo, int hi) {
+    const int tid = threadIdx.x;
+    const int g = cl_div(tid, v.magicv), r = g * v.per - v.H;
+    ClRows q;
+    q.c = (tid - g * v.nvp) * ClVec<A>::n;
+    q.r0 = max(r, lo);
+    q.r1 = min(r + v.per, hi);
+    return q;
+}
+
+// One point of a step with the FD operator, kappa = 1 (P, its neighbours and b).
+// FP64 folds the constants: kb b + k0 P + kx (W + E) + ky (S + N), six operations where the rate is two per
+// cycle and SM.  FP32 keeps the differences P - W, ..., which are exact for smooth fields, so the residual's
+// cancellation costs no digits: kw (b - kA (sigma P + ex (...) + ey (...))) + mP P.  16-bit storage takes
+// the level kernels' formula operation by operation: its results are rounded to the storage format, and the
+// roundings are pinned.
+template <bool SCALED>
+__device__ __forceinline__ double cl_fd(const ClL<double>&, const double* cf, double, int, double b, double P, double W,
+                                        double E, double S, double N) {
+    double s = cf[0] * b;
+    s += cf[1] * P;
+    s += cf[2] * (W + E);
+    return s + cf[3] * (S + N);
+}
+template <bool SCALED>
+__device__ __forceinline__ float cl_fd(const ClL<float>& v, const float* cf, float mP, int mode, float b, float P, float W,
+                                       float E, float S, float N) {
+    if constexpr (SCALED) {
+        if (mode == 1) return cf[0] * b;
+        const float K = v.hx2 * (2.f * P - W - E) + v.hy2 * (2.f * P - S - N);
+        const float res = b - (v.sigma * P + v.c * K);
+        return mode == 2 ? res : P + cf[0] * res;
+    } else {
+        float s = cf[1] * P;
+        s += cf[2] * ((P - W) + (P - E));
+        s += cf[3] * ((P - S) + (P - N));
+        return cf[0] * (b - s) + mP * P;
+    }
+}
+
+// One step of a level on own rows and ext ghost rows per side, from buffer kin (x) and b into buffer
+// kout.  mode 0: damped Jacobi x + w (b - A x); 1: the same from x = 0 (w b); 2: the residual b - A x; 3 (FD,
+// kappa = 1, kin = 2): two sweeps from x = 0, whose first is w0 b.  The modes are coefficients of one formula
+// (mode 1 reads no x: zeros take its place).  depth > 0: also store the own edge rows into the other CTAs.
+template <class SI, bool FACES, bool GLOBAL, class A>
+__device__ __forceinline__ void cl_step(const ClL<A>& v, int rank, int mode, int kin, int kout, int ext, int depth,
+                                        bool inbox) {
+    constexpr int VN = ClVec<A>::n;
+    A* const sm = cl_sm<A>();
+    const ClRows q = cl_rows(v, max(-ext, -v.a), min(v.nr + ext, v.rest));
+    if (q.r0 >= q.r1) return;
+    const int ld = v.ld, c = q.c;
+    const int nvalid = v.n0 - c;                  // columns from here on (below VN in a ragged last vector)
+    const int at = v.X + q.r0 * ld + c;
+    const A* xm = sm + at + kin * v.xs;
+    const A* bm = sm + at + 2 * v.xs;
+    A* om = sm + at + kout * v.xs;
+    A S[VN], P[VN], N[VN];
+#pragma unroll
+    for (int i = 0; i < VN; ++i) S[i] = P[i] = N[i] = A(0);
+    const bool ax = mode != 1;
+    if (ax) {
+        cl_vload(xm - ld, S);
+        cl_vload(xm, P);
+    }
+    auto finish = [&](int lr, A* out) {
+        if (VN > 1 && nvalid < VN) {
+#pragma unroll
+            for (int i = 0; i < VN; ++i)
+                if (i >= nvalid) out[i] = A(0);
+        }
+        cl_vstore(om, out);
+        if (depth > 0 && lr >= 0 && lr < v.nr) cl_push(v, rank, kout, lr, c, out, depth, inbox);
+        om += ld;
+        xm += ld;
+        bm += ld;
+#pragma unroll
+        for (int i = 0; i < VN; ++i) {
+            S[i] = P[i];
+            P[i] = N[i];
+        }
+    };
+    if (v.kind == 1) {
+        A cf[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) cf[i] = v.cf[mode][i];
+        const A mP = v.mP[mode];
+#pragma unroll 1
+        for (int r = q.r0; r < q.r1; ++r) {
+            A b[VN], out[VN], l = A(0), e = A(0);
+            cl_vload(bm, b);
+            if (ax) {
+                cl_vload(xm + ld, N);
+                l = xm[-1];
+                e = xm[VN];
+            }
+#pragma unroll
+            for (int i = 0; i < VN; ++i) {
+                const A W = i == 0 ? l : P[i - 1], E = i == VN - 1 ? e : P[i + 1];
+                out[i] = cl_fd<PT<SI>::scaled>(v, cf, mP, mode, b[i], P[i], W, E, S[i], N[i]);
+            }
+            finish(r, out);
+        }
+        return;
+    }
+    const int wrow = v.nvp * VN;
+    const A* wm = sm + v.W + q.r0 * wrow + c;
+    const A mP = mode == 0 ? A(1) : A(0);
+    if (FACES && v.kind == 2) {
+        const A sigma = v.sigma, cK = v.c;
+        const A* fx = sm + v.fx + q.r0 * ld + c;
+        const A* fy = sm + v.fy + q.r0 * wrow + c;
+#pragma unroll 1
+        for (int r = q.r0; r < q.r1; ++r) {
+            A b[VN], w[VN], out[VN];
+            cl_vload(bm, b);
+            cl_vload(wm, w);
+            if (ax) {
+                A f0[VN], s0[VN], s1[VN];
+                cl_vload(xm + ld, N);
+                cl_vload(fx, f0);
+                const A f4 = fx[VN];
+                cl_vload(fy, s0);
+                cl_vload(fy + wrow, s1);
+                const A l = xm[-1], e = xm[VN];
+#pragma unroll
+                for (int i = 0; i < VN; ++i) {
+                    const A W = i == 0 ? l : P[i - 1], E = i == VN - 1 ? e : P[i + 1];
+                    const A fE = i == VN - 1 ? f4 : f0[i + 1];
+                    const A K = f0[i] * (P[i] - W) + fE * (P[i] - E) + s0[i] * (P[i] - S[i]) + s1[i] * (P[i] - N[i]);
+                    b[i] -= sigma * P[i] + cK * K;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < VN; ++i) out[i] = (mode == 2 ? A(1) : w[i]) * b[i] + mP * P[i];
+            fx += ld;
+            fy += wrow;
+            wm += wrow;
+            finish(r, out);
+        }
+        return;
+    }
+    // stored 9-point stencil: components (dx + 1) + 3 (dy + 1)
+    A sl = A(0), sr = A(0), pl = A(0), pr = A(0), nl = A(0), nr = A(0);
+    if (ax) {
+        sl = xm[-ld - 1];
+        sr = xm[-ld + VN];
+        pl = xm[-1];
+        pr = xm[VN];
+    }
+    const int cs = v.cs;
+    const A* Sm = sm + v.S + q.r0 * wrow + c;
+    const SI* Gm = reinterpret_cast<const SI*>(v.Sg) + q.r0 * v.n0 + c;
+    const bool global = GLOBAL && v.Sg != nullptr;
+#pragma unroll 1
+    for (int r = q.r0; r < q.r1; ++r) {
+        A b[VN], w[VN], out[VN];
+        cl_vload(bm, b);
+        cl_vload(wm, w);
+        if (ax) {
+            A K[9][VN];
+            cl_vload(xm + ld, N);
+            nl = xm[ld - 1];
+            nr = xm[ld + VN];
+            if (global) {
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    if constexpr (std::is_same<SI, A>::value) {
+                        cl_vload(Gm + (long long)k * cs, K[k]);
+                    } else {
+                        // 16-bit storage: VN values (8 bytes) per component, times its scale
+                        const uint2 raw = *reinterpret_cast<const uint2*>(Gm + (long long)k * cs);
+                        const SI* e = reinterpret_cast<const SI*>(&raw);
+#pragma unroll
+                        for (int i = 0; i < VN; ++i) K[k][i] = PT<SI>::ld(e[i]) * v.Ssc[k];
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 9; ++k) cl_vload(Sm + k * cs, K[k]);
+            }
+#pragma unroll
+            for (int i = 0; i < VN; ++i) {
+                if constexpr (PT<SI>::scaled) {
+                    // the level kernels' order (see cl_fd)
+                    A acc = A(0);
+                    acc += K[0][i] * (i == 0 ? sl : S[i - 1]);
+                    acc += K[1][i] * S[i];
+                    acc += K[2][i] * (i == VN - 1 ? sr : S[i + 1]);
+                    acc += K[3][i] * (i == 0 ? pl : P[i - 1]);
+                    acc += K[4][i] * P[i];
+                    acc += K[5][i] * (i == VN - 1 ? pr : P[i + 1]);
+                    acc += K[6][i] * (i == 0 ? nl : N[i - 1]);
+                    acc += K[7][i] * N[i];
+                    acc += K[8][i] * (i == VN - 1 ? nr : N[i + 1]);
+                    b[i] -= acc;
+                    continue;
+                }
+                // three chains, one per row
+                A s0 = K[0][i] * (i == 0 ? sl : S[i - 1]);
+                A s1 = K[3][i] * (i == 0 ? pl : P[i - 1]);
+                A s2 = K[6][i] * (i == 0 ? nl : N[i - 1]);
+                s0 += K[1][i] * S[i];
+                s1 += K[4][i] * P[i];
+                s2 += K[7][i] * N[i];
+                s0 += K[2][i] * (i == VN - 1 ? sr : S[i + 1]);
+                s1 += K[5][i] * (i == VN - 1 ? pr : P[i + 1]);
+                s2 += K[8][i] * (i == VN - 1 ? nr : N[i + 1]);
+                b[i] -= s0 + s1 + s2;
+            }
+        }
+        Gm += v.n0;
+        Sm += wrow;
+#pragma unroll
+        for (int i = 0; i < VN; ++i) out[i] = (mode == 2 ? A(1) : w[i]) * b[i] + mP * P[i];
+        wm += wrow;
+        finish(r, out);
+        sl = pl;
+        sr = pr;
+        pl = nl;
+        pr = nr;
+    }
+}
+
+// b_c = P^T r (buffer kr of the fine level f) on the own rows of the distributed coarse level v, and
+// (kx >= 0) its first sweep w b_c into buffer kx; both stored into the other CTAs' ghost rows too.
+template <bool SCALED, class A>
+__device__ __forceinline__ void cl_restrict(const ClL<A>& f, const ClL<A>& v, int rank, int kr, int kx) {
+    constexpr int VN = ClVec<A>::n;
+    A* const sm = cl_sm<A>();
+    const ClRows q = cl_rows(v, 0, v.nr);
+    const int nvalid = v.n0 - q.c, ld = f.ld;
+    const A* row = sm + f.X + kr * f.xs + (2 * (v.a + q.r0) - f.a) * ld + 2 * q.c;    // fine row 2J (0-based) of three
+    const int om = v.X + q.r0 * v.ld + q.c;
+    const A* wm = sm + v.W + q.r0 * v.nvp * VN + q.c;
+    int step = 0;
+#pragma unroll 1
+    for (int r = q.r0; r < q.r1; ++r) {
+        A x[3][2 * VN + 1], out[VN];
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+            if constexpr (VN > 1) {
+                cl_vload(row + dy * ld, x[dy]);
+                cl_vload(row + dy * ld + VN, x[dy] + VN);
+            } else {
+                x[dy][0] = row[dy * ld];
+                x[dy][1] = row[dy * ld + 1];
+            }
+            x[dy][2 * VN] = row[dy * ld + 2 * VN];
+        }
+        if constexpr (SCALED) {
+#pragma unroll
+            for (int i = 0; i < VN; ++i) out[i] = A(0);
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+                const A wy = dy == 1 ? A(1) : A(0.5);
+#pragma unroll
+                for (int i = 0; i < VN; ++i) {
+                    out[i] += A(0.5) * wy * x[dy][2 * i];
+                    out[i] += wy * x[dy][2 * i + 1];
+                    out[i] += A(0.5) * wy * x[dy][2 * i + 2];
+                }
+            }
+        } else {
+            // weights 1/4, 1/2, 1/4 of the outer rows, twice that of the middle one
+            A s[2 * VN + 1];
+#pragma unroll
+            for (int i = 0; i <= 2 * VN; ++i) s[i] = x[1][i] + A(0.5) * (x[0][i] + x[2][i]);
+#pragma unroll
+            for (int i = 0; i < VN; ++i) out[i] = s[2 * i + 1] + A(0.5) * (s[2 * i] + s[2 * i + 2]);
+        }
+        if (VN > 1 && nvalid < VN) {
+#pragma unroll
+            for (int i = 0; i < VN; ++i)
+                if (i >= nvalid) out[i] = A(0);
+        }
+        cl_vstore(sm + om + 2 * v.xs + step * v.ld, out);
+        cl_push(v, rank, 2, r, q.c, out, v.H, false);
+        if (kx >= 0) {
+            A w[VN];
+            cl_vload(wm + step * v.nvp * VN, w);
+#pragma unroll
+            for (int i = 0; i < VN; ++i) out[i] *= w[i];
+            cl_vstore(sm + om + kx * v.xs + step * v.ld, out);
+            cl_push(v, rank, kx, r, q.c, out, v.H, false);
+        }
+        row += 2 * ld;
+        ++step;
     }
 }
 
@@ -475,586 +564,480 @@ __device__ __forceinline__ void cl_interp(int F, int& j0, int& j1, bool& inj) {
     }
 }
 
-// x_f (buffer kx) += P x_c (buffer kc) on the fine rows this CTA computes.
-template <class A>
-__device__ __forceinline__ void cl_prolong(const ClL<A>& fin, const ClL<A>& cvin, int kx, int kc, int tid, int nthr) {
-    if (tid >= fin.nr * fin.n0) return;
-    const ClL<A> f = fin, cv = cvin;
-    const int n0 = f.n0;
-    const int np = f.nr * n0;
-    for (int p = tid; p < np; p += nthr) {
-        const int lr = cl_div(p, f.magic);
-        const int c = p - lr * n0;
-        int y0, y1, x0, x1;
-        bool yi, xi;
-        cl_interp(f.a + lr, y0, y1, yi);
-        cl_interp(c, x0, x1, xi);
-        // injection in a direction: one coarse index, the second term gets weight 0
-        const A wy = yi ? A(1) : A(0.5), wx = xi ? A(1) : A(0.5);
-        const A w00 = wy * wx, w01 = xi ? A(0) : w00, w10 = yi ? A(0) : w00, w11 = (xi || yi) ? A(0) : w00;
-        const A* r0 = cv.el(kc, y0 - cv.a, 0);
-        const A* r1 = cv.el(kc, y1 - cv.a, 0);
-        A acc = *f.el(kx, lr, c);
-        acc += w00 * r0[x0];
-        acc += w01 * r0[x1];
-        acc += w10 * r1[x0];
-        acc += w11 * r1[x1];
-        f.put(kx, lr, c, acc);
-    }
-}
-
-// xh = x_f (buffer kx) + P x_c (buffer kc) into buffer kout for this CTA's rows and its two ghost
-// rows (rows outside the grid stay zero): the first post-smoothing sweep then reads xh without a
-// cluster barrier, because each CTA computes its own ghost rows from its ghost rows of x_f and x_c.
-// With kout == kx every element is read and written by the same thread.
-template <class A>
-__device__ __forceinline__ void cl_prolong_ext(const ClL<A>& fin, const ClL<A>& cvin, int kx, int kc, int kout,
-                                               int tid, int nthr) {
-    if (fin.nr == 0 || tid >= (fin.nr + 2) * fin.n0) return;
-    const ClL<A> f = fin, cv = cvin;
-    const int n0 = f.n0;
-    const int np = f.nr > 0 ? (f.nr + 2) * n0 : 0;
-    for (int p = tid; p < np; p += nthr) {
-        const int lr = cl_div(p, f.magic) - 1;
-        const int c = p - (lr + 1) * n0;
-        const int F = f.a + lr;
-        if (F < 0 || F >= f.n1) continue;
-        int y0, y1, x0, x1;
-        bool yi, xi;
-        cl_interp(F, y0, y1, yi);
-        cl_interp(c, x0, x1, xi);
-        const A wy = yi ? A(1) : A(0.5), wx = xi ? A(1) : A(0.5);
-        const A w00 = wy * wx, w01 = xi ? A(0) : w00, w10 = yi ? A(0) : w00, w11 = (xi || yi) ? A(0) : w00;
-        const A* r0 = cv.el(kc, y0 - cv.a, 0);
-        const A* r1 = cv.el(kc, y1 - cv.a, 0);
-        A acc = *f.el(kx, lr, c);
-        acc += w00 * r0[x0];
-        acc += w01 * r0[x1];
-        acc += w10 * r1[x0];
-        acc += w11 * r1[x1];
-        *f.el(kout, lr, c) = acc;
-    }
-}
-
-// cl_prolong_ext with 16-byte vectors of fine points (fine n0 a multiple of the vector width): one
-// vector load and store of x_f, the three coarse values beside each vector from each coarse row;
-// per point the operations of cl_prolong_ext in the same order.
-template <class A>
-__device__ __forceinline__ void cl_prolong_ext_v(const ClL<A>& fin, const ClL<A>& cvin, int kx, int kc, int kout,
-                                                 int tid, int nthr) {
+// x_f (buffer kx) += P x_c (buffer kc of the coarse level, its inbox beyond the own rows) on own rows and ext
+// ghost rows, in place.  A vector starts at an even column c: its points average coarse columns
+// c/2 - 1, c/2 and take c/2 in turn.  depth > 0: the last step of the level, stored into the inboxes.
+template <bool SCALED, class A>
+__device__ __forceinline__ void cl_prolong(const ClL<A>& f, const ClL<A>& v, int rank, int kx, int kc, int ext, int depth) {
     constexpr int VN = ClVec<A>::n;
-    const int nv = fin.n0 / VN;
-    if (fin.nr == 0 || tid >= (fin.nr + 2) * nv) return;
-    const ClL<A> f = fin, cv = cvin;
-    const int np = (f.nr + 2) * nv;
-    for (int q = tid; q < np; q += nthr) {
-        const int lr = cl_div(q, f.magicv) - 1;
-        const int c = (q - (lr + 1) * nv) * VN;
-        const int F = f.a + lr;
-        if (F < 0 || F >= f.n1) continue;
+    A* const sm = cl_sm<A>();
+    const ClRows q = cl_rows(f, max(-ext, -f.a), min(f.nr + ext, f.rest));
+    const int nvalid = f.n0 - q.c, ldc = v.ld;
+    // row y of x_c: own rows in buffer kc, the others in the inbox (the coarsest level: all in the buffer)
+    const int xc = v.X + kc * v.xs + (q.c >> 1), in = v.in + (q.c >> 1) + v.ix * ldc, ac = v.a, nc = v.nr, ix = v.ix;
+    auto at = [&](int y) {
+        const int lr = y - ac;
+        if (ix == 0 || (lr >= 0 && lr < nc)) return xc + lr * ldc;
+        return in + (lr < 0 ? lr : lr - nc) * ldc;
+    };
+    A* x = sm + f.X + kx * f.xs + q.r0 * f.ld + q.c;
+#pragma unroll 1
+    for (int r = q.r0; r < q.r1; ++r) {
         int y0, y1;
         bool yi;
-        cl_interp(F, y0, y1, yi);
-        const A wy = yi ? A(1) : A(0.5);
-        const A* r0 = cv.el(kc, y0 - cv.a, 0);
-        const A* r1 = cv.el(kc, y1 - cv.a, 0);
-        A xv[VN], out[VN];
-        cl_vload(f.el(kx, lr, c), xv);
+        cl_interp(f.a + r, y0, y1, yi);
+        const A* p0 = sm + at(y0);
+        const A* p1 = sm + at(y1);
+        A out[VN], m[VN / 2 + 2];
+        cl_vload(x, out);
+        if constexpr (VN == 1) {
+            // column c averages coarse columns c/2 - 1 and c/2, or (c odd) takes c/2
+            const int o = (q.c & 1) - 1;
+            const A s0 = p0[o] + p1[o], s1 = p0[0] + p1[0];
+            out[0] += A(0.25) * (s0 + s1);
+        } else if constexpr (SCALED) {
+            const A wy = yi ? A(1) : A(0.5);
 #pragma unroll
-        for (int t = 0; t < VN; ++t) {
-            int x0, x1;
-            bool xi;
-            cl_interp(c + t, x0, x1, xi);
-            const A wx = xi ? A(1) : A(0.5);
-            const A w00 = wy * wx, w01 = xi ? A(0) : w00, w10 = yi ? A(0) : w00, w11 = (xi || yi) ? A(0) : w00;
-            A acc = xv[t];
-            acc += w00 * r0[x0];
-            acc += w01 * r0[x1];
-            acc += w10 * r1[x0];
-            acc += w11 * r1[x1];
-            out[t] = acc;
-        }
-        cl_vstore(f.el(kout, lr, c), out);
-    }
-}
-
-// cl_restrict from a distributed fine level into a distributed coarse one with 16-byte vectors of
-// coarse points: each fine row contributes two vector loads and one scalar; per point the operations
-// of cl_restrict in the same order.  Both levels' n0 must be multiples of the vector width (the fine
-// rows are read as vectors: with an odd fine n0 the row stride n0 + 2 kClPad is odd).
-template <class A>
-__device__ __forceinline__ void cl_restrict_v(const ClL<A>& fin, const ClL<A>& cvin, int kr, int tid, int nthr) {
-    constexpr int VN = ClVec<A>::n;
-    const int nv = cvin.n0 / VN;
-    if (tid >= cvin.nr * nv) return;
-    const ClL<A> f = fin, cv = cvin;
-    const int np = cv.nr * nv;
-    for (int q = tid; q < np; q += nthr) {
-        const int lr = cl_div(q, cv.magicv);
-        const int I0 = (q - lr * nv) * VN;
-        const int J = cv.a + lr;
-        A acc[VN];
+            for (int i = 0; i < VN; ++i) {
+                const bool xi = i & 1;
+                const int x0 = xi ? i / 2 : i / 2 - 1, x1 = i / 2;
+                const A wx = xi ? A(1) : A(0.5);
+                const A w00 = wy * wx, w01 = xi ? A(0) : w00, w10 = yi ? A(0) : w00, w11 = (xi || yi) ? A(0) : w00;
+                out[i] += w00 * p0[x0];
+                out[i] += w01 * p0[x1];
+                out[i] += w10 * p1[x0];
+                out[i] += w11 * p1[x1];
+            }
+        } else {
+            // the coarse row of this fine row: injected (y0 = y1) or the average of two
 #pragma unroll
-        for (int t = 0; t < VN; ++t) acc[t] = A(0);
+            for (int i = 0; i <= VN / 2; ++i) m[i] = A(0.5) * (p0[i - 1] + p1[i - 1]);
 #pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int fj = 2 * J + 1 + dy;
-            const A wy = dy == 0 ? A(1) : A(0.5);
-            const A* row = f.el(kr, fj - f.a, 0) + 2 * I0;     // own or ghost row (zero beyond the boundary)
-            A fv[2 * VN + 1];
-            cl_vload(row, fv);
-            cl_vload(row + VN, fv + VN);
-            fv[2 * VN] = row[2 * VN];                          // the zero column when 2 (I0 + VN) == n0
-#pragma unroll
-            for (int t = 0; t < VN; ++t) {
-                acc[t] += A(0.5) * wy * fv[2 * t];
-                acc[t] += A(1) * wy * fv[2 * t + 1];
-                acc[t] += A(0.5) * wy * fv[2 * t + 2];
+            for (int i = 0; i < VN / 2; ++i) {
+                out[2 * i] += A(0.5) * (m[i] + m[i + 1]);
+                out[2 * i + 1] += m[i + 1];
             }
         }
-        cl_vstore(cv.el(2, lr, I0), acc);
-        if (lr == 0) {
-            A* u = cv.pu(2);
-            if (u) cl_vstore(u + I0, acc);
+        if (VN > 1 && nvalid < VN) {
+#pragma unroll
+            for (int i = 0; i < VN; ++i)
+                if (i >= nvalid) out[i] = A(0);
         }
-        if (lr == cv.nr - 1) {
-            A* d = cv.pd(2);
-            if (d) cl_vstore(d + I0, acc);
-        }
+        cl_vstore(x, out);
+        if (depth > 0 && r >= 0 && r < f.nr) cl_push(f, rank, kx, r, q.c, out, depth, true);
+        x += f.ld;
     }
 }
 
-// Asynchronous copy of 4 bytes global -> shared (no register round trip).
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
+// Asynchronous copies global -> shared of one value and of 16 bytes (aligned).
+template <class A> __device__ __forceinline__ void cp_async1(A* smem_dst, const A* gmem_src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
+    if constexpr (sizeof(A) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gmem_src) : "memory");
 }
-
-// Asynchronous copy of 16 bytes global -> shared (both addresses 16-byte aligned).
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
 }
 
-// n floats global -> shared: 16-byte copies where both ends are 16-byte aligned and n is a multiple
-// of 4, else 4-byte copies.
-__device__ __forceinline__ void cl_copy_async(float* dst, const float* src, int n, int tid, int nthr) {
-    if (((reinterpret_cast<unsigned long long>(dst) | reinterpret_cast<unsigned long long>(src)) & 15ULL) == 0 &&
-        (n & 3) == 0) {
-        for (int p = tid * 4; p < n; p += nthr * 4) cp_async16(dst + p, src + p);
-    } else {
-        for (int p = tid; p < n; p += nthr) cp_async4(dst + p, src + p);
-    }
-}
-
-// Staging for FP32 storage: every copy (b with ghost rows, faces, this CTA's stencil rows and rows
-// of the coarsest inverse) is issued asynchronously before one wait; the Jacobi weights follow
-// from the staged data.  Same values as the register path.
+// The staged constants of CTA blockIdx.x (a plan's images are laid out once per handle): stencils, weights
+// and faces on own and ghost rows, padded to whole vectors with zeros, and the CTA's rows of the coarsest
+// inverse, and the program (nprog operations).
 template <class SI>
-__device__ __forceinline__ void cl_stage_async(const ClCtx<SI>& t, int rank, int L, int T, float* sm, const Vec<SI>& bv,
-                                               int item, int tid, int nthr) {
-    const Geo& g = t.g[0];
-    const int a = t.rlo[0][rank], nr = t.rlo[0][rank + 1] - a;
-    const int ld0 = g.n0 + 2 * kClPad, xs0 = (t.maxr[0] + 2) * ld0;
-    float* B0 = sm + t.off[0] + 2 * xs0;
-    const float* bsrc = reinterpret_cast<const float*>(bv.d) + (long long)item * bv.bs;
-    const bool b16 = (g.n0 & 3) == 0 && (reinterpret_cast<unsigned long long>(bsrc) & 15ULL) == 0;
-    if (nr > 0 && b16) {
-        // rows of 16-byte vectors (padded shared rows start aligned)
-        const int nv = g.n0 / 4, nb0 = (nr + 2) * nv;
-        for (int q = tid; q < nb0; q += nthr) {
-            const int lr = cl_div(q, t.magicv[0]) - 1;
-            const int row = a + lr, c = (q - (lr + 1) * nv) * 4;
-            float* d = B0 + (lr + 1) * ld0 + c + kClPad;
-            if (row >= 0 && row < g.n1) cp_async16(d, bsrc + (long long)row * g.n0 + c);
-            else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
+__global__ void __launch_bounds__(kBlock) k_cluster_image(const __grid_constant__ ClCtx<SI> t, typename PT<SI>::A* imgs,
+                                                          const ClOp* prog, int nprog) {
+    pdl_prologue();
+    using A = typename PT<SI>::A;
+    constexpr int VN = ClVec<A>::n;
+    const int rank = blockIdx.x, tid = threadIdx.x;
+    A* img = imgs + (long long)rank * t.img_len - t.img_off;      // indexed by shared-memory offsets
+    for (int p = tid; p < nprog; p += kBlock)
+        reinterpret_cast<ClOp*>(reinterpret_cast<char*>(img) + t.prog_off)[p] = prog[p];
+    // rows [a - E, a + nr + E) of src(row, col) inside the grid, n columns, at dst (row -E first), stride ss
+    auto rows = [&](A* dst, int ss, int l, int E, int extra, int n, auto&& src) {
+        const int a = t.rlo[l][rank], nr = t.rlo[l][rank + 1] - a + extra, n1 = t.n1[l] + extra;
+        for (int p = tid; p < (nr + 2 * E) * ss; p += kBlock) {
+            const int r = p / ss, c = p - r * ss, row = a + r - E;
+            dst[p] = c < n && row >= 0 && row < n1 ? src(row, c) : A(0);
         }
-    } else if (nr > 0) {
-        const int nb0 = (nr + 2) * g.n0;
-        for (int p = tid; p < nb0; p += nthr) {
-            const int lr = cl_div(p, t.magic[0]) - 1;
-            const int row = a + lr, c = p - (lr + 1) * g.n0;
-            if (row >= 0 && row < g.n1) cp_async4(B0 + (lr + 1) * ld0 + c + kClPad, bsrc + (long long)row * g.n0 + c);
-            else B0[(lr + 1) * ld0 + c + kClPad] = 0.f;
-        }
+    };
+    for (int l = 0; l < t.T; ++l) {
+        const int np = t.nvp[l] * VN, n0 = t.n0[l], H = t.H[l];
+        if (t.woff[l] >= 0)
+            rows(img + t.woff[l], np, l, H, 0, n0, [&](int r, int c) { return t.W[l][(long long)r * n0 + c]; });
+        if (t.soff[l] >= 0)
+            for (int k = 0; k < 9; ++k)
+                rows(img + t.soff[l] + k * (t.maxr[l] + 2 * (H - 1)) * np, np, l, H - 1, 0, n0, [&](int r, int c) {
+                    A v = PT<SI>::ld(t.sten[l][(long long)k * n0 * t.n1[l] + (long long)r * n0 + c]);
+                    if constexpr (PT<SI>::scaled) v *= t.sten_sc[l][k];
+                    return v;
+                });
     }
-    const int w = g.n0 + 1;
-    if (t.fine0 && t.has_faces) {
-        const int nfx = nr * w, nfy = (nr + 1) * g.n0;
-        const float* fx = reinterpret_cast<const float*>(t.fx) + (long long)a * w;
-        const float* fy = reinterpret_cast<const float*>(t.fy) + (long long)a * g.n0;
-        for (int p = tid; p < nfx; p += nthr) cp_async4(sm + t.fxoff + p, fx + p);
-        for (int p = tid; p < nfy; p += nthr) cp_async4(sm + t.fyoff + p, fy + p);
-    }
-    for (int l = t.fine0 ? 1 : 0; l < L - 1; ++l) {
-        if (t.sten_global[l]) continue;
-        const Geo& gl = t.g[l];
-        const bool dist = l < T;
-        const int al = dist ? t.rlo[l][rank] : 0;
-        const int npl = dist ? (t.rlo[l][rank + 1] - al) * gl.n0 : (int)gl.nx;
-        const int cs = t.maxr[l] * gl.n0;
-        const float* src = reinterpret_cast<const float*>(t.sten[l]) + (long long)al * gl.n0;
-        for (int q = 0; q < 9; ++q) cl_copy_async(sm + t.soff[l] + q * cs, src + (long long)q * gl.nx, npl, tid, nthr);
+    if (t.has_faces) {
+        const int n0 = t.n0[0], np = t.nvp[0] * VN, E = t.H[0] - 1;
+        rows(img + t.fxoff, np + 2 * kClPad, 0, E, 0, n0 + 1, [&](int r, int c) { return t.fx[(long long)r * (n0 + 1) + c]; });
+        rows(img + t.fyoff, np, 0, E, 1, n0, [&](int r, int c) { return t.fy[(long long)r * n0 + c]; });
     }
     if (!t.dinv_global) {
-        const int nc = (int)t.g[L - 1].nx;
-        const int n = (t.cs[rank + 1] - t.cs[rank]) * nc;
-        const float* src = reinterpret_cast<const float*>(t.Dinv) + (long long)t.cs[rank] * nc;
-        cl_copy_async(sm + t.dinv_off, src, n, tid, nthr);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    // Jacobi weights omega / a_PP from the staged faces / stencil centres
-    if (t.fine0 && !t.w0_const) {
-        const int np0 = nr * g.n0;
-        for (int p = tid; p < np0; p += nthr) {
-            float kd;
-            if (t.has_faces) {
-                const int lr = cl_div(p, t.magic[0]);
-                const int c = p - lr * g.n0;
-                const float* fxr = sm + t.fxoff + lr * w;
-                const float* fyr = sm + t.fyoff + lr * g.n0;
-                kd = fxr[c] + fxr[c + 1] + fyr[c] + fyr[c + g.n0];
-            } else {
-                kd = 2.f * (float)g.hx2 + 2.f * (float)g.hy2;
-            }
-            sm[t.woff[0] + p] = t.omega / (t.sigma + t.c * kd);
-        }
-    }
-    for (int l = t.fine0 ? 1 : 0; l < L - 1; ++l) {
-        const Geo& gl = t.g[l];
-        const bool dist = l < T;
-        const int al = dist ? t.rlo[l][rank] : 0;
-        const int npl = dist ? (t.rlo[l][rank + 1] - al) * gl.n0 : (int)gl.nx;
-        const int cs = t.maxr[l] * gl.n0;
-        if (t.sten_global[l]) {
-            const float* ctr = reinterpret_cast<const float*>(t.sten[l]) + 4 * gl.nx + (long long)al * gl.n0;
-            for (int p = tid; p < npl; p += nthr) sm[t.woff[l] + p] = t.omega / ctr[p];
-        } else {
-            for (int p = tid; p < npl; p += nthr) sm[t.woff[l] + p] = t.omega / sm[t.soff[l] + 4 * cs + p];
+        const int nc = t.n0[t.T] * t.n1[t.T], m = (t.cs[rank + 1] - t.cs[rank]) * t.ncp;
+        for (int p = tid; p < m; p += kBlock) {
+            const int r = p / t.ncp, c = p - r * t.ncp;
+            img[t.dinv_off + p] = c < nc ? t.Dinv[(long long)(t.cs[rank] + r) * nc + c] : A(0);
         }
     }
 }
 
 // All mg_cycles V-cycles of (M + c K) x = b, b and x in global memory: cluster k of the grid solves
 // batch item k (grid = C x items CTAs; clusters never wait on one another).
-template <class SI>
-__global__ void __launch_bounds__(kClThreads, 1) k_cluster_mg(const ClCtx<SI>* __restrict__ ctx, const int* active,
+template <class SI, bool FACES, bool GLOBAL>
+__global__ void __launch_bounds__(kClThreads, 1) k_cluster_mg(const __grid_constant__ ClCtx<SI> t, const int* active,
                                                               Vec<SI> bv, Vec<SI> xout) {
     pdl_prologue();
     using A = typename PT<SI>::A;
-    __shared__ ClShared<SI> S;
-    extern __shared__ __align__(16) unsigned char cl_smem[];
-    A* sm = reinterpret_cast<A*>(cl_smem);
+    constexpr int VN = ClVec<A>::n;
+    constexpr bool kSame = std::is_same<SI, A>::value;
+    __shared__ ClL<A> lev[kClMaxLevels];
+    A* const sm = cl_sm<A>();
     const int item = cl_item();               // one cluster per batch item
     if (active && !active[item]) return;      // the same decision in every CTA of the cluster
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    {
-        const int* src = reinterpret_cast<const int*>(ctx);
-        int* dst = reinterpret_cast<int*>(&S.t);
-        for (int i = tid; i < (int)(sizeof(ClCtx<SI>) / sizeof(int)); i += nthr) dst[i] = src[i];
-    }
-    __syncthreads();
-    const ClCtx<SI>& t = S.t;
+    const int tid = threadIdx.x, nthr = kClThreads;
     const int rank = (int)cl_rank();
-    const int L = t.L, T = t.T;
-    if (tid == 0) S.rank = rank;
-    // zero the padding columns and ghost rows of every x / b buffer (interiors are written before
-    // they are read; the zeros stand for the Dirichlet boundary)
-    for (int l = 0; l < L; ++l) {
-        const int ld = t.g[l].n0 + 2 * kClPad, rows = t.maxr[l] + 2, xs = rows * ld;
-        const int nrl = l < T ? t.rlo[l][rank + 1] - t.rlo[l][rank] : t.g[l].n1;   // this CTA's rows
-        A* base = sm + t.off[l];
-        const int nedge = 2 * ld + 2 * rows;          // ghost rows -1 and nrl, two padding columns
-        for (int i = tid; i < 3 * nedge; i += nthr) {
-            const int k = i / nedge, e = i - k * nedge;
-            int idx;
-            if (e < ld) idx = e;                                  // ghost row -1
-            else if (e < 2 * ld) idx = (nrl + 1) * ld + e - ld;   // ghost row nrl
-            else if (e < 2 * ld + rows) idx = (e - 2 * ld) * ld + kClPad - 1;          // column -1
-            else idx = (e - 2 * ld - rows) * ld + kClPad + t.g[l].n0;                 // column n0
-            base[k * xs + idx] = A(0);
-        }
-    }
-    if (tid < T) {
-        const int l = tid;
-        ClLev<A>& v = S.lv[l];
-        v.a = t.rlo[l][rank];
-        v.nr = t.rlo[l][rank + 1] - v.a;
-        int pr = rank - 1;
-        while (pr >= 0 && t.rlo[l][pr + 1] == t.rlo[l][pr]) --pr;
-        int nx = rank + 1;
-        while (nx < t.C && t.rlo[l][nx + 1] == t.rlo[l][nx]) ++nx;
-        const int ld = t.g[l].n0 + 2 * kClPad, xs = (t.maxr[l] + 2) * ld;
-        for (int k = 0; k < 3; ++k) {
-            v.pu[k] = nullptr;
-            v.pd[k] = nullptr;
-            if (v.nr > 0 && v.a > 0 && pr >= 0) {
-                const int cnt = t.rlo[l][pr + 1] - t.rlo[l][pr];     // its ghost row below is row cnt
-                v.pu[k] = cl_map(sm + t.off[l] + k * xs + (cnt + 1) * ld + kClPad, (unsigned)pr);
-            }
-            if (v.nr > 0 && v.a + v.nr < t.g[l].n1 && nx < t.C)
-                v.pd[k] = cl_map(sm + t.off[l] + k * xs + kClPad, (unsigned)nx);     // its ghost row -1
-        }
-    }
-    // row table of level T-1 (the restriction into the coarsest level reads every row of it)
-    const A** rowtab = reinterpret_cast<const A**>(sm + t.rowtab_off);
+    const int C = t.C, L = t.L, T = t.T;
+    // ---- the constants' image
     {
-        const int l = T - 1;
-        const int ld = t.g[l].n0 + 2 * kClPad;
-        for (int i = tid; i < t.g[l].n1; i += nthr) {
-            int r = 0;
-            while (r + 1 < t.C && t.rlo[l][r + 1] <= i) ++r;
-            A* q = sm + t.off[l] + (i - t.rlo[l][r] + 1) * ld + kClPad;
-            rowtab[i] = r == rank ? q : cl_map(q, (unsigned)r);
-        }
+        const A* src = t.img + (long long)rank * t.img_len;
+        constexpr int N16 = 16 / (int)sizeof(A);
+        for (int p = tid * N16; p < t.img_len; p += nthr * N16) cp_async16(sm + t.img_off + p, src + p);
     }
-    if (tid == 0 && t.w0_const) {
-        // the formula of the staged weights (FD, kappa = 1: the same at every point)
-        const Geo& g = t.g[0];
-        const A kd = A(2) * A(g.hx2) + A(2) * A(g.hy2);
-        S.w0 = t.omega / (t.sigma + t.c * kd);
-    }
-    __syncthreads();
-    if (tid < L) S.lev[tid] = cl_level(S, sm, tid);
-    if constexpr (std::is_same<SI, float>::value && std::is_same<typename PT<SI>::A, float>::value) {
-        cl_stage_async(t, rank, L, T, sm, bv, item, tid, nthr);
-    } else {
-        // ---- stage b, faces, stencils, Jacobi weights and this CTA's rows of the coarsest inverse
-        // (loads from global memory are issued in groups before the shared-memory stores)
-        {
-            constexpr int U = 4;
-            const Geo& g = t.g[0];
-            const int a = t.rlo[0][rank], nr = t.rlo[0][rank + 1] - a;
-            const int np0 = nr * g.n0, ld0 = g.n0 + 2 * kClPad, xs0 = (t.maxr[0] + 2) * ld0;
-            View<SI> bs = view_of(bv, item, 0, g.n0);
-            A* B0 = sm + t.off[0] + 2 * xs0;
-            // rows a-1 .. a+nr of b (the ghost rows too: the residual of a zero guess is b)
-            const int nb0 = nr > 0 ? (nr + 2) * g.n0 : 0;
-            for (int p0 = tid; p0 < nb0; p0 += U * nthr) {
-                A v[U];
-    #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int p = p0 + u * nthr;
-                    const int lr = cl_div(p, t.magic[0]) - 1;
-                    const int row = a + lr;
-                    v[u] = p < nb0 && row >= 0 && row < g.n1 ? bs.at(row, p - (lr + 1) * g.n0) : A(0);
-                }
-    #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int p = p0 + u * nthr;
-                    const int lr = cl_div(p, t.magic[0]) - 1;
-                    if (p < nb0) B0[(lr + 1) * ld0 + p - (lr + 1) * g.n0 + kClPad] = v[u];
-                }
+    // ---- b on own and ghost rows (rows beyond the grid and padding columns are zero)
+    {
+        const int a = t.rlo[0][rank], nr = t.rlo[0][rank + 1] - a, H = t.H[0], n0 = t.n0[0], n1 = t.n1[0];
+        const int nvp = t.nvp[0], ld = nvp * VN + 2 * kClPad;
+        A* B = sm + t.off[0] + 2 * (t.maxr[0] + 2 * H) * ld + kClPad;
+        const A* src = reinterpret_cast<const A*>(bv.d) + (long long)item * bv.bs;
+        View<SI> bs = view_of(bv, item, 0, n0);
+        const bool vec = kSame && sizeof(A) == 4 && n0 % VN == 0 && (reinterpret_cast<unsigned long long>(src) & 15ULL) == 0;
+        for (int i = tid; i < (nr + 2 * H) * nvp; i += nthr) {
+            const int r = cl_div(i, t.magicv[0]), c = (i - r * nvp) * VN, row = a + r - H;
+            A* d = B + r * ld + c;
+            const bool in = row >= 0 && row < n1;
+            if (in && vec) {
+                cp_async16(d, src + (long long)row * n0 + c);
+                continue;
             }
-            if (t.fine0 && !t.w0_const) {
-                const int w = g.n0 + 1;
-                if (t.has_faces) {
-                    const int nfx = nr * w, nfy = (nr + 1) * g.n0;
-                    const A* fx = t.fx + (long long)a * w;
-                    const A* fy = t.fy + (long long)a * g.n0;
-                    for (int p0 = tid; p0 < nfx; p0 += U * nthr) {
-                        A v[U];
-    #pragma unroll
-                        for (int u = 0; u < U; ++u) v[u] = p0 + u * nthr < nfx ? fx[p0 + u * nthr] : A(0);
-    #pragma unroll
-                        for (int u = 0; u < U; ++u)
-                            if (p0 + u * nthr < nfx) sm[t.fxoff + p0 + u * nthr] = v[u];
-                    }
-                    for (int p0 = tid; p0 < nfy; p0 += U * nthr) {
-                        A v[U];
-    #pragma unroll
-                        for (int u = 0; u < U; ++u) v[u] = p0 + u * nthr < nfy ? fy[p0 + u * nthr] : A(0);
-    #pragma unroll
-                        for (int u = 0; u < U; ++u)
-                            if (p0 + u * nthr < nfy) sm[t.fyoff + p0 + u * nthr] = v[u];
-                    }
-                }
-                for (int p0 = tid; p0 < np0; p0 += U * nthr) {
-                    A kd[U];
-    #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int p = p0 + u * nthr;
-                        const int lr = cl_div(p, t.magic[0]);
-                        const int c = p - lr * g.n0;
-                        if (t.has_faces && p < np0) {
-                            const long long fxi = (long long)(a + lr) * w + c, fyi = (long long)(a + lr) * g.n0 + c;
-                            kd[u] = t.fx[fxi] + t.fx[fxi + 1] + t.fy[fyi] + t.fy[fyi + g.n0];
-                        } else {
-                            kd[u] = A(2) * A(g.hx2) + A(2) * A(g.hy2);
-                        }
-                    }
-    #pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (p0 + u * nthr < np0) sm[t.woff[0] + p0 + u * nthr] = t.omega / (t.sigma + t.c * kd[u]);
-                }
-            }
-            for (int l = t.fine0 ? 1 : 0; l < L - 1; ++l) {
-                const Geo& gl = t.g[l];
-                const bool dist = l < T;
-                const int al = dist ? t.rlo[l][rank] : 0;
-                const int npl = dist ? (t.rlo[l][rank + 1] - al) * gl.n0 : (int)gl.nx;
-                const int cs = t.maxr[l] * gl.n0;
-                const SI* src = t.sten[l] + (long long)al * gl.n0;
-                if (t.sten_global[l]) {
-                    // read in place by the vector steps: only the Jacobi weights are staged
-                    for (int p = tid; p < npl; p += nthr) {
-                        A ctr = PT<SI>::ld(src[4 * gl.nx + p]);
-                        if constexpr (PT<SI>::scaled) ctr *= t.sten_sc[l][4];
-                        sm[t.woff[l] + p] = t.omega / ctr;
-                    }
-                    continue;
-                }
-                for (int p = tid; p < npl; p += nthr) {
-                    A v[9];
-    #pragma unroll
-                    for (int q = 0; q < 9; ++q) v[q] = PT<SI>::ld(src[(long long)q * gl.nx + p]);
-    #pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        if constexpr (PT<SI>::scaled) v[q] *= t.sten_sc[l][q];
-                        sm[t.soff[l] + q * cs + p] = v[q];
-                    }
-                    sm[t.woff[l] + p] = t.omega / v[4];
-                }
-            }
-            if (!t.dinv_global) {
-                const int nc = (int)t.g[L - 1].nx;
-                const int n = (t.cs[rank + 1] - t.cs[rank]) * nc;
-                const A* src = t.Dinv + (long long)t.cs[rank] * nc;
-                for (int p0 = tid; p0 < n; p0 += U * nthr) {
-                    A v[U];
-    #pragma unroll
-                    for (int u = 0; u < U; ++u) v[u] = p0 + u * nthr < n ? src[p0 + u * nthr] : A(0);
-    #pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (p0 + u * nthr < n) sm[t.dinv_off + p0 + u * nthr] = v[u];
+#pragma unroll
+            for (int q = 0; q < VN; ++q) {
+                if (!in || c + q >= n0) {
+                    d[q] = A(0);
+                } else if constexpr (kSame) {
+                    cp_async1(d + q, src + (long long)row * n0 + c + q);
+                } else {
+                    d[q] = bs.at(row, c + q);
                 }
             }
         }
+        for (int i = tid; i < 2 * (t.maxr[0] + 2 * H); i += nthr)      // columns -1 and beside the last vector
+            B[(i >> 1) * ld + ((i & 1) ? nvp * VN : -1)] = A(0);
     }
+    // ---- zero x of every level, b of the others, the inboxes (the boundary's ghost rows and columns)
+    {
+        const A z[VN] = {};
+        for (int l = 0; l < L; ++l) {
+            const int xs = (t.maxr[l] + 2 * t.H[l]) * (t.nvp[l] * VN + 2 * kClPad);
+            for (int p = tid * VN; p < (l == 0 ? 2 : 3) * xs; p += nthr * VN) cl_vstore(sm + t.off[l] + p, z);
+            const int in = 2 * t.ix[l] * (t.nvp[l] * VN + 2 * kClPad);
+            for (int p = tid * VN; p < in; p += nthr * VN) cl_vstore(sm + t.ioff[l] + p, z);
+        }
+        for (int p = tid; p < t.ncp; p += nthr) sm[t.boff + p] = A(0);      // the padding stays zero
+    }
+    // ---- the levels of this CTA
+    if (tid < L) {
+        const int l = tid;
+        ClL<A>& v = lev[l];
+        const int np = t.nvp[l] * VN, H = t.H[l];
+        v.n0 = t.n0[l];
+        v.nvp = t.nvp[l];
+        v.ld = np + 2 * kClPad;
+        v.H = H;
+        v.ix = t.ix[l];
+        v.xs = (t.maxr[l] + 2 * H) * v.ld;
+        v.magicv = t.magicv[l];
+        v.a = l < T ? t.rlo[l][rank] : 0;
+        v.nr = l < T ? t.rlo[l][rank + 1] - v.a : t.n1[l];
+        v.rest = t.n1[l] - v.a;
+        v.per = t.per[l];
+        v.X = t.off[l] + H * v.ld + kClPad;
+        v.in = t.ioff[l] + kClPad;
+        v.W = t.woff[l] + H * np;
+        v.kind = l == 0 && t.fine0 ? (t.has_faces ? 2 : 1) : 0;
+        v.fx = t.fxoff + (H - 1) * v.ld;
+        v.fy = t.fyoff + (H - 1) * np;
+        v.S = t.soff[l] + (H - 1) * np;
+        v.cs = (t.maxr[l] + 2 * (H - 1)) * np;
+        v.Sg = nullptr;
+        v.Ssc = nullptr;
+        if (l < T && t.sten_global[l]) {
+            v.cs = v.n0 * t.n1[l];
+            v.Sg = t.sten[l] + (long long)v.a * v.n0;
+            v.Ssc = t.sten_sc[l];
+        }
+        if constexpr (std::is_same<A, double>::value) {
+            v.cf[0][0] = v.cf[1][0] = v.cf[3][0] = t.w0;
+            v.cf[0][1] = t.k0;
+            v.cf[0][2] = t.kx;
+            v.cf[0][3] = t.ky;
+            v.cf[2][0] = A(1);
+            v.cf[2][1] = -t.d0;
+            v.cf[2][2] = t.ex;
+            v.cf[2][3] = t.ey;
+            for (int q = 1; q < 4; ++q) v.cf[3][q] = t.w0 * v.cf[0][q];
+        } else {
+            for (int q = 0; q < 4; ++q) {
+                const A k = q == 3 ? t.w0 : A(1);          // mode 3: A acts on w0 b
+                v.cf[q][0] = q == 2 ? A(1) : t.w0;
+                v.cf[q][1] = k * t.sigma;
+                v.cf[q][2] = k * t.ex;
+                v.cf[q][3] = k * t.ey;
+            }
+        }
+        v.cf[1][1] = v.cf[1][2] = v.cf[1][3] = A(0);
+        v.mP[0] = A(1);
+        v.mP[1] = v.mP[2] = A(0);
+        v.mP[3] = t.w0;
+        v.hx2 = t.hx2;
+        v.hy2 = t.hy2;
+        v.sigma = t.sigma;
+        v.c = t.c;
+        auto rows = [&](int r) { return l < T && r >= 0 && r < C ? t.rlo[l][r + 1] - t.rlo[l][r] : 0; };
+        const int reach = max(H, t.ix[l]);
+        for (int q = 0; q < kClReach; ++q) {
+            v.prev[q] = rows(rank - 1 - q);
+            v.next[q] = rows(rank + 1 + q);
+        }
+        v.far = (v.prev[0] > 0 && v.prev[0] < reach) || (v.next[0] > 0 && v.next[0] < reach);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     cl_sync();     // every CTA of the cluster is resident and staged before any remote access
-    unsigned cur = 0u;       // bit l: buffer of level l holding the iterate
+    const int nc = t.n0[T] * t.n1[T];
+    const ClOp* prog = reinterpret_cast<const ClOp*>(cl_sm<unsigned char>() + t.prog_off);
+#pragma unroll 1
     for (int cyc = 0; cyc < t.cycles; ++cyc) {
-        bool zero = cyc == 0;
-        // ---- down: distributed levels (l < T) step with cluster barriers, replicated ones with
-        // block barriers
-        for (int l = 0; l < L - 1; ++l) {
-            const bool dist = l < T;
-            const ClL<A>& f = S.lev[l];
-            int k = (cur >> l) & 1u;
-            for (int sw = 0; sw < t.nu1; ++sw) {
-                cl_sweep_any<SI>(f, k, zero && sw == 0, tid, nthr);
-                k ^= 1;
-                cl_step_sync(dist);
-            }
-            int kr;
-            if (zero && t.nu1 == 0) {
-                // x = 0: the residual is b; clear x (own and ghost rows) for the interpolation later
-                kr = 2;
-                const int nz = f.nr > 0 ? (f.nr + 2) * f.n0 : 0;
-                for (int p = tid; p < nz; p += nthr) {
-                    const int lr = cl_div(p, f.magic) - 1;
-                    *f.el(k, lr, p - (lr + 1) * f.n0) = A(0);
+        const int part = cyc == 0 ? 0 : 2 - (cyc & 1);
+        const int end = t.pc[part + 1];
+        ClOp next = prog[t.pc[part]];
+#pragma unroll 1
+        for (int pc = t.pc[part]; pc < end; ++pc) {
+            ClOp op = next;
+            next = prog[pc + 1];                      // (the program ends with a spare operation)
+            const ClL<A>& f = lev[op.lev];
+            // the last operation's rows go to no further cycle
+            if (pc == end - 1 && cyc == t.cycles - 1) op.depth = op.flags = 0;
+            if (op.kind == kClStep) {
+                cl_step<SI, FACES, GLOBAL>(f, rank, op.mode, op.kin, op.kc, op.ext, op.depth, (op.flags & 1) != 0);
+            } else if (op.kind == kClProlong) {
+                cl_prolong<PT<SI>::scaled>(f, lev[op.lev + 1], rank, op.kin, op.kc, op.ext, op.depth);
+            } else if (op.kind == kClRestrict) {
+                cl_restrict<PT<SI>::scaled>(f, lev[op.lev + 1], rank, op.kin, op.mode ? op.kc : -1);
+            } else if (op.kind == kClRestrictLast) {
+                // into every CTA's copy of the coarsest b: one value and one destination per thread
+                const int n0c = t.n0[T], ja = t.rlo[T][rank], nv = (t.rlo[T][rank + 1] - ja) * n0c;
+                for (int i = tid; i < nv * C; i += nthr) {
+                    const int p = i / C, dst = i - p * C;
+                    const int jr = cl_div(p, t.magic[T]), I = p - jr * n0c, J = ja + jr;
+                    const A* row = sm + f.X + op.kin * f.xs + (2 * J - f.a) * f.ld + 2 * I;
+                    A acc = A(0);
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const A wy = dy == 1 ? A(1) : A(0.5);
+                        acc += A(0.5) * wy * row[dy * f.ld];
+                        acc += wy * row[dy * f.ld + 1];
+                        acc += A(0.5) * wy * row[dy * f.ld + 2];
+                    }
+                    cl_rstore(t.boff + J * n0c + I, dst, acc);
                 }
-                cl_step_sync(dist);                       // b rows were written by this level's restriction
-            } else {
-                cl_residual_any<SI>(f, k, tid, nthr);
-                kr = k ^ 1;
-                cl_step_sync(dist);
-            }
-            cur = (cur & ~(1u << l)) | ((unsigned)k << l);
-            const ClL<A>& cv = S.lev[l + 1];
-            // vector restriction: coarse points in vectors and the fine rows 16-byte aligned too
-            if (dist && l + 1 < T && cv.vec && f.n0 % ClVec<A>::n == 0) cl_restrict_v(f, cv, kr, tid, nthr);
-            else cl_restrict(f, cv, kr, dist && l + 1 >= T, rowtab, tid, nthr);
-            __syncthreads();
-            zero = true;
-        }
-        // ---- coarsest level, held whole by every CTA: x = A_c^{-1} b, this CTA's rows one warp
-        // per row, then the other CTAs' rows gathered after a cluster barrier
-        {
-            const int l = L - 1;
-            const ClL<A> v = S.lev[l];
-            const int nc = v.n0 * v.n1;
-            const int k = (cur >> l) & 1u;
-            A* bvec = v.X + (1 - k) * v.xs;           // b of the coarsest level, unpadded copy
-            for (int p = tid; p < nc; p += nthr) {
-                const int lr = cl_div(p, v.magic);
-                bvec[p] = *v.el(2, lr, p - lr * v.n0);
-            }
-            __syncthreads();
-            const A* Di = t.dinv_global ? t.Dinv + (long long)t.cs[rank] * nc : sm + t.dinv_off;
-            const int lo = t.cs[rank], hi = t.cs[rank + 1];
-            const int w = tid >> 5, lane = tid & 31, nw = nthr >> 5;
-            for (int p = lo + w; p < hi; p += nw) {
-                const A* row = Di + (p - lo) * nc;
-                A acc = A(0);
-                for (int q = lane; q < nc; q += kWarp) acc += row[q] * bvec[q];
-                acc = warp_sum(acc);
-                if (lane == 0) {
-                    const int lr = cl_div(p, v.magic);
-                    *v.el(k, lr, p - lr * v.n0) = acc;
+            } else if (op.kind == kClSolve) {
+                // this CTA's rows of A_c^{-1} b, eight lanes per row (fewer sums across lanes than a warp per
+                // row), stored into every CTA's x
+                const A* b = sm + t.boff;
+                const int lo = t.cs[rank], hi = t.cs[rank + 1], j = tid & 7, ncp = t.ncp;
+                for (int p0 = lo; p0 < hi; p0 += nthr / 8) {
+                    const int p = p0 + (tid >> 3);
+                    A acc[4] = {A(0), A(0), A(0), A(0)};
+                    if (p < hi) {
+                        const A* row = t.dinv_global ? t.Dinv + (long long)p * ncp : sm + t.dinv_off + (p - lo) * ncp;
+                        if constexpr (VN > 1) {
+#pragma unroll 4
+                            for (int q = j * VN; q < ncp; q += 8 * VN) {
+                                A d[VN], u[VN];
+                                cl_vload(row + q, d);
+                                cl_vload(b + q, u);
+#pragma unroll
+                                for (int i = 0; i < VN; ++i) acc[i] += d[i] * u[i];
+                            }
+                        } else {
+                            int q = j;
+                            for (; q + 24 < ncp; q += 32)
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) acc[i] += row[q + 8 * i] * b[q + 8 * i];
+                            for (; q < ncp; q += 8) acc[0] += row[q] * b[q];
+                        }
+                    }
+                    A s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    if (p < hi) {
+                        const int lr = cl_div(p, t.magic[T]), at = f.X + lr * f.ld + p - lr * f.n0;
+                        for (int d = j; d < C; d += 8) cl_rstore(at, d, s);
+                    }
                 }
-            }
-            cl_sync();
-            for (int p = tid; p < nc; p += nthr) {
-                if (p >= lo && p < hi) continue;
-                int r = 0;
-                while (r + 1 < t.C && t.cs[r + 1] <= p) ++r;
-                const int lr = cl_div(p, v.magic);
-                A* q = v.el(k, lr, p - lr * v.n0);
-                *q = *cl_map(q, (unsigned)r);
-            }
-            __syncthreads();
-        }
-        // ---- up
-        for (int l = L - 2; l >= 0; --l) {
-            const bool dist = l < T;
-            const ClL<A>& f = S.lev[l];
-            const ClL<A>& cv = S.lev[l + 1];
-            int k = (cur >> l) & 1u;
-            const int kc = (cur >> (l + 1)) & 1u;
-            if (t.nu2 > 0) {
-                // x += P x_c in place on own and ghost rows (no remote store: every CTA computes its
-                // ghost rows itself), then the first sweep into the other buffer; a neighbour's
-                // stores of that sweep land in a buffer nobody reads during this step
-                if (f.vec) cl_prolong_ext_v(f, cv, k, kc, k, tid, nthr);
-                else cl_prolong_ext(f, cv, k, kc, k, tid, nthr);
-                __syncthreads();
-                for (int sw = 0; sw < t.nu2; ++sw) {
-                    cl_sweep_any<SI>(f, k, false, tid, nthr);
-                    k ^= 1;
-                    cl_step_sync(dist);
+            } else if (op.kind == kClInbox) {
+                // the previous cycle's x: its ghost rows arrived in the inbox
+                const int H = f.H;
+                for (int i = tid; i < 2 * H * f.nvp; i += nthr) {
+                    const int r = cl_div(i, f.magicv), c = (i - r * f.nvp) * VN;
+                    A x[VN];
+                    cl_vload(sm + f.in + r * f.ld + c, x);
+                    cl_vstore(sm + f.X + op.kin * f.xs + (r < H ? r - H : f.nr + r - H) * f.ld + c, x);
                 }
             } else {
-                cl_prolong(f, cv, k, kc, tid, nthr);
-                cl_step_sync(dist);
+                // no sweep on a zero guess: clear x for the interpolation later
+                const A z[VN] = {};
+                for (int i = tid; i < (f.nr + 2 * f.H) * f.nvp; i += nthr) {
+                    const int r = cl_div(i, f.magicv), c = (i - r * f.nvp) * VN;
+                    cl_vstore(sm + f.X + op.kin * f.xs + (r - f.H) * f.ld + c, z);
+                }
             }
-            cur = (cur & ~(1u << l)) | ((unsigned)k << l);
+            cl_step_sync((op.flags & 2) != 0);
         }
     }
     // ---- write this CTA's rows of x_0
     {
-        const ClL<A> v = S.lev[0];
-        const int k = cur & 1u;
+        const ClL<A>& v = lev[0];
+        const int k = t.kfin;
         if constexpr (PT<SI>::scaled) {
             const int w = tid >> 5, lane = tid & 31, nw = nthr >> 5;
             for (int lr = w; lr < v.nr; lr += nw) {
                 SI* o;
                 float* osc;
                 row_store_ptrs(xout, item, 0, v.a + lr, v.n0, o, osc);
-                const A* X = v.el(k, lr, 0);
+                const A* X = sm + v.X + k * v.xs + lr * v.ld;
                 row_store<SI>(o, osc, v.n0, lane, [&](int c) -> A { return X[c]; });
             }
         } else {
             SI* o = xout.d + (long long)item * xout.bs + (long long)v.a * v.n0;
-            for (int p = tid; p < v.nr * v.n0; p += nthr) {
-                const int lr = cl_div(p, v.magic);
-                o[p] = PT<SI>::st(*v.el(k, lr, p - lr * v.n0));
+            const bool vec = v.n0 % VN == 0;
+            for (int i = tid; i < v.nr * v.nvp; i += nthr) {
+                const int r = cl_div(i, v.magicv), c = (i - r * v.nvp) * VN;
+                const A* x = sm + v.X + k * v.xs + r * v.ld + c;
+                A* d = reinterpret_cast<A*>(o) + r * v.n0 + c;
+                if (vec) {
+                    A u[VN];
+                    cl_vload(x, u);
+                    cl_vstore(d, u);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < VN; ++q)
+                        if (c + q < v.n0) d[q] = x[q];
+                }
             }
         }
     }
+}
+
+// The program of a plan: the operations of the first cycle, of an odd and of an even later one (the
+// buffers alternate with the number of sweeps), and the buffer x_0 ends in.  Every CTA runs the same
+// program, so its barriers match.  A step writes ghost rows of other CTAs' buffers (depth > 0 without
+// the inbox flag) only where a cluster barrier separates it from the last read of those rows: with H = 1 an
+// exchange follows every sweep; on levels with deeper ghost regions (at most two post-sweeps) no sweep but
+// the first post-sweep can be such a step, and the buffer it writes was last read by the restriction.  b and
+// the inboxes are read before the barriers of the steps in between.
+template <class SI> inline std::vector<ClOp> cl_program(ClCtx<SI>& t) {
+    std::vector<ClOp> prog;
+    const int T = t.T, nu1 = t.nu1, nu2 = t.nu2;
+    auto emit = [&](int kind, int l, int mode, int kin, int kc, int ext, int depth, int flags) {
+        prog.push_back(ClOp{(unsigned char)kind, (unsigned char)l, (unsigned char)mode, (unsigned char)kin,
+                            (unsigned char)kc, (unsigned char)ext, (unsigned char)depth,
+                            (unsigned char)(flags | (depth > 0 ? 2 : 0))});
+    };
+    int cur[kClMaxLevels] = {}, reach[kClMaxLevels] = {};     // buffer of x; valid ghost rows of the pre-smoothed x
+    int after[3] = {};
+    for (int part = 0; part < 3; ++part) {
+        t.pc[part] = (int)prog.size();
+        for (int l = 0; l < T; ++l) {
+            const int H = t.H[l];
+            int k = cur[l], v = H;
+            bool zero = part == 0 || l > 0;
+            int sw = 0;
+            if (!zero) {
+                emit(kClInbox, l, 0, k, 0, 0, 0, 0);
+            } else if (l > 0 && nu1 > 0) {
+                sw = 1;                        // the restriction has done the first sweep, into buffer k ^ 1
+                zero = false;
+                k ^= 1;
+            } else if (l == 0 && nu1 > 1 && t.fuse0) {
+                // two sweeps from b at once
+                const int ext = std::min(v - 1, nu1 - 2 + 2), depth = ext == 0 ? H : 0;
+                emit(kClStep, l, 3, 2, k, ext, depth, 0);
+                v = depth > 0 ? H : ext;
+                sw = 2;
+                zero = false;
+            }
+            for (; sw < nu1; ++sw) {
+                // the result is read up to (sweeps left) + 2 rows beyond the own ones
+                const int ext = std::min(zero ? v : v - 1, nu1 - 1 - sw + 2);
+                const int depth = ext == 0 ? H : 0;
+                emit(kClStep, l, zero ? 1 : 0, k, k ^ 1, ext, depth, 0);
+                v = depth > 0 ? H : ext;
+                zero = false;
+                k ^= 1;
+            }
+            int kr = 2;                        // no sweep on a zero guess: the residual is b
+            if (zero) {
+                emit(kClClear, l, 0, k, 0, 0, 0, 0);
+            } else {
+                emit(kClStep, l, 2, k, k ^ 1, v >= 2 ? 1 : 0, v >= 2 ? 0 : 1, 0);
+                kr = k ^ 1;
+            }
+            cur[l] = k;
+            reach[l] = v;
+            emit(l + 1 < T ? kClRestrict : kClRestrictLast, l, nu1 > 0 ? 1 : 0, kr, cur[l + 1] ^ 1, 0, 0, 2);
+        }
+        emit(kClSolve, T, 0, 0, 0, 0, 0, 2);
+        for (int l = T - 1; l >= 0; --l) {
+            int k = cur[l];
+            // interpolate on up to nu2 ghost rows: e of them need (e + 2) / 2 rows of x_c beyond the own ones
+            int v = std::min(reach[l], nu2);
+            if (l + 1 < T) v = std::min(v, 2 * t.ix[l + 1] - 1);
+            emit(kClProlong, l, 0, k, l + 1 < T ? cur[l + 1] : 0, v, nu2 == 0 ? t.ix[l] : 0, 0);
+            for (int sw = 0; sw < nu2; ++sw) {
+                const bool fin = sw == nu2 - 1;
+                const int e = std::min(v - 1, nu2 - 1 - sw);
+                const int depth = fin ? t.ix[l] : (e == 0 ? t.H[l] : 0);
+                emit(kClStep, l, 0, k, k ^ 1, e, depth, fin ? 1 : 0);
+                v = depth > 0 ? t.H[l] : e;
+                k ^= 1;
+            }
+            cur[l] = k;
+        }
+        after[part] = cur[0];
+    }
+    t.pc[3] = (int)prog.size();
+    prog.push_back(ClOp{});
+    const int last = t.cycles - 1;
+    t.kfin = after[last == 0 ? 0 : 2 - (last & 1)];
+    return prog;
+}
+
+// omega / a_PP of every point of a level, from its stored stencil or the FD diagonal.
+template <class SI>
+__global__ void __launch_bounds__(kBlock) k_jacobi_weights(LevelOp<SI> op, typename PT<SI>::A omega,
+                                                           typename PT<SI>::A* out) {
+    pdl_prologue();
+    const long long p = (long long)blockIdx.x * kBlock + threadIdx.x;
+    if (p >= op.g.nx) return;
+    const int row = (int)(p / op.g.n0), c = (int)(p - (long long)row * op.g.n0);
+    out[p] = omega / level_diag(op, row, row, 0, c);
 }
 
 }  // namespace aao

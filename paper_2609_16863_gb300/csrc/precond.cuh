@@ -45,6 +45,7 @@ class Precond : public PrecondBase {
     int L = 0;
     Level lev[kMaxLevels];
     A* Dinv[kMaxS] = {};           // dense coarsest inverse per stage
+    A* jacw[kClMaxLevels][kMaxS] = {};   // 2D: Jacobi weights omega / a_PP of the distributed levels
     Faces<A> facesA;
     SpaceOp<A> sopA;                 // fine-grid K (and M for Q1) for the stage kernels
     A* cheb[3] = {};                 // Q1: Chebyshev x, r, d ((nt+1)*nx each)
@@ -86,7 +87,8 @@ class Precond : public PrecondBase {
     struct ClPlan {
         int C = 0;                 // CTAs per cluster; 0: none
         size_t smem = 0;
-        ClCtx<SI>* ctx = nullptr;  // device, one context per stage
+        void (*kernel)(const ClCtx<SI>, const int*, Vec<SI>, Vec<SI>) = nullptr;
+        ClCtx<SI> ctx[kMaxS];      // one context per stage, passed by value
     };
     ClPlan clp[2];                 // [0] single items, [1] batches of at least kClBatch8 items
     int* hact = nullptr;           // pinned mirror of activeh (profiling)
@@ -492,38 +494,48 @@ class Precond : public PrecondBase {
 
     // Plan the cluster-resident shifted solve: 2D, at least one level above the coarsest, every
     // CTA owning rows of every distributed level, its share within shared memory, and the cluster
-    // co-resident on the device.  Two plans: one for single items (16 CTAs where the full layout
+    // co-resident on the device.  Two plans: one for single items (16 CTAs where a layout
     // fits, else 8) and one for batches (8 CTAs, so that about twice as many items run at once:
-    // at 256^2 only 7 clusters of 16 are resident).  A plan that does not fit shared memory is made
-    // lean step by step: level 0's Jacobi weight as a scalar (FD, kappa = 1), the rows of A_c^{-1}
-    // read from global memory, then the coarse stencils read from global memory (L2) from level 1
-    // on (only where the storage type is the arithmetic type).  Lean plans give the same values.
-    bool plan_cluster(int C, int lean, long long dyn_max, ClCtx<SI>& t, long long& bytes) {
+    // at 256^2 only 7 clusters of 16 are resident).  deep: ghost rows for whole smoothing phases (1: on
+    // the coarse levels, 2: on the finest too), else one ghost row.  lean: what is read from global
+    // memory (L2) instead of being staged: 1: the rows of A_c^{-1}, 2: the first coarse stencil, 3: every
+    // coarse stencil.  All give the same values.
+    using ClKernel = void (*)(const ClCtx<SI>, const int*, Vec<SI>, Vec<SI>);
+    // The instance with the code a plan needs: faces of a kappa field, stencils in global memory (less
+    // code is fetched without them).
+    static ClKernel cluster_kernel(const ClCtx<SI>& t) {
+        bool global = false;
+        for (int l = 0; l < t.T; ++l) global = global || t.sten_global[l];
+        if (t.has_faces) return global ? (ClKernel)k_cluster_mg<SI, true, true> : (ClKernel)k_cluster_mg<SI, true, false>;
+        return global ? (ClKernel)k_cluster_mg<SI, false, true> : (ClKernel)k_cluster_mg<SI, false, false>;
+    }
+
+    bool plan_cluster(int C, int deep, int lean, long long dyn_max, ClCtx<SI>& t, long long& bytes) {
         const Geo& g0 = h->g;
         const int T = L - 1;
-        if (g0.n1 < C) return false;
+        constexpr int VN = ClVec<A>::n;
+        if (g0.n1 < C || L > kClMaxLevels) return false;
         const bool fine0 = !h->q1;
         const bool faces = fine0 && h->has_kappa;
-        const bool same = std::is_same<SI, A>::value;
-        const bool w0c = lean >= 1 && fine0 && !faces;
-        // lean >= 2 reads coarse stencils from global memory: in place where the storage type is the
-        // arithmetic type, else (16-bit storage) through the vector steps only, so those levels
-        // must take vectors (checked below)
+        const int nu1 = h->opt.mg_pre, nu2 = h->opt.mg_post;
+        // ghost rows for a whole phase leave no exchange between two sweeps that would write ghost rows a
+        // neighbour still reads; that covers at most two post-sweeps
+        if (deep > 0 && (nu2 > 2 || nu1 > 3)) return false;
         std::memset(&t, 0, sizeof(t));
         t.C = C;
         t.L = L;
         t.T = T;
         t.cycles = h->opt.mg_cycles;
-        t.nu1 = h->opt.mg_pre;
-        t.nu2 = h->opt.mg_post;
-        t.omega = (A)h->opt.mg_omega;
+        t.nu1 = nu1;
+        t.nu2 = nu2;
         t.sigma = A(1);
         t.fine0 = fine0 ? 1 : 0;
         t.has_faces = faces ? 1 : 0;
+        t.fuse0 = fine0 && !faces && !PT<SI>::scaled ? 1 : 0;
         t.fx = facesA.fx;
         t.fy = facesA.fy;
-        t.w0_const = w0c ? 1 : 0;
         t.dinv_global = lean >= 1 ? 1 : 0;
+        auto magic = [](long long d) { return (unsigned)((4294967296ULL + (unsigned long long)d - 1) / (unsigned long long)d); };
 
         long long o = 0;
         auto take = [&](long long n) {
@@ -531,56 +543,76 @@ class Precond : public PrecondBase {
             o += (n + 3) / 4 * 4;
             return (int)at;
         };
-        // Every CTA must own at least one row of every distributed level: a CTA whose coarse
-        // range is empty would interpolate from coarse ghost rows that no neighbour stores to
-        // (neighbours push only to non-empty CTAs).  Grids with few rows for their width
-        // (e.g. 120 x 17 at C = 16) fail this and take a smaller cluster or the level kernels.
-        bool nonempty = true;
         for (int l = 0; l < L; ++l) {
             const Geo& gl = lev[l].g;
-            t.g[l] = gl;
-            t.magic[l] = (unsigned)((4294967296ULL + (unsigned long long)gl.n0 - 1) / (unsigned long long)gl.n0);
-            // 16-byte vectors of points: the FD level 0 with kappa = 1 and every stored-stencil level
-            constexpr int VN = (int)(16 / sizeof(A));
-            const bool stencil_level = l >= 1 || !fine0;
-            t.vec[l] = (l < L - 1 && gl.n0 % VN == 0 && (stencil_level || !faces)) ? 1 : 0;
-            const unsigned long long nv = (unsigned long long)(gl.n0 / VN > 0 ? gl.n0 / VN : 1);
-            t.magicv[l] = (unsigned)((4294967296ULL + nv - 1) / nv);
-            if (l < T) {
-                for (int r = 0; r <= C; ++r)
-                    t.rlo[l][r] = l == 0 ? (int)((long long)r * gl.n1 / C) : t.rlo[l - 1][r] / 2;
-                int mr = 0;
+            const int nvp = std::max((gl.n0 + VN - 1) / VN, 2);
+            if (nvp > kClThreads) return false;
+            t.n0[l] = gl.n0;
+            t.n1[l] = gl.n1;
+            t.nvp[l] = nvp;
+            t.magicv[l] = magic(nvp);
+            t.magic[l] = magic(std::max(gl.n0, 2));
+            for (int r = 0; r <= C; ++r)
+                t.rlo[l][r] = l == 0 ? (int)((long long)r * gl.n1 / C) : t.rlo[l - 1][r] / 2;
+            // Every CTA must own at least one row of every distributed level (neighbours store edge rows
+            // into the CTAs that own the rows beside theirs; grids with few rows for their width fail
+            // this), and its ghost rows must belong to the kClReach CTAs on either side.
+            int mr = 1;
+            auto covered = [&](int need) {
                 for (int r = 0; r < C; ++r) {
-                    mr = std::max(mr, t.rlo[l][r + 1] - t.rlo[l][r]);
-                    nonempty = nonempty && t.rlo[l][r + 1] > t.rlo[l][r];
+                    if (std::max(t.rlo[l][r] - need, 0) < t.rlo[l][std::max(r - kClReach, 0)]) return false;
+                    const int top = r + 1 + kClReach >= C ? gl.n1 : t.rlo[l][r + 1 + kClReach];
+                    if (std::min(t.rlo[l][r + 1] + need, gl.n1) > top) return false;
                 }
-                t.maxr[l] = std::max(mr, 1);
-            } else {
-                t.maxr[l] = gl.n1;
+                return true;
+            };
+            for (int r = 0; r < C; ++r) {
+                const int own = t.rlo[l][r + 1] - t.rlo[l][r];
+                mr = std::max(mr, own);
+                if (l < T && own < 1) return false;
             }
-            t.off[l] = take(3LL * (t.maxr[l] + 2) * (gl.n0 + 2 * kClPad));
+            const int deepH = std::max(l == 0 ? nu1 + 2 : nu1 + 1, 2);
+            const bool dl = deep >= (l == 0 ? 2 : 1) && l < T && covered(deepH);
+            if (deep == 2 && l == 0 && !dl) return false;
+            t.H[l] = dl ? deepH : 1;
+            t.ix[l] = l >= T ? 0 : (l == 0 ? t.H[0] : (deep > 0 && covered(2) ? 2 : 1));
+            t.maxr[l] = l < T ? mr : gl.n1;
+            const int groups = kClThreads / nvp;
+            t.per[l] = (t.maxr[l] + 2 * t.H[l] + groups - 1) / groups;
+            const long long ld = (long long)nvp * VN + 2 * kClPad;
+            t.off[l] = take(3LL * (t.maxr[l] + 2 * t.H[l]) * ld);
+            t.ioff[l] = take(2LL * t.ix[l] * ld);
         }
-        if (!nonempty) return false;
-        for (int l = 1; l < L - 1; ++l) {
-            t.sten_global[l] = (lean >= 3 || (lean == 2 && l == 1)) ? 1 : 0;
-            if (t.sten_global[l] && !same && !t.vec[l]) return false;
-        }
+        const long long ncst = lev[T].g.nx;
+        t.ncp = (int)((ncst + VN - 1) / VN * VN);
+        t.boff = take(t.ncp);
+        // the image of constants, the program at its end
+        t.img_off = (int)o;
         for (int l = 0; l < L; ++l) {
             t.soff[l] = t.woff[l] = -1;
-            if ((l >= 1 || !fine0) && l < L - 1 && !t.sten_global[l]) t.soff[l] = take(9LL * t.maxr[l] * lev[l].g.n0);
-            if (l < L - 1 && !(l == 0 && w0c)) t.woff[l] = take((long long)t.maxr[l] * lev[l].g.n0);
+            if (l >= T) continue;
+            const long long np = (long long)t.nvp[l] * VN;
+            const bool fd = l == 0 && fine0;
+            if (!fd) {
+                t.sten_global[l] = l >= 1 && (lean >= 3 || (lean == 2 && l == 1)) ? 1 : 0;
+                if (t.sten_global[l] && lev[l].g.n0 % VN != 0) return false;     // read as whole vectors
+                if (!t.sten_global[l]) t.soff[l] = take(9LL * (t.maxr[l] + 2 * (t.H[l] - 1)) * np);
+            }
+            if (!fd || faces) t.woff[l] = take((long long)(t.maxr[l] + 2 * t.H[l]) * np);
         }
-        t.fxoff = t.fyoff = -1;
         if (faces) {
-            t.fxoff = take((long long)t.maxr[0] * (g0.n0 + 1));
-            t.fyoff = take((long long)(t.maxr[0] + 1) * g0.n0);
+            const long long np = (long long)t.nvp[0] * VN, rows = t.maxr[0] + 2 * (t.H[0] - 1);
+            t.fxoff = take(rows * (np + 2 * kClPad));
+            t.fyoff = take((rows + 1) * np);
         }
-        const long long ncst = lev[L - 1].g.nx;
         int msl = 0;
         for (int r = 0; r <= C; ++r) t.cs[r] = (int)((long long)r * ncst / C);
         for (int r = 0; r < C; ++r) msl = std::max(msl, t.cs[r + 1] - t.cs[r]);
-        t.dinv_off = t.dinv_global ? -1 : take((long long)msl * ncst);
-        t.rowtab_off = take(((long long)lev[T - 1].g.n1 * (long long)sizeof(void*) + sizeof(A) - 1) / sizeof(A));
+        t.dinv_off = t.dinv_global ? -1 : take((long long)msl * t.ncp);
+        const long long nprog = (long long)cl_program(t).size();
+        t.prog_off = (int)(o * (long long)sizeof(A));
+        take((nprog * (long long)sizeof(ClOp) + (long long)sizeof(A) - 1) / (long long)sizeof(A));
+        t.img_len = (int)(o - t.img_off);
         bytes = o * (long long)sizeof(A);
         if (bytes > dyn_max) return false;
         cudaLaunchConfig_t cfg = {};
@@ -595,60 +627,105 @@ class Precond : public PrecondBase {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int nclusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclusters, k_cluster_mg<SI>, &cfg) != cudaSuccess || nclusters < 1) {
+        if (cudaOccupancyMaxActiveClusters(&nclusters, cluster_kernel(t), &cfg) != cudaSuccess || nclusters < 1) {
             cudaGetLastError();
             return false;
         }
         return true;
     }
 
-    aao_status store_cluster_plan(ClPlan& pl, const ClCtx<SI>& t, long long bytes) {
-        ClCtx<SI> hc[kMaxS];
+    aao_status store_cluster_plan(ClPlan& pl, const ClCtx<SI>& plan, long long bytes) {
+        ClCtx<SI> t = plan;
+        const std::vector<ClOp> prog = cl_program(t);
+        ClOp* dprog;
+        AAO_TRY(ar.alloc(&dprog, prog.size()));
+        AAO_CUDA_TRY(cudaMemcpy(dprog, prog.data(), sizeof(ClOp) * prog.size(), cudaMemcpyHostToDevice));
         for (int i = 0; i < h->s; ++i) {
-            hc[i] = t;
-            hc[i].c = (A)(h->tau * h->D[i]);
+            ClCtx<SI>& q = pl.ctx[i];
+            q = t;
+            const double c = h->tau * h->D[i], hx2 = h->g.hx2, hy2 = h->g.hy2;
+            const double d0 = 1.0 + c * (2.0 * hx2 + 2.0 * hy2), w = h->opt.mg_omega / d0;
+            q.c = (A)c;
+            // omega / a_PP by the staged weights' operations
+            const A kd = A(2) * (A)hx2 + A(2) * (A)hy2;
+            q.w0 = (A)h->opt.mg_omega / std::fma((A)c, kd, A(1));
+            q.hx2 = (A)hx2;
+            q.hy2 = (A)hy2;
+            q.k0 = (A)(1.0 - h->opt.mg_omega);
+            q.kx = (A)(w * c * hx2);
+            q.ky = (A)(w * c * hy2);
+            q.d0 = (A)d0;
+            q.ex = (A)(c * hx2);
+            q.ey = (A)(c * hy2);
             for (int l = 0; l < L; ++l) {
-                hc[i].sten[l] = lev[l].sten[i];
-                hc[i].sten_sc[l] = lev[l].sten_sc[i];
+                q.sten[l] = lev[l].sten[i];
+                q.sten_sc[l] = lev[l].sten_sc[i];
+                q.W[l] = jacw[l][i];
             }
-            hc[i].Dinv = Dinv[i];
+            q.Dinv = Dinv[i];
+            const int ncst = (int)lev[L - 1].g.nx;
+            A* dpad = nullptr;
+            if (t.dinv_global && t.ncp != ncst) {
+                AAO_TRY(ar.alloc(&dpad, (size_t)ncst * t.ncp));
+                AAO_CUDA_TRY(cudaMemsetAsync(dpad, 0, sizeof(A) * (size_t)ncst * t.ncp, st()));
+                AAO_CUDA_TRY(cudaMemcpy2DAsync(dpad, sizeof(A) * t.ncp, Dinv[i], sizeof(A) * ncst, sizeof(A) * ncst, ncst,
+                                               cudaMemcpyDeviceToDevice, st()));
+            }
+            A* img;
+            AAO_TRY(ar.alloc(&img, (size_t)t.img_len * t.C));
+            AAO_CUDA_TRY(cudaMemsetAsync(img, 0, sizeof(A) * (size_t)t.img_len * t.C, st()));
+            launch(k_cluster_image<SI>, (unsigned)t.C, kBlock, 0, st(), q, img, (const ClOp*)dprog, (int)prog.size());
+            AAO_LAUNCH_CHECK();
+            q.img = img;
+            if (dpad) q.Dinv = dpad;
         }
-        AAO_TRY(ar.alloc(&pl.ctx, (size_t)h->s));
-        AAO_CUDA_TRY(cudaMemcpy(pl.ctx, hc, sizeof(ClCtx<SI>) * h->s, cudaMemcpyHostToDevice));
         pl.C = t.C;
         pl.smem = (size_t)bytes;
+        pl.kernel = cluster_kernel(t);
         return AAO_OK;
     }
 
     aao_status build_cluster(int optin) {
         cl_C = 0;
-        clp[0] = clp[1] = ClPlan{};
+        clp[0].C = clp[1].C = 0;
         const Geo& g0 = h->g;
         if (g0.d != 2 || L < 2) return AAO_OK;
-        cudaFuncAttributes fa;
-        AAO_CUDA_TRY(cudaFuncGetAttributes(&fa, k_cluster_mg<SI>));
-        const long long dyn_max = (long long)optin - (long long)fa.sharedSizeBytes;
-        if (dyn_max <= 0) return AAO_OK;
-        AAO_CUDA_TRY(cudaFuncSetAttribute(k_cluster_mg<SI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_max));
-        AAO_CUDA_TRY(cudaFuncSetAttribute(k_cluster_mg<SI>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        long long dyn_max = optin;
+        for (ClKernel k : {(ClKernel)k_cluster_mg<SI, false, false>, (ClKernel)k_cluster_mg<SI, false, true>,
+                           (ClKernel)k_cluster_mg<SI, true, false>, (ClKernel)k_cluster_mg<SI, true, true>}) {
+            cudaFuncAttributes fa;
+            AAO_CUDA_TRY(cudaFuncGetAttributes(&fa, (const void*)k));
+            dyn_max = std::min(dyn_max, (long long)optin - (long long)fa.sharedSizeBytes);
+            if (dyn_max <= 0) return AAO_OK;
+            AAO_CUDA_TRY(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              optin - (int)fa.sharedSizeBytes));
+            AAO_CUDA_TRY(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        }
         ClCtx<SI> t;
         long long bytes = 0;
-        // single items: the full layout first (staged once per launch), 16 CTAs before 8
-        bool found = false;
-        for (int C : {16, 8}) {
-            for (int lean = 0; lean <= 3 && !found; ++lean) found = plan_cluster(C, lean, dyn_max, t, bytes);
-            if (found) break;
+        // FP64 arithmetic is too slow for redundant rows; else the deepest ghost regions that fit, before
+        // staging less
+        const int deepest = std::is_same<A, double>::value ? 0 : 2;
+        auto find = [&](int C) {
+            for (int lo = 0; lo <= 2; lo += 2)          // lean 0 and 1 for every depth, then 2 and 3
+                for (int deep = deepest; deep >= 0; --deep)
+                    for (int lean = lo; lean <= lo + 1; ++lean)
+                        if (plan_cluster(C, deep, lean, dyn_max, t, bytes)) return true;
+            return false;
+        };
+        if (!find(16) && !find(8)) return AAO_OK;
+        for (int l = 0; l < L - 1; ++l) {
+            if (l == 0 && !h->q1 && !h->has_kappa) continue;     // the scalar weight
+            for (int i = 0; i < h->s; ++i) {
+                AAO_TRY(ar.alloc(&jacw[l][i], (size_t)lev[l].g.nx));
+                launch(k_jacobi_weights<SI>, (unsigned)((lev[l].g.nx + kBlock - 1) / kBlock), kBlock, 0, st(),
+                       level_op(l, i), (A)h->opt.mg_omega, jacw[l][i]);
+            }
         }
-        if (!found) return AAO_OK;
+        AAO_LAUNCH_CHECK();
         AAO_TRY(store_cluster_plan(clp[0], t, bytes));
-        // batches: 8 CTAs per item, the leanest layout that fits
-        if (clp[0].C == 8) {
-            clp[1] = clp[0];
-        } else {
-            bool fb = false;
-            for (int lean = 0; lean <= 3 && !fb; ++lean) fb = plan_cluster(8, lean, dyn_max, t, bytes);
-            if (fb) AAO_TRY(store_cluster_plan(clp[1], t, bytes));
-        }
+        if (clp[0].C == 8) clp[1] = clp[0];
+        else if (find(8)) AAO_TRY(store_cluster_plan(clp[1], t, bytes));
         cl_C = clp[0].C;
         return AAO_OK;
     }
@@ -923,8 +1000,8 @@ class Precond : public PrecondBase {
             // one cluster per item: small batches (single time steps, MGRIT's batched steps)
             const ClPlan& pl = B >= kClBatch8 && clp[1].C > 0 ? clp[1] : clp[0];
             bytes_hint(2.0 * nact * h->g.nx * sizeof(SI));
-            launch_cluster(k_cluster_mg<SI>, dim3((unsigned)(pl.C * B)), dim3(kClThreads), pl.smem, st(), pl.C,
-                           (const ClCtx<SI>*)(pl.ctx + stage), act, b, out);
+            launch_cluster(pl.kernel, dim3((unsigned)(pl.C * B)), dim3(kClThreads), pl.smem, st(), pl.C,
+                           pl.ctx[stage], act, b, out);
             AAO_LAUNCH_CHECK();
             return AAO_OK;
         }
