@@ -452,8 +452,7 @@ static aao_status matvec_dev(Handle* h, const double* x, double* y, const double
         return AAO_OK;
     }
     bytes_hint(8.0 * h->nst * (rhs ? 3 : 2));
-    launch(k_matvec, blocks_for_rows((long long)(h->nt + 1) * g.R), kBlock, 0, h->stream, 
-        g, h->nt, h->tab, h->tau, h->faces64, x, y, rhs, transpose, (const int*)nullptr);
+    launch_matvec(g, h->nt, h->tab, h->tau, h->faces64, x, y, rhs, transpose, (const int*)nullptr, h->stream);
     AAO_LAUNCH_CHECK();
     return AAO_OK;
 }
@@ -474,8 +473,7 @@ static aao_status matvec_relaxed(Handle* h, const double* z, double* y, int k, i
            h->opt.relax_matvec, h->opt.tol, h->m, (const double*)(h->beta + 1), (const double*)(h->gv + k),
            h->relax_flag);
     bytes_hint(8.0 * h->nst * 2);
-    launch(k_matvec, nblk, kBlock, 0, h->stream, g, h->nt, h->tab, h->tau, h->faces64, z, y, (const double*)nullptr,
-           transpose, (const int*)h->relax_flag);
+    launch_matvec(g, h->nt, h->tab, h->tau, h->faces64, z, y, nullptr, transpose, (const int*)h->relax_flag, h->stream);
     AAO_LAUNCH_CHECK();
     return AAO_OK;
 }
