@@ -587,6 +587,33 @@ __global__ void __launch_bounds__(kArThreads) k_rana_vec(Geo g, InvH2<typename P
     st_n<N>(out.d + (long long)b * out.bs + (long long)row * g.n0 + c, acc);
 }
 
+// The same in 16-bit storage: a thread per point of whole rows (the row's scale is a block reduction).
+template <class SV, class SZ>
+__global__ void __launch_bounds__(kPtMaxThreads) k_rana_pt(Geo g, InvH2<typename PT<SZ>::A> hh, PtMap pm, int B,
+                                                           const int* active, Vec<SV> V, long long rows, int stage,
+                                                           Vec<SZ> Z, StageCoef<typename PT<SZ>::A> cf,
+                                                           Faces<typename PT<SZ>::A> faces, Vec<SZ> out) {
+    pdl_prologue();
+    using A = typename PT<SZ>::A;
+    PtPos q = pt_pos(pm, B, g.R, active);
+    const int row = (int)q.row;
+    int j = 0, k = 0;
+    if (q.valid) row_jk(g, row, j, k);
+    SZ* o; float* osc;
+    row_store_ptrs(out, q.b, 0, q.row, g.n0, o, osc);
+    pt_store<SZ>(o, osc, pm, q.c0, q.valid, [&](int c) -> A {
+        A acc;
+        field_of(V, q.b, rows, stage, g).template row_n<1>(row, c, &acc);
+#pragma unroll 2
+        for (int jj = cf.j0; jj < cf.j1; ++jj) {
+            A P, K;
+            fd_K_n<1>(field_of(Z, q.b, rows, jj, g), g, hh, faces, row, j, k, c, &P, &K);
+            acc -= cf.c[jj] * K;
+        }
+        return acc;
+    });
+}
+
 // ---------------------------------------------------------------------------
 // S_tilde's recurrence (one item, or B of MGRIT's intervals: item b at time index sp->n + b * stride).
 // Its states are FP64 vectors that hold values of the arithmetic type A.

@@ -24,6 +24,7 @@ template <class S> struct LevelOp {
     const S* sten = nullptr; // coarse: ncoef*nx, component-major
     const float* sten_sc = nullptr;  // coarse, scaled types: one scale per component
     int ncoef = 9;
+    A hx2 = A(0), hy2 = A(0), hz2 = A(0);   // 1 / h^2 of g in the arithmetic type (matrix-free 3D tiles)
 };
 
 template <class S>
@@ -272,6 +273,32 @@ __device__ __forceinline__ void level_apply_k(const LevelOp<S>& op, const View<S
         }
         Au = acc;
         diag = sten_coef(op, 4, p);
+    } else if constexpr (KIND == 3) {
+        // stored 27-point stencil: every load is issued before the sum (a point outside the grid adds an exact
+        // zero where level_apply skips it)
+        const unsigned nx = (unsigned)g.nx, p = (unsigned)row * g.n0 + c;
+        const bool xm = c > 0, xp = c + 1 < g.n0;
+        A v[27];
+#pragma unroll
+        for (int r = 0; r < 9; ++r) {
+            const int dy = r % 3 - 1, dz = r / 3 - 1;
+            const bool in = j + dy >= 0 && j + dy < g.n1 && k + dz >= 0 && k + dz < g.n2;
+            const int rr = (int)row + dy + dz * g.n1;
+            v[3 * r] = in && xm ? A(u.at(rr, c - 1)) : A(0);
+            v[3 * r + 1] = in ? A(u.at(rr, c)) : A(0);
+            v[3 * r + 2] = in && xp ? A(u.at(rr, c + 1)) : A(0);
+        }
+        A s[27];
+#pragma unroll
+        for (int q = 0; q < 27; ++q) {
+            s[q] = PT<S>::ld(op.sten[q * nx + p]);
+            if constexpr (PT<S>::scaled) s[q] *= op.sten_sc[q];
+        }
+        A acc = A(0);
+#pragma unroll
+        for (int q = 0; q < 27; ++q) acc += s[q] * v[q];
+        Au = acc;
+        diag = s[13];
     } else {
         level_apply(op, u, row, j, k, c, Au, diag);
     }
@@ -282,6 +309,7 @@ __device__ __forceinline__ typename PT<S>::A level_diag_k(const LevelOp<S>& op, 
     using A = typename PT<S>::A;
     if constexpr (KIND == 1 || KIND == 4) return op.sigma + op.c * fd_K_diag<A>(op.g, op.faces, row, j, k, c);
     else if constexpr (KIND == 2) return sten_coef(op, 4, row * op.g.n0 + c);
+    else if constexpr (KIND == 3) return sten_coef(op, 13, row * op.g.n0 + c);
     else return level_diag(op, row, j, k, c);
 }
 
@@ -834,6 +862,31 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_restrict(Geo gf, Geo gc, PtMa
     View<S> rr = view_of(rv, q.b, 0, gf.n0);
     S* out; float* osc;
     row_store_ptrs(bcv, q.b, 0, row, gc.n0, out, osc);
+    if (gf.d == 3) {
+        // every load before the sum (rows and columns beyond the grid add exact zeros)
+        pt_store<S>(out, osc, pm, q.c0, q.valid, [&](int I) -> A {
+            const bool xp = 2 * I + 2 < gf.n0;
+            A v[27];
+#pragma unroll
+            for (int r = 0; r < 9; ++r) {
+                const int fj = 2 * J + r % 3, fk = 2 * Kc + r / 3;
+                const bool in = fj < gf.n1 && fk < gf.n2;
+                const int frow = fj + gf.n1 * fk;
+                v[3 * r] = in ? rr.at(frow, 2 * I) : A(0);
+                v[3 * r + 1] = in ? rr.at(frow, 2 * I + 1) : A(0);
+                v[3 * r + 2] = in && xp ? rr.at(frow, 2 * I + 2) : A(0);
+            }
+            A acc = A(0);
+#pragma unroll
+            for (int e = 0; e < 27; ++e) {
+                const A wx = e % 3 == 1 ? A(1) : A(0.5), wy = e / 3 % 3 == 1 ? A(1) : A(0.5),
+                        wz = e / 9 == 1 ? A(1) : A(0.5);
+                acc += wx * wy * wz * v[e];
+            }
+            return acc;
+        });
+        return;
+    }
     pt_store<S>(out, osc, pm, q.c0, q.valid, [&](int I) -> A {
         A acc = A(0);
         const int zlo = gf.d == 3 ? -1 : 0, zhi = gf.d == 3 ? 1 : 0;
@@ -896,6 +949,32 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_prolong_add(Geo gf, Geo gc, P
     int mz = gf.d == 3 ? interp_1d(k, gc.n2, Jz, wz) : 1;
     S* out; float* osc;
     row_store_ptrs(xout, q.b, 0, row, gf.n0, out, osc);
+    if (gf.d == 3) {
+        // up to eight coarse points, every load before the sum (a missing one adds an exact zero)
+        pt_store<S>(out, osc, pm, q.c0, q.valid, [&](int c) -> A {
+            int Jx[2] = {0, 0};
+            float wx[2] = {0.f, 0.f};
+            const int mx = interp_1d(c, gc.n0, Jx, wx);
+            const A base = has_in ? xi.at(row, c) : A(0);
+            A v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int x = e & 1, y = e >> 1 & 1, z = e >> 2;
+                const bool in = x < mx && y < my && z < mz;
+                v[e] = in ? xc.at(Jy[y] + gc.n1 * Jz[z], Jx[x]) : A(0);
+            }
+            A acc = base;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int x = e & 1, y = e >> 1 & 1, z = e >> 2;
+                const bool in = x < mx && y < my && z < mz;
+                const A w = in ? A(wy[y]) * A(wz[z]) * A(wx[x]) : A(0);
+                acc += w * v[e];
+            }
+            return acc;
+        });
+        return;
+    }
     pt_store<S>(out, osc, pm, q.c0, q.valid, [&](int c) -> A {
         int Jx[2];
         float wx[2];
@@ -1000,27 +1079,286 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_prolong_smooth(LevelOp<S> op,
     });
 }
 
-// x = Dinv b at the coarsest level (Dinv dense, nc x nc, row-major, arithmetic type).
+// ---------------------------------------------------------------------------
+// The finest 3D level's fused steps (two sweeps; residual and restriction; interpolation and sweep), a tile of
+// whole grid rows per CTA: the inner step's values are formed once in shared memory instead of being
+// recomputed at every neighbour (seven times the arithmetic and 49 loads per point).  Same operations per
+// point as k_smooth2, k_resid_restrict and k_prolong_smooth.  Tiles of 4 x 4 rows (2 x 2 coarse rows): a
+// 47 x 39 x 43 grid gives 110 CTAs; a warp per row, so a row's storage scale is a warp reduction.
+// ---------------------------------------------------------------------------
+constexpr int kT3Threads = 256;
+constexpr int kT3Warps = kT3Threads / kWarp;
+constexpr int kT3 = 4;                       // output rows per axis
+inline size_t t3_smem_smooth2(int n0, size_t a) { return (size_t)((kT3 + 4) * (kT3 + 4) + (kT3 + 2) * (kT3 + 2)) * n0 * a; }
+inline size_t t3_smem_restrict(int n0, size_t a) { return (size_t)((kT3 + 3) * (kT3 + 3) + (kT3 + 1) * (kT3 + 1)) * n0 * a; }
+inline size_t t3_smem_prolong(int n0, size_t a) { return (size_t)(kT3 + 2) * (kT3 + 2) * n0 * a; }
+inline dim3 t3_grid(int n1, int n2, int tile, int B) {
+    return dim3((unsigned)((n1 + tile - 1) / tile), (unsigned)((n2 + tile - 1) / tile), (unsigned)B);
+}
+
+// Rows of a tile region in shared memory: w rows per axis, the first one (j0, k0), n0 columns.
+template <class A> struct T3Rows {
+    const A* d;
+    int w, j0, k0, n0;
+    __device__ __forceinline__ A operator()(int j, int k, int c) const { return d[((k - k0) * w + j - j0) * n0 + c]; }
+};
+
+// (A u)_P and a_PP of the matrix-free 3D level from u(j, k, c) in shared memory.
+template <class S, class A>
+__device__ __forceinline__ void t3_apply(const LevelOp<S>& op, const T3Rows<A>& u, int j, int k, int c, A& Au, A& diag) {
+    const Geo& g = op.g;
+    const A uP = u(j, k, c);
+    const A uW = c > 0 ? u(j, k, c - 1) : A(0), uE = c + 1 < g.n0 ? u(j, k, c + 1) : A(0);
+    const A uS = j > 0 ? u(j - 1, k, c) : A(0), uN = j + 1 < g.n1 ? u(j + 1, k, c) : A(0);
+    const A uD = k > 0 ? u(j, k - 1, c) : A(0), uU = k + 1 < g.n2 ? u(j, k + 1, c) : A(0);
+    const Faces<A>& f = op.faces;
+    A Ku, kd;
+    if (f.fx == nullptr) {
+        Ku = op.hx2 * (A(2) * uP - uW - uE) + op.hy2 * (A(2) * uP - uS - uN);
+        Ku += op.hz2 * (A(2) * uP - uD - uU);
+        kd = A(2) * op.hx2 + A(2) * op.hy2;
+        kd += A(2) * op.hz2;
+    } else {
+        const int row = j + g.n1 * k, fxi = row * (g.n0 + 1) + c, fyi = (k * (g.n1 + 1) + j) * g.n0 + c;
+        const int fzi = row * g.n0 + c, pl = g.n1 * g.n0;
+        const A x0 = f.fx[fxi], x1 = f.fx[fxi + 1], y0 = f.fy[fyi], y1 = f.fy[fyi + g.n0], z0 = f.fz[fzi], z1 = f.fz[fzi + pl];
+        Ku = x0 * (uP - uW) + x1 * (uP - uE) + y0 * (uP - uS) + y1 * (uP - uN);
+        Ku += z0 * (uP - uD) + z1 * (uP - uU);
+        kd = x0 + x1 + y0 + y1;
+        kd += z0 + z1;
+    }
+    Au = op.sigma * uP + op.c * Ku;
+    diag = op.sigma + op.c * kd;
+}
+
+// Load the rows [j0, j0 + w) x [k0, k0 + w) of v that lie inside the grid.
+template <class S, class A>
+__device__ __forceinline__ void t3_load(const Geo& g, const View<S>& v, int w, int j0, int k0, A* dst) {
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int r = wp; r < w * w; r += kT3Warps) {
+        const int j = j0 + r % w, k = k0 + r / w;
+        if (j < 0 || j >= g.n1 || k < 0 || k >= g.n2) continue;
+#pragma unroll 2
+        for (int c = lane; c < g.n0; c += kWarp) dst[r * g.n0 + c] = v.at(j + g.n1 * k, c);
+    }
+}
+
 template <class S>
-__global__ void __launch_bounds__(kPtMaxThreads) k_coarse_solve(Geo g, PtMap pm, int B, const int* active,
-                                                       const typename PT<S>::A* Dinv, Vec<S> bv, Vec<S> xv) {
+__global__ void __launch_bounds__(kT3Threads) k_smooth2_tile(LevelOp<S> op, const int* active, Vec<S> xin, Vec<S> bv,
+                                                             Vec<S> xout, typename PT<S>::A omega) {
     pdl_prologue();
     using A = typename PT<S>::A;
-    PtPos q = pt_pos(pm, B, g.R, active);
-    if constexpr (!PT<S>::scaled) {
-        if (!q.valid) return;
+    extern __shared__ __align__(16) unsigned char t3_smem[];
+    const Geo& g = op.g;
+    const int b = blockIdx.z;
+    if (active && !active[b]) return;
+    const int j0 = blockIdx.x * kT3, k0 = blockIdx.y * kT3, n0 = g.n0;
+    constexpr int W0 = kT3 + 4, W1 = kT3 + 2;
+    A* x0 = reinterpret_cast<A*>(t3_smem);
+    A* x1 = x0 + W0 * W0 * n0;
+    View<S> bb = view_of(bv, b, 0, n0);
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool has = xin.d != nullptr;
+    if (has) t3_load(g, view_of(xin, b, 0, n0), W0, j0 - 2, k0 - 2, x0);
+    __syncthreads();
+    const T3Rows<A> u0{x0, W0, j0 - 2, k0 - 2, n0};
+    for (int r = wp; r < W1 * W1; r += kT3Warps) {
+        const int j = j0 - 1 + r % W1, k = k0 - 1 + r / W1;
+        if (j < 0 || j >= g.n1 || k < 0 || k >= g.n2) continue;
+        for (int c = lane; c < n0; c += kWarp) {
+            const A bp = bb.at(j + g.n1 * k, c);
+            if (has) {
+                A Au, dg;
+                t3_apply(op, u0, j, k, c, Au, dg);
+                x1[r * n0 + c] = u0(j, k, c) + omega * (bp - Au) / dg;
+            } else {
+                x1[r * n0 + c] = omega * bp / level_diag(op, j + g.n1 * k, j, k, c);
+            }
+        }
     }
-    const long long row = q.row;
-    View<S> bb = view_of(bv, q.b, 0, g.n0);
-    S* out; float* osc;
-    row_store_ptrs(xv, q.b, 0, row, g.n0, out, osc);
-    const int nc = (int)g.nx;
-    pt_store<S>(out, osc, pm, q.c0, q.valid, [&](int c) -> A {
-        long long p = row * g.n0 + c;
+    __syncthreads();
+    const T3Rows<A> u1{x1, W1, j0 - 1, k0 - 1, n0};
+    for (int r = wp; r < kT3 * kT3; r += kT3Warps) {
+        const int j = j0 + r % kT3, k = k0 + r / kT3;
+        if (j >= g.n1 || k >= g.n2) continue;
+        A* x2 = x0 + r * n0;                      // x_in is not read again
+        for (int c = lane; c < n0; c += kWarp) {
+            A Au, dg;
+            t3_apply(op, u1, j, k, c, Au, dg);
+            x2[c] = u1(j, k, c) + omega * (bb.at(j + g.n1 * k, c) - Au) / dg;
+        }
+        S* out; float* osc;
+        row_store_ptrs(xout, b, 0, j + g.n1 * k, n0, out, osc);
+        row_store<S>(out, osc, n0, lane, [&](int c) -> A { return x2[c]; });
+    }
+}
+
+template <class S>
+__global__ void __launch_bounds__(kT3Threads) k_resid_restrict_tile(LevelOp<S> op, Geo gc, const int* active, Vec<S> xv,
+                                                                    Vec<S> bv, Vec<S> bcv) {
+    pdl_prologue();
+    using A = typename PT<S>::A;
+    extern __shared__ __align__(16) unsigned char t3_smem[];
+    const Geo& g = op.g;
+    const int b = blockIdx.z;
+    if (active && !active[b]) return;
+    constexpr int CT = kT3 / 2, WR = kT3 + 1, WX = kT3 + 3;     // coarse rows; fine rows 2J .. 2J + 2; one more around
+    const int J0 = blockIdx.x * CT, K0 = blockIdx.y * CT, j0 = 2 * J0, k0 = 2 * K0, n0 = g.n0;
+    A* x0 = reinterpret_cast<A*>(t3_smem);
+    A* rs = x0 + WX * WX * n0;
+    View<S> bb = view_of(bv, b, 0, n0);
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool has = xv.d != nullptr;
+    if (has) t3_load(g, view_of(xv, b, 0, n0), WX, j0 - 1, k0 - 1, x0);
+    __syncthreads();
+    const T3Rows<A> u{x0, WX, j0 - 1, k0 - 1, n0};
+    for (int r = wp; r < WR * WR; r += kT3Warps) {
+        const int j = j0 + r % WR, k = k0 + r / WR;
+        const bool in = j < g.n1 && k < g.n2;
+        for (int c = lane; c < n0; c += kWarp) {
+            A res = A(0);
+            if (in) {
+                res = bb.at(j + g.n1 * k, c);
+                if (has) {
+                    A Au, dg;
+                    t3_apply(op, u, j, k, c, Au, dg);
+                    res -= Au;
+                }
+            }
+            rs[r * n0 + c] = res;
+        }
+    }
+    __syncthreads();
+    for (int r = wp; r < CT * CT; r += kT3Warps) {
+        const int J = J0 + r % CT, K = K0 + r / CT;
+        if (J >= gc.n1 || K >= gc.n2) continue;
+        const A* base = rs + ((2 * (r / CT)) * WR + 2 * (r % CT)) * n0;
+        A* bc = x0 + r * n0;
+        for (int I = lane; I < gc.n0; I += kWarp) {
+            const bool xp = 2 * I + 2 < n0;
+            A acc = A(0);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                const A wy = e % 3 == 1 ? A(1) : A(0.5), wz = e / 3 == 1 ? A(1) : A(0.5);
+                const A* row = base + ((e / 3) * WR + e % 3) * n0 + 2 * I;
+                acc += A(0.5) * wy * wz * row[0];
+                acc += wy * wz * row[1];
+                acc += A(0.5) * wy * wz * (xp ? row[2] : A(0));
+            }
+            bc[I] = acc;
+        }
+        S* out; float* osc;
+        row_store_ptrs(bcv, b, 0, J + gc.n1 * K, gc.n0, out, osc);
+        row_store<S>(out, osc, gc.n0, lane, [&](int c) -> A { return bc[c]; });
+    }
+}
+
+template <class S>
+__global__ void __launch_bounds__(kT3Threads) k_prolong_smooth_tile(LevelOp<S> op, Geo gc, const int* active, Vec<S> xcv,
+                                                                    Vec<S> xin, Vec<S> bv, Vec<S> xout,
+                                                                    typename PT<S>::A omega) {
+    pdl_prologue();
+    using A = typename PT<S>::A;
+    extern __shared__ __align__(16) unsigned char t3_smem[];
+    const Geo& g = op.g;
+    const int b = blockIdx.z;
+    if (active && !active[b]) return;
+    const int j0 = blockIdx.x * kT3, k0 = blockIdx.y * kT3, n0 = g.n0;
+    constexpr int W1 = kT3 + 2;
+    A* xp = reinterpret_cast<A*>(t3_smem);
+    View<S> bb = view_of(bv, b, 0, n0), xc = view_of(xcv, b, 0, gc.n0);
+    const bool has = xin.d != nullptr;
+    View<S> xi = has ? view_of(xin, b, 0, n0) : View<S>{nullptr, nullptr, n0};
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int r = wp; r < W1 * W1; r += kT3Warps) {
+        const int j = j0 - 1 + r % W1, k = k0 - 1 + r / W1;
+        if (j < 0 || j >= g.n1 || k < 0 || k >= g.n2) continue;
+        int Jy[2] = {0, 0}, Jz[2] = {0, 0};
+        float wy[2] = {0.f, 0.f}, wz[2] = {0.f, 0.f};
+        const int my = interp_1d(j, gc.n1, Jy, wy), mz = interp_1d(k, gc.n2, Jz, wz);
+        for (int c = lane; c < n0; c += kWarp) {
+            int Jx[2] = {0, 0};
+            float wx[2] = {0.f, 0.f};
+            const int mx = interp_1d(c, gc.n0, Jx, wx);
+            A acc = has ? xi.at(j + g.n1 * k, c) : A(0);
+            A v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int x = e & 1, y = e >> 1 & 1, z = e >> 2;
+                v[e] = x < mx && y < my && z < mz ? xc.at(Jy[y] + gc.n1 * Jz[z], Jx[x]) : A(0);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int x = e & 1, y = e >> 1 & 1, z = e >> 2;
+                const A w = x < mx && y < my && z < mz ? A(wy[y]) * A(wz[z]) * A(wx[x]) : A(0);
+                acc += w * v[e];
+            }
+            xp[r * n0 + c] = acc;
+        }
+    }
+    __syncthreads();
+    const T3Rows<A> u{xp, W1, j0 - 1, k0 - 1, n0};
+    A val[(kMaxRowLen + kWarp - 1) / kWarp > 4 ? 4 : 4];
+    for (int r = wp; r < kT3 * kT3; r += kT3Warps) {
+        const int j = j0 + r % kT3, k = k0 + r / kT3;
+        const bool in = j < g.n1 && k < g.n2;
+        // columns lane, lane + 32, ... (at most four: t3_ok)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = lane + kWarp * q;
+            val[q] = A(0);
+            if (in && c < n0) {
+                A Au, dg;
+                t3_apply(op, u, j, k, c, Au, dg);
+                val[q] = u(j, k, c) + omega * (bb.at(j + g.n1 * k, c) - Au) / dg;
+            }
+        }
+        if (!in) continue;
+        S* out; float* osc;
+        row_store_ptrs(xout, b, 0, j + g.n1 * k, n0, out, osc);
+        row_store<S>(out, osc, n0, lane, [&](int c) -> A {
+            const int q = c / kWarp;
+            return q == 0 ? val[0] : (q == 1 ? val[1] : (q == 2 ? val[2] : val[3]));
+        });
+    }
+}
+
+// Whether the finest level's fused steps take the tiles: 3D matrix-free, rows of at most 128 points whose tiles
+// fit the default 48 KB of shared memory.
+template <class S> inline bool t3_ok(const LevelOp<S>& op) {
+    return op.fine && op.g.d == 3 && op.g.n0 <= 128 &&
+           t3_smem_smooth2(op.g.n0, sizeof(typename PT<S>::A)) <= 48 * 1024;
+}
+
+// x = Dinv b at the coarsest level (Dinv dense, nc x nc, row-major, arithmetic type): a block per grid
+// row, a warp per point of it, b in shared memory.  (One thread per point read its row of Dinv alone:
+// nc dependent uncoalesced loads.)
+constexpr int kCoarseThreads = 256;
+template <class S>
+__global__ void __launch_bounds__(kCoarseThreads) k_coarse_solve(Geo g, int B, const int* active,
+                                                                 const typename PT<S>::A* Dinv, Vec<S> bv, Vec<S> xv) {
+    pdl_prologue();
+    using A = typename PT<S>::A;
+    __shared__ A bs[kMaxCoarsest], xs[kMaxCoarsest];
+    const int b = blockIdx.y, row = blockIdx.x, nc = (int)g.nx;
+    if (b >= B || (active && !active[b])) return;
+    View<S> bb = view_of(bv, b, 0, g.n0);
+    for (int q = threadIdx.x; q < nc; q += kCoarseThreads) bs[q] = bb.at(q / g.n0, q % g.n0);
+    __syncthreads();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int c = w; c < g.n0; c += kCoarseThreads / kWarp) {
+        const A* D = Dinv + (long long)(row * g.n0 + c) * nc;
         A acc = A(0);
-        for (int qq = 0; qq < nc; ++qq) acc += Dinv[p * nc + qq] * bb.at(qq / g.n0, qq % g.n0);
-        return acc;
-    });
+#pragma unroll 8
+        for (int q = lane; q < nc; q += kWarp) acc += D[q] * bs[q];
+        acc = warp_sum(acc);
+        if (lane == 0) xs[c] = acc;
+    }
+    __syncthreads();
+    if (w != 0) return;
+    S* out; float* osc;
+    row_store_ptrs(xv, b, 0, row, g.n0, out, osc);
+    row_store<S>(out, osc, g.n0, lane, [&](int c) -> A { return xs[c]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -1365,7 +1703,8 @@ __device__ __forceinline__ void tail_smooth(const TailCtx<SI>& t, int l, typenam
                 Xn[p] = t.omega * Bv[p] / level_diag(op, row, j, k, c);
             } else {
                 A Au, dg;
-                level_apply(op, xv, row, j, k, c, Au, dg);
+                if (op.fine) level_apply(op, xv, row, j, k, c, Au, dg);
+                else level_apply_k<3>(op, xv, row, j, k, c, Au, dg);
                 Xn[p] = Xc[p] + t.omega * (Bv[p] - Au) / dg;
             }
         }
@@ -1434,7 +1773,8 @@ __global__ void __launch_bounds__(1024) k_vcycle_tail(TailCtx<SI> t, int B, cons
                 int j, k;
     row_jk(gf, row, j, k);
                 A Au, dg;
-                level_apply(op, xv, row, j, k, c, Au, dg);
+                if (op.fine) level_apply(op, xv, row, j, k, c, Au, dg);
+                else level_apply_k<3>(op, xv, row, j, k, c, Au, dg);
                 Rf[p] = Bv[p] - Au;
             }
         }

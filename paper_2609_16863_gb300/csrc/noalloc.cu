@@ -220,7 +220,7 @@ extern "C" aao_status aao_rk_shifted_solve_noalloc(const aao_grid* grid, double 
             const Geo& gl = lev[l];
             const PtMap pm = ptmap(gl.n0);
             if (l == L - 1) {
-                launch(k_coarse_solve<double>, pt_grid(pm, gl.R, 1), pt_block(pm), 0, st, gl, pm, 1, (const int*)nullptr, dinv,
+                launch(k_coarse_solve<double>, dim3((unsigned)gl.R), kCoarseThreads, 0, st, gl, 1, (const int*)nullptr, dinv,
                        bvec, xout);
                 AAO_LAUNCH_CHECK();
                 return AAO_OK;

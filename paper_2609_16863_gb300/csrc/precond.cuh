@@ -788,6 +788,9 @@ class Precond : public PrecondBase {
         LevelOp<SI> op;
         op.g = lev[l].g;
         op.ncoef = op.g.d == 3 ? 27 : 9;
+        op.hx2 = (A)op.g.hx2;
+        op.hy2 = (A)op.g.hy2;
+        op.hz2 = (A)op.g.hz2;
         if (l == 0 && !h->q1) {
             op.fine = 1;
             op.sigma = A(1);
@@ -847,6 +850,7 @@ class Precond : public PrecondBase {
         }
         if (kind == 4) launch(k_smooth<SI, 4>, grid, block, 0, st(), args...);
         else if (kind == 2) launch(k_smooth<SI, 2>, grid, block, 0, st(), args...);
+        else if (kind == 3) launch(k_smooth<SI, 3>, grid, block, 0, st(), args...);
         else launch(k_smooth<SI, 0>, grid, block, 0, st(), args...);
     }
     void launch_residual(int kind, dim3 grid, dim3 block, const LevelOp<SI>& op, const PtMap& pm, int B,
@@ -883,6 +887,7 @@ class Precond : public PrecondBase {
         }
         if (kind == 4) launch(k_residual<SI, 4>, grid, block, 0, st(), args...);
         else if (kind == 2) launch(k_residual<SI, 2>, grid, block, 0, st(), args...);
+        else if (kind == 3) launch(k_residual<SI, 3>, grid, block, 0, st(), args...);
         else launch(k_residual<SI, 0>, grid, block, 0, st(), args...);
     }
 
@@ -892,7 +897,8 @@ class Precond : public PrecondBase {
         const PtMap pm = ptmap(g.n0);
         const dim3 pbl = pt_grid(pm, g.R, B), pth = pt_block(pm);
         const Tail& T = tails[B > 1 ? 1 : 0];
-        if (l == T.lc) {
+        // (a tail that is the coarsest level alone: its rows on as many SMs instead of one)
+        if (l == T.lc && l < L - 1) {
             bytes_hint((xin.d ? 3.0 : 2.0) * nact * g.nx * sizeof(SI));
             if (g.d == 2)
                 launch(k_vcycle_tail_2d<SI>, (unsigned)B, dim3(32, 32), T.smem, st(), T.ctx[stage], B, act, b, xin,
@@ -904,8 +910,8 @@ class Precond : public PrecondBase {
         }
         if (l == L - 1) {
             bytes_hint(2.0 * nact * g.nx * sizeof(SI));
-            launch(k_coarse_solve<SI>, pt_grid(pm, g.R, B), pt_block(pm), 0, st(), g, pm, B, act, Dinv[stage], b,
-                   xout);
+            launch(k_coarse_solve<SI>, dim3((unsigned)g.R, (unsigned)B), kCoarseThreads, 0, st(), g, B, act,
+                   (const A*)Dinv[stage], b, xout);
             AAO_LAUNCH_CHECK();
             return AAO_OK;
         }
@@ -924,6 +930,7 @@ class Precond : public PrecondBase {
         // than the fused kernels' recomputation)
         const bool fuse = (long long)B * g.nx <= kFuseMaxPoints && (g.d == 2 || op.fine) && !vec16_ok(op);
         const bool f2 = fuse && nu1 >= 2, fps = fuse && nu2 >= 1;
+        const bool tiles = t3_ok(op) && B <= 65535;
         const int pre_l = f2 ? nu1 - 1 : nu1;
         const int post_l = fps ? nu2 : nu2 + 1;
         const int nops = pre_l + post_l;
@@ -938,7 +945,10 @@ class Precond : public PrecondBase {
         if (f2) {
             Vec<SI> d = dest();
             bytes_hint((cur.d ? 3.0 : 2.0) * nact * g.nx * sizeof(SI));
-            launch(k_smooth2<SI>, pbl, pth, 0, st(), op, pm, B, act, cur, b, d, om);
+            if (tiles)
+                launch(k_smooth2_tile<SI>, t3_grid(g.n1, g.n2, kT3, B), kT3Threads, t3_smem_smooth2(g.n0, sizeof(A)), st(),
+                       op, act, cur, b, d, om);
+            else launch(k_smooth2<SI>, pbl, pth, 0, st(), op, pm, B, act, cur, b, d, om);
             cur = d;
             q = 2;
         }
@@ -951,7 +961,10 @@ class Precond : public PrecondBase {
         // residual and restriction
         if (fuse) {
             bytes_hint(((cur.d ? 2.0 : 1.0) * g.nx + gc.nx) * nact * sizeof(SI));
-            launch(k_resid_restrict<SI>, cbl, cth, 0, st(), op, gc, pmc, B, act, cur, b, lev[l + 1].Bb);
+            if (tiles)
+                launch(k_resid_restrict_tile<SI>, t3_grid(gc.n1, gc.n2, kT3 / 2, B), kT3Threads,
+                       t3_smem_restrict(g.n0, sizeof(A)), st(), op, gc, act, cur, b, lev[l + 1].Bb);
+            else launch(k_resid_restrict<SI>, cbl, cth, 0, st(), op, gc, pmc, B, act, cur, b, lev[l + 1].Bb);
         } else if (cur.d == nullptr) {
             bytes_hint(1.0 * nact * (g.nx + gc.nx) * sizeof(SI));
             launch(k_restrict<SI>, cbl, cth, 0, st(), g, gc, pmc, B, act, b, lev[l + 1].Bb);
@@ -968,7 +981,10 @@ class Precond : public PrecondBase {
         if (fps) {
             Vec<SI> d = dest();
             bytes_hint(1.0 * nact * (gc.nx + (cur.d ? 3.0 : 2.0) * g.nx) * sizeof(SI));
-            launch(k_prolong_smooth<SI>, pbl, pth, 0, st(), op, gc, pm, B, act, lev[l + 1].X, cur, b, d, om);
+            if (tiles)
+                launch(k_prolong_smooth_tile<SI>, t3_grid(g.n1, g.n2, kT3, B), kT3Threads, t3_smem_prolong(g.n0, sizeof(A)),
+                       st(), op, gc, act, lev[l + 1].X, cur, b, d, om);
+            else launch(k_prolong_smooth<SI>, pbl, pth, 0, st(), op, gc, pm, B, act, lev[l + 1].X, cur, b, d, om);
             cur = d;
             q = 1;
         } else {
@@ -1032,6 +1048,15 @@ class Precond : public PrecondBase {
             if constexpr (!PT<SI>::scaled) {
                 if (!h->q1) {
                     launch_rana_vec(B, act, V, i, Z, transpose);
+                    AAO_TRY(mg_solve(i, B, act, mgb, Zi));
+                    continue;
+                }
+            }
+            if constexpr (PT<SI>::scaled) {
+                if (!h->q1) {
+                    launch(k_rana_pt<SP, SI>, pt_grid(pm0, g.R, B), pt_block(pm0), 0, st(), g, inv_h2<A>(g), pm0, B, act, V,
+                           (long long)s * g.R, i, Z, stage_coef(i, transpose), facesA, mgb);
+                    AAO_LAUNCH_CHECK();
                     AAO_TRY(mg_solve(i, B, act, mgb, Zi));
                     continue;
                 }
@@ -1108,14 +1133,20 @@ class Precond : public PrecondBase {
         }
     }
 
-    void launch_rana_vec(int B, const int* act, Vec<SP> V, int i, Vec<SI> Z, int transpose) {
-        const Geo& g = h->g;
+    StageCoef<A> stage_coef(int i, int transpose) const {
         const int s = h->s;
         StageCoef<A> cf{};
         cf.j0 = transpose ? i + 1 : 0;
         cf.j1 = transpose ? s : i;
         for (int j = cf.j0; j < cf.j1; ++j)
             cf.c[j] = (A)h->tau * (A)(transpose ? h->L[j * s + i] * h->D[i] : h->L[i * s + j] * h->D[j]);
+        return cf;
+    }
+
+    void launch_rana_vec(int B, const int* act, Vec<SP> V, int i, Vec<SI> Z, int transpose) {
+        const Geo& g = h->g;
+        const int s = h->s;
+        const StageCoef<A> cf = stage_coef(i, transpose);
         with_int(rows_vec(), [&](auto big) {
             constexpr int N = decltype(big)::value ? kVN : 1;
             const long long pos = (long long)(g.n0 / N) * g.R;
