@@ -27,7 +27,9 @@ namespace aao {
 
 constexpr int kArThreads = 128;
 constexpr int kArWarps = kArThreads / kWarp;
-constexpr int kArBlocks = 152 * 8;       // blocks of a reducing launch over the whole batch
+constexpr int kArBlocks = 152 * 48;      // blocks of a reducing launch over the whole batch: beyond three or so
+                                         // per thread slot, positions are chained per thread (128 blocks of 256^2
+                                         // in k_theta_dots: 277 us with eight blocks per SM)
 constexpr int kArSmallK = 5;             // inner iterations of the small instance (the defaults: 3 and 5)
 
 // N consecutive stored values as arithmetic values: one 8- or 16-byte load where N values make one
@@ -622,14 +624,13 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_rana_pt(Geo g, InvH2<typename
 // double -> float for values a float holds exactly, by integer operations (an FP64 conversion costs as
 // much as an FP64 operation); false where d is not a float of moderate size or zero.
 __device__ __forceinline__ bool exact_float(double d, float& f) {
-    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-    const unsigned e = hi >> 20 & 0x7ffu;
-    if ((hi << 1 | lo) == 0u) {
-        f = 0.f;
-        return true;
-    }
-    f = __uint_as_float((hi & 0x80000000u) | (e - 896u) << 23 | (hi & 0xfffffu) << 3 | lo >> 29);
-    return (lo & 0x1fffffffu) == 0u && e - 940u < 170u;      // 2^-83 <= |d| < 2^87
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), mag = hi & 0x7fffffffu;
+    // the exponent field minus 896 and the upper 23 bits of the fraction, then the sign
+    const unsigned bits = (__funnelshift_l(lo, hi, 3) - (896u << 23)) | (hi & 0x80000000u);
+    const bool zero = (mag | lo) == 0u;
+    f = zero ? 0.f : __uint_as_float(bits);
+    // 2^-83 <= |d| < 2^87, no fraction bits beyond a float's
+    return zero || ((lo & 0x1fffffffu) == 0u && mag - (940u << 20) < (170u << 20));
 }
 __device__ __forceinline__ float to_arith(double d, float) {
     float f;
@@ -643,26 +644,27 @@ __device__ __forceinline__ double to_fp64(float v) {
 }
 __device__ __forceinline__ double to_fp64(double v) { return v; }
 
-// Double-float values (hi + lo, about 48 bits): error-free sums and differences after Knuth (TAOCP 2,
-// 4.2.2) and products by one fused multiply-add.
+// Double-float values (hi + lo, about 48 bits): error-free sums after Knuth (TAOCP 2, 4.2.2), products by one
+// fused multiply-add.
 struct FF {
     float hi, lo;
 };
 __device__ __forceinline__ FF ff_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = s - a;
-    return FF{s, (a - (s - bb)) + (b - bb)};
+    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
+    return FF{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
+}
+// 2 P - a - b
+__device__ __forceinline__ FF ff_diff2(float P, float a, float b) {
+    const FF x = ff_sum(P, -a), y = ff_sum(P, -b), s = ff_sum(x.hi, y.hi);
+    return FF{s.hi, s.lo + (x.lo + y.lo)};
 }
 __device__ __forceinline__ FF ff_add(FF a, FF b) {
     const FF s = ff_sum(a.hi, b.hi);
-    const float lo = s.lo + (a.lo + b.lo);
-    const float h = s.hi + lo;
-    return FF{h, lo - (h - s.hi)};
+    return FF{s.hi, s.lo + (a.lo + b.lo)};
 }
 __device__ __forceinline__ FF ff_mul(FF a, FF b) {
     const float p = __fmul_rn(a.hi, b.hi);
-    const float lo = fmaf(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi);
-    const float h = __fadd_rn(p, lo);
-    return FF{h, lo - (h - p)};
+    return FF{p, fmaf(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi)};
 }
 struct H2FF {
     FF x, y, z;
@@ -674,82 +676,63 @@ inline FF to_ff(double d) {
     return f;
 }
 
-// K z at N consecutive points from its FP64 values, rounded once to A (FD).  For A = float the sums run
-// in double-float arithmetic, whose error (2^-46 of the largest term) is below the final rounding by as
-// wide a margin as FP64's in practice: K z cancels to 1e-4 of its terms on the finest grids, so the
-// rounded results agree but for ties.  FP64 needs 7 operations per point at two per cycle and SM.
-// A point whose values are not floats of moderate size, and Q1, take FP64.
-template <int N, class A>
-__device__ __forceinline__ void schur_K(const double* u, const Geo& g, const H2FF& h, const SpaceOp<A>& op, int row,
-                                        int j, int k, int c, A* out) {
+// K z at a point in FP64, rounded to A (out of line: FP32's rare path, Q1 and FP64).
+template <class A>
+__device__ __noinline__ A schur_K64(const double* u, const Geo& g, const SpaceOp<A>& op, int row, int j, int k, int c) {
+    const View<double> z{u, nullptr, g.n0};
+    return (A)op_K(z, g, op, row, j, k, c);
+}
+
+// K z at a point from its FP64 values, rounded once to A (FD).  For A = float the sums run in double-float
+// arithmetic, whose error (2^-46 of the largest term) is below the final rounding by as wide a margin as
+// FP64's in practice: K z cancels to 1e-4 of its terms on the finest grids, so the rounded results agree
+// but for ties.  FP64 needs 7 operations per point at two per cycle and SM.  A point whose values are not floats
+// of moderate size takes FP64.  One point per thread and the FP64 code out of line: four points per thread,
+// all inline, were 98 KB of code and 63 us for 14 items of 256^2, most of it instruction fetches.
+template <class A, bool D3>
+__device__ __forceinline__ A schur_K(const double* u, const Geo& g, const H2FF& h, const SpaceOp<A>& op, int row, int j,
+                                     int k, int c) {
     if constexpr (std::is_same<A, float>::value) {
-        if (!op.q1) {
-            const double* p = u + (long long)row * g.n0 + c;
-            const long long pl = (long long)g.n0 * g.n1;
-            const bool hs = j > 0, hn = j + 1 < g.n1, hd = g.d == 3 && k > 0, hu = g.d == 3 && k + 1 < g.n2;
-            double dp[N + 2], ds[N], dn[N], dd[N], du[N];
-            dp[0] = c > 0 ? p[-1] : 0.0;
-            dp[N + 1] = c + N < g.n0 ? p[N] : 0.0;
+        const double* p = u + (long long)row * g.n0 + c;
+        const int pl = g.n0 * g.n1;
+        double d[7];
+        d[0] = p[0];
+        d[1] = c > 0 ? p[-1] : 0.0;
+        d[2] = c + 1 < g.n0 ? p[1] : 0.0;
+        d[3] = j > 0 ? p[-g.n0] : 0.0;
+        d[4] = j + 1 < g.n1 ? p[g.n0] : 0.0;
+        if (D3) {
+            d[5] = k > 0 ? p[-pl] : 0.0;
+            d[6] = k + 1 < g.n2 ? p[pl] : 0.0;
+        }
+        float f[7];
+        bool ok = !op.q1;
 #pragma unroll
-            for (int t = 0; t < N; ++t) {
-                dp[t + 1] = p[t];
-                ds[t] = hs ? p[t - g.n0] : 0.0;
-                dn[t] = hn ? p[t + g.n0] : 0.0;
-                if (g.d == 3) {
-                    dd[t] = hd ? p[t - pl] : 0.0;
-                    du[t] = hu ? p[t + pl] : 0.0;
+        for (int q = 0; q < (D3 ? 7 : 5); ++q) ok = exact_float(d[q], f[q]) && ok;
+        if (ok) {
+            FF r;
+            if (op.faces.fx == nullptr) {
+                r = ff_add(ff_mul(ff_diff2(f[0], f[1], f[2]), h.x), ff_mul(ff_diff2(f[0], f[3], f[4]), h.y));
+                if (D3) r = ff_add(r, ff_mul(ff_diff2(f[0], f[5], f[6]), h.z));
+            } else {
+                const int fxi = row * (g.n0 + 1) + c, fyi = (k * (g.n1 + 1) + j) * g.n0 + c;
+                auto term = [&](float nb, float face) { return ff_mul(ff_sum(f[0], -nb), FF{face, 0.f}); };
+                r = ff_add(ff_add(term(f[1], op.faces.fx[fxi]), term(f[2], op.faces.fx[fxi + 1])),
+                           ff_add(term(f[3], op.faces.fy[fyi]), term(f[4], op.faces.fy[fyi + g.n0])));
+                if (D3) {
+                    const int fzi = row * g.n0 + c;
+                    r = ff_add(r, ff_add(term(f[5], op.faces.fz[fzi]), term(f[6], op.faces.fz[fzi + pl])));
                 }
             }
-            float P[N + 2];
-            bool okp[N + 2];
-#pragma unroll
-            for (int t = 0; t < N + 2; ++t) okp[t] = exact_float(dp[t], P[t]);
-#pragma unroll
-            for (int t = 0; t < N; ++t) {
-                float S, Nn, D = 0.f, U = 0.f;
-                const float Pc = P[t + 1];
-                bool ok = okp[t] && okp[t + 1] && okp[t + 2];
-                ok = exact_float(ds[t], S) && ok;
-                ok = exact_float(dn[t], Nn) && ok;
-                if (g.d == 3) {
-                    ok = exact_float(dd[t], D) && ok;
-                    ok = exact_float(du[t], U) && ok;
-                }
-                if (!ok) {
-                    const View<double> z{u, nullptr, g.n0};
-                    out[t] = (A)op_K(z, g, op, row, j, k, c + t);
-                    continue;
-                }
-                FF r;
-                if (op.faces.fx == nullptr) {
-                    r = ff_add(ff_mul(ff_add(ff_sum(Pc, -P[t]), ff_sum(Pc, -P[t + 2])), h.x),
-                               ff_mul(ff_add(ff_sum(Pc, -S), ff_sum(Pc, -Nn)), h.y));
-                    if (g.d == 3) r = ff_add(r, ff_mul(ff_add(ff_sum(Pc, -D), ff_sum(Pc, -U)), h.z));
-                } else {
-                    const long long fxi = (long long)row * (g.n0 + 1) + c + t;
-                    const long long fyi = ((long long)k * (g.n1 + 1) + j) * g.n0 + c + t;
-                    auto term = [&](float nb, float face) { return ff_mul(ff_sum(Pc, -nb), FF{face, 0.f}); };
-                    r = ff_add(ff_add(term(P[t], op.faces.fx[fxi]), term(P[t + 2], op.faces.fx[fxi + 1])),
-                               ff_add(term(S, op.faces.fy[fyi]), term(Nn, op.faces.fy[fyi + g.n0])));
-                    if (g.d == 3) {
-                        const long long fzi = ((long long)k * g.n1 + j) * g.n0 + c + t;
-                        r = ff_add(r, ff_add(term(D, op.faces.fz[fzi]),
-                                             term(U, op.faces.fz[fzi + (long long)g.n1 * g.n0])));
-                    }
-                }
-                out[t] = r.hi + r.lo;
-            }
-            return;
+            return r.hi + r.lo;
         }
     }
-    const View<double> z{u, nullptr, g.n0};
-#pragma unroll
-    for (int t = 0; t < N; ++t) out[t] = (A)op_K(z, g, op, row, j, k, c + t);
+    return schur_K64<A>(u, g, op, row, j, k, c);
 }
 
 // t = K z_{v,n} (every stage's right-hand side: one copy) and the start of the step's inner solves with
 // ||r|| = sqrt(s) ||t||.
-template <class A, int N>
+template <class A, bool D3>
 __global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, H2FF h, int s, const StepPtrs* sp, int stride, A* t,
                                                             SpaceOp<A> sop, ArRed red, ArItems it) {
     pdl_prologue();
@@ -757,17 +740,15 @@ __global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, H2FF h, int s
     const int b = blockIdx.y;
     const double* z = sp->z + (long long)(sp->n + b * stride) * g.nx;
     A* tb = t + (long long)b * g.nx;
-    const unsigned nv = (unsigned)g.n0 / N, npos = nv * (unsigned)g.R;
     A acc = A(0);
-    for (unsigned q = blockIdx.x * kArThreads + threadIdx.x; q < npos; q += red.nchunk * kArThreads) {
-        const int row = (int)(q / nv), c = (int)(q - row * nv) * N;
+#pragma unroll 1
+    for (unsigned q = blockIdx.x * kArThreads + threadIdx.x; q < (unsigned)g.nx; q += red.nchunk * kArThreads) {
+        const int row = (int)(q / (unsigned)g.n0), c = (int)(q - row * g.n0);
         int j, k;
         row_jk(g, row, j, k);
-        A v[N];
-        schur_K<N, A>(z, g, h, sop, row, j, k, c, v);
-        st_n<N>(tb + (long long)q * N, v);
-#pragma unroll
-        for (int i = 0; i < N; ++i) acc += v[i] * v[i];
+        const A v = schur_K<A, D3>(z, g, h, sop, row, j, k, c);
+        tb[q] = v;
+        acc += v * v;
     }
     if (ar_reduce<1>(&acc, 1u, red, sum, [] {}) && threadIdx.x == 0) ar_init(it, b, sqrt((double)s * sum[0]));
 }

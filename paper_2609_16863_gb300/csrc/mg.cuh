@@ -10,6 +10,8 @@
 // along x, so a row's per-row scale (16-bit storage) is one warp reduction.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace aao {
@@ -787,6 +789,278 @@ inline dim3 vec16_grid(const LevelOp<S>& op, int B) {
     return dim3((unsigned)((op.g.R + rows_per_block - 1) / rows_per_block), (unsigned)B, 1);
 }
 
+// 1D interpolation stencil of fine 0-based index F: up to two coarse indices.
+__device__ __forceinline__ int interp_1d(int F, int nc, int* J, float* wt) {
+    int g = F + 1;  // 1-based
+    if ((g & 1) == 0) {
+        J[0] = g / 2 - 1;
+        wt[0] = 1.f;
+        return 1;
+    }
+    int m = 0;
+    int j1 = (g - 1) / 2 - 1, j2 = (g + 1) / 2 - 1;
+    if (j1 >= 0 && j1 < nc) { J[m] = j1; wt[m] = 0.5f; ++m; }
+    if (j2 >= 0 && j2 < nc) { J[m] = j2; wt[m] = 0.5f; ++m; }
+    return m;
+}
+
+// The power-of-two scale of a 16-bit row whose values res[0..N) are held by a group of gs lanes of a warp
+// (pt_store's rule); returns its reciprocal.
+template <int N> __device__ __forceinline__ float group_scale(const float* res, int gs, float& sc) {
+    float m = 0.f;
+#pragma unroll
+    for (int t = 0; t < N; ++t) m = fmaxf(m, fabsf(res[t]));
+    for (int o = gs >> 1; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int ex = 0;
+    sc = 1.f;
+    float inv = 1.f;
+    if (m > 0.f && m <= 3.0e38f) {
+        frexpf(m, &ex);
+        sc = ldexpf(1.f, ex - 14);
+        inv = ldexpf(1.f, 14 - ex);
+    }
+    return inv;
+}
+// Lanes of a row's group: the power of two that holds n0 / N vectors.
+inline int row_group(int n0, int N) {
+    int gs = 1;
+    while (gs < n0 / N) gs <<= 1;
+    return gs;
+}
+template <class S> inline dim3 row_group_grid(const Geo& g, int N, int B) {
+    const int rows = (kVecThreads / kWarp) * (kWarp / row_group(g.n0, N));
+    return dim3((unsigned)((g.R + rows - 1) / rows), (unsigned)B, 1);
+}
+
+// A 3D level with a stored 27-point stencil, FP32 arithmetic: a thread owns 4 consecutive columns of a row, so
+// a row of x costs one vector load and two scalars for 12 products and a stencil component one vector load
+// for 4; the lanes of a row form a group within a warp for the storage scale.  MODE 0: damped Jacobi; 1: from x =
+// 0; 2: residual.  The operations of level_apply_k<3> per point in its order.  Bound by instructions: one
+// point per thread spent about 300 per point on addresses, conversions and predicates.
+template <class S, int MODE>
+__global__ void __launch_bounds__(kVecThreads) k_st27(LevelOp<S> op, int gs, const int* active, Vec<S> xin, Vec<S> bv,
+                                                      Vec<S> out, float omega) {
+    pdl_prologue();
+    constexpr int N = 4;
+    constexpr bool SC = PT<S>::scaled;
+    using RT = typename std::conditional<sizeof(S) == 2, uint2, uint4>::type;
+    __shared__ float ssc[27];
+    if (SC) {
+        if (threadIdx.x < 27) ssc[threadIdx.x] = op.sten_sc[threadIdx.x];
+        __syncthreads();
+    }
+    const Geo& g = op.g;
+    const int b = blockIdx.y;
+    if (active && !active[b]) return;
+    const int n0 = g.n0, tpr = n0 / N, nx = (int)g.nx;
+    const int lane = threadIdx.x & 31, grp = lane / gs, gl = lane - grp * gs;
+    const int row = (blockIdx.x * (kVecThreads / 32) + (threadIdx.x >> 5)) * (32 / gs) + grp;
+    const bool valid = row < g.R && gl < tpr;
+    const int c = gl * N;
+    float res[N] = {0.f, 0.f, 0.f, 0.f};
+    auto ld4 = [](const S* p, float* v) {
+        const RT r = *reinterpret_cast<const RT*>(p);
+        const S* e = reinterpret_cast<const S*>(&r);
+#pragma unroll
+        for (int t = 0; t < N; ++t) v[t] = PT<S>::ld(e[t]);
+    };
+    if (valid) {
+        int j, k;
+        row_jk(g, row, j, k);
+        const int p = row * n0 + c;
+        const S* X = MODE == 1 ? nullptr : xin.d + (long long)b * xin.bs;
+        const float* XS = SC && MODE != 1 ? xin.sc + (long long)b * xin.bs / n0 : nullptr;
+        float bq[N], ctr[N], P[N];
+        ld4(bv.d + (long long)b * bv.bs + p, bq);
+        if (SC) {
+            const float f = bv.sc[(long long)b * bv.bs / n0 + row];
+#pragma unroll
+            for (int t = 0; t < N; ++t) bq[t] *= f;
+        }
+        if (MODE == 1) {
+            ld4(op.sten + 13 * nx + p, ctr);
+#pragma unroll
+            for (int t = 0; t < N; ++t) res[t] = omega * bq[t] / (SC ? ctr[t] * ssc[13] : ctr[t]);
+        } else {
+            float acc[N] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int r = 0; r < 9; ++r) {
+                const int dy = r % 3 - 1, dz = r / 3 - 1;
+                if (j + dy < 0 || j + dy >= g.n1 || k + dz < 0 || k + dz >= g.n2) continue;
+                const int rr = row + dy + dz * g.n1;
+                const S* xr = X + rr * n0 + c;
+                float x[N + 2];
+                ld4(xr, x + 1);
+                x[0] = c > 0 ? PT<S>::ld(xr[-1]) : 0.f;
+                x[N + 1] = c + N < n0 ? PT<S>::ld(xr[N]) : 0.f;
+                if (SC) {
+                    const float f = XS[rr];
+#pragma unroll
+                    for (int t = 0; t < N + 2; ++t) x[t] *= f;
+                }
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    float s[N];
+                    ld4(op.sten + (3 * r + d) * nx + p, s);
+                    if (SC) {
+                        const float f = ssc[3 * r + d];
+#pragma unroll
+                        for (int t = 0; t < N; ++t) s[t] *= f;
+                    }
+#pragma unroll
+                    for (int t = 0; t < N; ++t) acc[t] += s[t] * x[t + d];
+                    if (3 * r + d == 13) {
+#pragma unroll
+                        for (int t = 0; t < N; ++t) {
+                            ctr[t] = s[t];
+                            P[t] = x[t + 1];
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t) res[t] = MODE == 0 ? P[t] + omega * (bq[t] - acc[t]) / ctr[t] : bq[t] - acc[t];
+        }
+    }
+    S* o = out.d + (long long)b * out.bs + (long long)row * n0 + c;
+    if constexpr (SC) {
+        float sc;
+        const float inv = group_scale<N>(res, gs, sc);
+        if (valid) {
+            RT ov;
+            S* oq = reinterpret_cast<S*>(&ov);
+#pragma unroll
+            for (int t = 0; t < N; ++t) oq[t] = PT<S>::st(res[t] * inv);
+            *reinterpret_cast<RT*>(o) = ov;
+            if (gl == 0) out.sc[(long long)b * out.bs / n0 + row] = sc;
+        }
+    } else if (valid) {
+        *reinterpret_cast<float4*>(o) = make_float4(res[0], res[1], res[2], res[3]);
+    }
+}
+// Whether a level takes k_st27: FP32 arithmetic, rows of whole 4-column vectors with at most 32 of them.
+template <class S> inline bool st27_ok(const LevelOp<S>& op) {
+    return std::is_same<typename PT<S>::A, float>::value && !op.fine && op.g.d == 3 && op.g.n0 % 4 == 0 && op.g.n0 <= 128;
+}
+
+// x_out = x_in + P xc (x_in.d == nullptr: 0) for 16-bit storage: a thread owns 8 fine columns; each of the (one,
+// two or four) coarse rows behind its row costs one vector load of 4 and two scalars.  Per point the sum of
+// k_prolong_add in its order.  (That kernel formed indices, weights and predicates per point and coarse value:
+// 17 us for a 96^3 item, 114 us for eight.)
+template <class S>
+__global__ void __launch_bounds__(kVecThreads) k_prolong16(Geo gf, Geo gc, int gs, const int* active, Vec<S> xcv,
+                                                           Vec<S> xin, Vec<S> xout) {
+    pdl_prologue();
+    static_assert(PT<S>::scaled, "16-bit storage only");
+    const int b = blockIdx.y;
+    if (active && !active[b]) return;
+    const int n0 = gf.n0, tpr = n0 / 8;
+    const int lane = threadIdx.x & 31, grp = lane / gs, gl = lane - grp * gs;
+    const int row = (blockIdx.x * (kVecThreads / 32) + (threadIdx.x >> 5)) * (32 / gs) + grp;
+    const bool valid = row < gf.R && gl < tpr;
+    const int c0 = gl * 8, cc = gl * 4;
+    float res[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) res[t] = 0.f;
+    if (valid) {
+        int j, k;
+        row_jk(gf, row, j, k);
+        int Jy[2] = {0, 0}, Jz[2] = {0, 0};
+        float wy[2], wz[2] = {1.f, 0.f};
+        const int my = interp_1d(j, gc.n1, Jy, wy), mz = gf.d == 3 ? interp_1d(k, gc.n2, Jz, wz) : 1;
+        if (xin.d) vec8_load(xin.d + (long long)b * xin.bs + row * n0 + c0, xin.sc[(long long)b * xin.bs / n0 + row], res);
+        const S* C = xcv.d + (long long)b * xcv.bs;
+        const float* CS = xcv.sc + (long long)b * xcv.bs / gc.n0;
+        for (int a = 0; a < mz; ++a)
+            for (int q = 0; q < my; ++q) {
+                const int cr = Jy[q] + gc.n1 * Jz[a];
+                const float f = CS[cr], w = wy[q] * wz[a], h = w * 0.5f;
+                const S* p = C + cr * gc.n0 + cc;
+                const uint2 raw = *reinterpret_cast<const uint2*>(p);
+                const S* e = reinterpret_cast<const S*>(&raw);
+                float v[6];
+                v[0] = cc > 0 ? PT<S>::ld(p[-1]) * f : 0.f;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) v[t + 1] = PT<S>::ld(e[t]) * f;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    res[2 * t] += h * v[t];
+                    res[2 * t] += h * v[t + 1];
+                    res[2 * t + 1] += w * v[t + 1];
+                }
+            }
+    }
+    float sc;
+    const float inv = group_scale<8>(res, gs, sc);
+    if (valid) {
+        uint4 ov;
+        S* oq = reinterpret_cast<S*>(&ov);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) oq[t] = PT<S>::st(res[t] * inv);
+        *reinterpret_cast<uint4*>(xout.d + (long long)b * xout.bs + (long long)row * n0 + c0) = ov;
+        if (gl == 0) xout.sc[(long long)b * xout.bs / n0 + row] = sc;
+    }
+}
+
+// bc = P^T r for 16-bit storage: a thread owns 4 coarse columns, 8 fine columns (one vector) and the one after
+// of each of its 9 (3 in 2D) fine rows; per point the sum of k_restrict in its order.
+template <class S>
+__global__ void __launch_bounds__(kVecThreads) k_restrict16(Geo gf, Geo gc, int gs, const int* active, Vec<S> rv,
+                                                            Vec<S> bcv) {
+    pdl_prologue();
+    static_assert(PT<S>::scaled, "16-bit storage only");
+    const int b = blockIdx.y;
+    if (active && !active[b]) return;
+    const int n0 = gc.n0, tpr = n0 / 4;
+    const int lane = threadIdx.x & 31, grp = lane / gs, gl = lane - grp * gs;
+    const int row = (blockIdx.x * (kVecThreads / 32) + (threadIdx.x >> 5)) * (32 / gs) + grp;
+    const bool valid = row < gc.R && gl < tpr;
+    const int I0 = gl * 4, f0 = gl * 8;
+    float res[4] = {0.f, 0.f, 0.f, 0.f};
+    if (valid) {
+        int J, K;
+        row_jk(gc, row, J, K);
+        const S* R = rv.d + (long long)b * rv.bs;
+        const float* RS = rv.sc + (long long)b * rv.bs / gf.n0;
+        const int nz = gf.d == 3 ? 3 : 1;
+#pragma unroll 1
+        for (int z = 0; z < nz; ++z) {
+            const int fk = gf.d == 3 ? 2 * K + z : 0;
+            if (fk >= gf.n2) continue;
+            const float wz = nz == 1 || z == 1 ? 1.f : 0.5f;
+#pragma unroll
+            for (int y = 0; y < 3; ++y) {
+                const int fj = 2 * J + y;
+                if (fj >= gf.n1) continue;
+                const int fr = fj + gf.n1 * fk;
+                const float w = (y == 1 ? 1.f : 0.5f) * wz, h = 0.5f * w, f = RS[fr];
+                const S* p = R + fr * gf.n0 + f0;
+                float v[9];
+                vec8_load(p, f, v);
+                v[8] = f0 + 8 < gf.n0 ? PT<S>::ld(p[8]) * f : 0.f;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    res[t] += h * v[2 * t];
+                    res[t] += w * v[2 * t + 1];
+                    res[t] += h * v[2 * t + 2];
+                }
+            }
+        }
+    }
+    float sc;
+    const float inv = group_scale<4>(res, gs, sc);
+    if (valid) {
+        uint2 ov;
+        S* oq = reinterpret_cast<S*>(&ov);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) oq[t] = PT<S>::st(res[t] * inv);
+        *reinterpret_cast<uint2*>(bcv.d + (long long)b * bcv.bs + (long long)row * n0 + I0) = ov;
+        if (gl == 0) bcv.sc[(long long)b * bcv.bs / n0 + row] = sc;
+    }
+}
+// Whether two levels' transfers take the 16-bit vector kernels: fine rows of whole 16-byte vectors, at most 32.
+template <class S> inline bool transfer16_ok(const Geo& gf) { return PT<S>::scaled && gf.n0 % 8 == 0 && gf.n0 <= 256; }
+
 // r = b - A x for unscaled storage, RPT rows per thread (as k_smooth_rows).
 template <class S, int KIND, int RPT>
 __global__ void __launch_bounds__(kPtMaxThreads) k_residual_rows(LevelOp<S> op, PtMap pm, int B, const int* active,
@@ -910,21 +1184,6 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_restrict(Geo gf, Geo gc, PtMa
         }
         return acc;
     });
-}
-
-// 1D interpolation stencil of fine 0-based index F: up to two coarse indices.
-__device__ __forceinline__ int interp_1d(int F, int nc, int* J, float* wt) {
-    int g = F + 1;  // 1-based
-    if ((g & 1) == 0) {
-        J[0] = g / 2 - 1;
-        wt[0] = 1.f;
-        return 1;
-    }
-    int m = 0;
-    int j1 = (g - 1) / 2 - 1, j2 = (g + 1) / 2 - 1;
-    if (j1 >= 0 && j1 < nc) { J[m] = j1; wt[m] = 0.5f; ++m; }
-    if (j2 >= 0 && j2 < nc) { J[m] = j2; wt[m] = 0.5f; ++m; }
-    return m;
 }
 
 // x_out = x_in + P xc  (fine row kernel); x_in.d == nullptr means 0.
@@ -1727,12 +1986,14 @@ __global__ void __launch_bounds__(1024) k_vcycle_tail(TailCtx<SI> t, int B, cons
     const int lc = t.lc, L = t.L;
     // per level: X0, X1 (x ping-pong; the free one holds the residual), B
     unsigned cur = 0u;      // bit l: which of level l's two x buffers holds the iterate
-    // copy the coarse stencils of levels >= stage_from into shared memory
+    // copy the coarse stencils of levels >= stage_from into shared memory, 16 bytes at a time
     for (int l = t.stage_from; l < L; ++l) {
         if (l < 1) continue;
-        const long long n = (long long)t.op[l].ncoef * t.op[l].g.nx;
+        const int n = t.op[l].ncoef * (int)t.op[l].g.nx, n16 = n * (int)sizeof(SI) / 16, per = 16 / (int)sizeof(SI);
         SI* dst = reinterpret_cast<SI*>(tail_smem + t.sten_off[l]);
-        for (long long i = tid; i < n; i += nt) dst[i] = t.op[l].sten[i];
+        const SI* src = t.op[l].sten;
+        for (int i = tid; i < n16; i += nt) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
+        for (int i = n16 * per + tid; i < n; i += nt) dst[i] = src[i];
     }
     {
         const Geo& g = t.op[lc].g;
@@ -1813,11 +2074,14 @@ __global__ void __launch_bounds__(1024) k_vcycle_tail(TailCtx<SI> t, int B, cons
         const Geo& g = t.op[L - 1].g;
         A* X = sm + t.off[L - 1] + (long long)((cur >> (L - 1)) & 1u) * g.nx;
         const A* Bv = sm + t.off[L - 1] + 2 * g.nx;
-        const int nc = (int)g.nx;
-        for (int p = tid; p < nc; p += nt) {
+        const int nc = (int)g.nx, w = tid >> 5, lane = tid & 31, nw = nt >> 5;
+        for (int p = w; p < nc; p += nw) {         // a warp per row of the inverse
+            const A* D = t.Dinv + (long long)p * nc;
             A acc = A(0);
-            for (int q = 0; q < nc; ++q) acc += t.Dinv[(long long)p * nc + q] * Bv[q];
-            X[p] = acc;
+#pragma unroll 4
+            for (int q = lane; q < nc; q += kWarp) acc += D[q] * Bv[q];
+            acc = warp_sum(acc);
+            if (lane == 0) X[p] = acc;
         }
     }
     __syncthreads();

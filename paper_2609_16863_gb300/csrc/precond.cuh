@@ -835,6 +835,15 @@ class Precond : public PrecondBase {
                 return;
             }
         }
+        if constexpr (std::is_same<A, float>::value) {
+            if (st27_ok(op)) {
+                const int gs = row_group(op.g.n0, 4);
+                const dim3 gr = row_group_grid<SI>(op.g, 4, B);
+                if (x.d) launch(k_st27<SI, 0>, gr, kVecThreads, 0, st(), op, gs, act, x, b, out, om);
+                else launch(k_st27<SI, 1>, gr, kVecThreads, 0, st(), op, gs, act, x, b, out, om);
+                return;
+            }
+        }
         launch_smooth_rows(kind, grid, block, op, pm, B, act, x, b, out, om);
     }
     template <class... Args> void launch_smooth_rows(int kind, dim3 grid, dim3 block, Args... args) {
@@ -873,7 +882,40 @@ class Precond : public PrecondBase {
                 return;
             }
         }
+        if constexpr (std::is_same<A, float>::value) {
+            if (st27_ok(op) && x.d) {
+                launch(k_st27<SI, 2>, row_group_grid<SI>(op.g, 4, B), kVecThreads, 0, st(), op, row_group(op.g.n0, 4), act, x,
+                       b, out, A(0));
+                return;
+            }
+        }
         launch_residual_rows(kind, grid, block, op, pm, B, act, x, b, out);
+    }
+    void launch_restrict(const Geo& gf, const Geo& gc, int B, const int* act, Vec<SI> r, Vec<SI> bc) {
+        if constexpr (PT<SI>::scaled) {
+            if (transfer16_ok<SI>(gf)) {
+                launch(k_restrict16<SI>, row_group_grid<SI>(gc, 4, B), kVecThreads, 0, st(), gf, gc, row_group(gc.n0, 4), act,
+                       r, bc);
+                return;
+            }
+        }
+        const PtMap pmc = ptmap(gc.n0);
+        launch(k_restrict<SI>, pt_grid(pmc, gc.R, B), pt_block(pmc), 0, st(), gf, gc, pmc, B, act, r, bc);
+    }
+    void launch_prolong(const Geo& gf, const Geo& gc, int B, const int* act, Vec<SI> xc, Vec<SI> x, Vec<SI> out) {
+        const PtMap pm = ptmap(gf.n0);
+        const dim3 pbl = pt_grid(pm, gf.R, B), pth = pt_block(pm);
+        if constexpr (PT<SI>::scaled) {
+            if (transfer16_ok<SI>(gf)) {
+                launch(k_prolong16<SI>, row_group_grid<SI>(gf, 8, B), kVecThreads, 0, st(), gf, gc, row_group(gf.n0, 8), act,
+                       xc, x, out);
+                return;
+            }
+        } else if (gf.d == 2 && B >= 16) {
+            launch(k_prolong_add_rows<SI, 4>, dim3((pbl.x + 3) / 4, pbl.y), pth, 0, st(), gf, gc, pm, B, act, xc, x, out);
+            return;
+        }
+        launch(k_prolong_add<SI>, pbl, pth, 0, st(), gf, gc, pm, B, act, xc, x, out);
     }
     template <class... Args> void launch_residual_rows(int kind, dim3 grid, dim3 block, Args... args) {
         if constexpr (!PT<SI>::scaled) {
@@ -967,12 +1009,12 @@ class Precond : public PrecondBase {
             else launch(k_resid_restrict<SI>, cbl, cth, 0, st(), op, gc, pmc, B, act, cur, b, lev[l + 1].Bb);
         } else if (cur.d == nullptr) {
             bytes_hint(1.0 * nact * (g.nx + gc.nx) * sizeof(SI));
-            launch(k_restrict<SI>, cbl, cth, 0, st(), g, gc, pmc, B, act, b, lev[l + 1].Bb);
+            launch_restrict(g, gc, B, act, b, lev[l + 1].Bb);
         } else {
             bytes_hint(3.0 * nact * g.nx * sizeof(SI));
             launch_residual(level_kind(op.fine, g.d), pbl, pth, op, pm, B, act, cur, b, lev[l].Rr);
             bytes_hint(1.0 * nact * (g.nx + gc.nx) * sizeof(SI));
-            launch(k_restrict<SI>, cbl, cth, 0, st(), g, gc, pmc, B, act, lev[l].Rr, lev[l + 1].Bb);
+            launch_restrict(g, gc, B, act, lev[l].Rr, lev[l + 1].Bb);
         }
         AAO_LAUNCH_CHECK();
         Vec<SI> zero{};
@@ -990,15 +1032,7 @@ class Precond : public PrecondBase {
         } else {
             Vec<SI> d = dest();
             bytes_hint(1.0 * nact * (gc.nx + (cur.d ? 2.0 : 1.0) * g.nx) * sizeof(SI));
-            bool rows_done = false;
-            if constexpr (!PT<SI>::scaled) {
-                if (g.d == 2 && B >= 16) {
-                    launch(k_prolong_add_rows<SI, 4>, dim3((pbl.x + 3) / 4, pbl.y), pth, 0, st(), g, gc, pm, B, act,
-                           lev[l + 1].X, cur, d);
-                    rows_done = true;
-                }
-            }
-            if (!rows_done) launch(k_prolong_add<SI>, pbl, pth, 0, st(), g, gc, pm, B, act, lev[l + 1].X, cur, d);
+            launch_prolong(g, gc, B, act, lev[l + 1].X, cur, d);
             cur = d;
         }
         for (; q < nu2; ++q) {
@@ -1221,7 +1255,7 @@ class Precond : public PrecondBase {
     template <class SR>
     aao_status inner(int B, const SR* src, long long sbs, double* out, long long obs, int transpose) {
         const long long item = (long long)h->s * h->g.nx;
-        const ArRed red = ar_red(B, item / 4 + 1);
+        const ArRed red = ar_red(B, item / 16 + 1);
         launch(k_ar_start<SR>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), item, src, sbs, red,
                ar_items());
         scale_basis<SR>(B, src, sbs, (const double*)betah, 1LL, V0, 0, nullptr);
@@ -1238,11 +1272,10 @@ class Precond : public PrecondBase {
         const Geo& g = h->g;
         const int s = h->s;
         const H2FF h2{to_ff(g.hx2), to_ff(g.hy2), to_ff(g.hz2)};
-        with_int(rows_vec(), [&](auto big) {
-            constexpr int N = decltype(big)::value ? kVN : 1;
-            const ArRed red = ar_red(B, (long long)(g.n0 / N) * g.R);
-            launch(k_schur_start<A, N>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g, h2, s,
-                   (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
+        const ArRed red = ar_red(B, g.nx);
+        with_int(g.d == 3, [&](auto d3) {
+            launch(k_schur_start<A, decltype(d3)::value>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g,
+                   h2, s, (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
         });
         scale_basis<A>(B, tbuf, g.nx, (const double*)betah, 1LL, V0, 1, stepp);
         AAO_LAUNCH_CHECK();
