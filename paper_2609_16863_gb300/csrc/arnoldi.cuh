@@ -193,6 +193,28 @@ template <class S> struct Basis {
     __device__ __forceinline__ const float* scale(int m, int b) const { return v.sc + m * srows + (long long)b * rows; }
 };
 
+// Double-float values (hi + lo, about 48 bits): error-free sums after Knuth (TAOCP 2, 4.2.2), products by one
+// fused multiply-add.
+struct FF {
+    float hi, lo;
+};
+__device__ __forceinline__ FF ff_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
+    return FF{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
+}
+// 2 P - a - b
+__device__ __forceinline__ FF ff_diff2(float P, float a, float b) {
+    const FF x = ff_sum(P, -a), y = ff_sum(P, -b), s = ff_sum(x.hi, y.hi);
+    return FF{s.hi, s.lo + (x.lo + y.lo)};
+}
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+    const FF s = ff_sum(a.hi, b.hi);
+    return FF{s.hi, s.lo + (a.lo + b.lo)};
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    return FF{p, fmaf(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi)};
+}
 // Reduction scratch of one preconditioner: nchunk blocks per item, up to nv values per block.
 struct ArRed {
     double* part;          // items * nchunk * nv
@@ -206,20 +228,39 @@ struct ArRed {
 // threads; visible to all on return): the item's state comes in the same trip to L2.
 template <int MV, class A, class F>
 __device__ __forceinline__ bool ar_reduce(const A* v, unsigned mask, const ArRed& red, double* sum, F&& preload) {
-    __shared__ double sh[kArWarps][MV];
+    // FP32 partial sums are added over the block in double-float arithmetic (FP64 adds at two per cycle and SM
+    // would take longer than the sums themselves: 45 us of k_theta_dots on 128 items of 256^2), FP64 beyond it
+    constexpr bool kFF = std::is_same<A, float>::value;
+    using SH = typename std::conditional<kFF, FF, double>::type;
+    __shared__ SH sh[kArWarps][MV];
     __shared__ bool last;
     const int w = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
 #pragma unroll
     for (int i = 0; i < MV; ++i)
         if (mask >> i & 1u) {
-            const double t = warp_sum((double)v[i]);
-            if (lane == 0) sh[w][i] = t;
+            if constexpr (kFF) {
+                FF t{v[i], 0.f};
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    t = ff_add(t, FF{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
+                if (lane == 0) sh[w][i] = t;
+            } else {
+                const double t = warp_sum(v[i]);
+                if (lane == 0) sh[w][i] = t;
+            }
         }
     __syncthreads();
     double* part = red.part + (long long)blockIdx.y * red.nchunk * MV;
     if (threadIdx.x < MV && (mask >> threadIdx.x & 1u)) {
-        double t = 0.0;
-        for (int i = 0; i < kArWarps; ++i) t += sh[i][threadIdx.x];
+        double t;
+        if constexpr (kFF) {
+            FF s = sh[0][threadIdx.x];
+            for (int i = 1; i < kArWarps; ++i) s = ff_add(s, sh[i][threadIdx.x]);
+            t = (double)s.hi + (double)s.lo;
+        } else {
+            t = 0.0;
+            for (int i = 0; i < kArWarps; ++i) t += sh[i][threadIdx.x];
+        }
         if (red.nchunk == 1) {
             sum[threadIdx.x] = t;       // the block is the item's only one
         } else {
@@ -644,28 +685,6 @@ __device__ __forceinline__ double to_fp64(float v) {
 }
 __device__ __forceinline__ double to_fp64(double v) { return v; }
 
-// Double-float values (hi + lo, about 48 bits): error-free sums after Knuth (TAOCP 2, 4.2.2), products by one
-// fused multiply-add.
-struct FF {
-    float hi, lo;
-};
-__device__ __forceinline__ FF ff_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
-    return FF{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
-}
-// 2 P - a - b
-__device__ __forceinline__ FF ff_diff2(float P, float a, float b) {
-    const FF x = ff_sum(P, -a), y = ff_sum(P, -b), s = ff_sum(x.hi, y.hi);
-    return FF{s.hi, s.lo + (x.lo + y.lo)};
-}
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-    const FF s = ff_sum(a.hi, b.hi);
-    return FF{s.hi, s.lo + (a.lo + b.lo)};
-}
-__device__ __forceinline__ FF ff_mul(FF a, FF b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    return FF{p, fmaf(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi)};
-}
 struct H2FF {
     FF x, y, z;
 };

@@ -938,9 +938,11 @@ __global__ void __launch_bounds__(kVecThreads) k_st27(LevelOp<S> op, int gs, con
         *reinterpret_cast<float4*>(o) = make_float4(res[0], res[1], res[2], res[3]);
     }
 }
-// Whether a level takes k_st27: FP32 arithmetic, rows of whole 4-column vectors with at most 32 of them.
-template <class S> inline bool st27_ok(const LevelOp<S>& op) {
-    return std::is_same<typename PT<S>::A, float>::value && !op.fine && op.g.d == 3 && op.g.n0 % 4 == 0 && op.g.n0 <= 128;
+// Whether a level takes k_st27: FP32 arithmetic, rows of whole 4-column vectors with at most 32 of them, and
+// enough points to fill the GPU with a quarter of the threads (one sweep in us, k_st27 / point per thread: 48^3 6.7 /
+// 9.3, eight items 13 / 34; 24^3 6.5 / 5.0, eight items 6.3 / 7.2; 12^3 6.6 / 4.8).
+template <class S> inline bool st27_ok(const LevelOp<S>& op, int B) {
+    return (long long)B * op.g.nx >= 1 << 16 && std::is_same<typename PT<S>::A, float>::value && !op.fine && op.g.d == 3 && op.g.n0 % 4 == 0 && op.g.n0 <= 128;
 }
 
 // x_out = x_in + P xc (x_in.d == nullptr: 0) for 16-bit storage: a thread owns 8 fine columns; each of the (one,

@@ -86,11 +86,13 @@ class Precond : public PrecondBase {
     int cl_C = 0;                  // CTAs per cluster of the single-item plan; 0: no cluster plan
     struct ClPlan {
         int C = 0;                 // CTAs per cluster; 0: none
+        int resident = 0;          // clusters on the device at once
         size_t smem = 0;
         void (*kernel)(const ClCtx<SI>, const int*, Vec<SI>, Vec<SI>) = nullptr;
         ClCtx<SI> ctx[kMaxS];      // one context per stage, passed by value
     };
-    ClPlan clp[2];                 // [0] single items, [1] batches of at least kClBatch8 items
+    static constexpr int kClPlans = 4;
+    ClPlan clp[kClPlans];          // [0] single items (16 or 8 CTAs), then batches: 8, 4 and 2 CTAs
     int* hact = nullptr;           // pinned mirror of activeh (profiling)
 
     cudaStream_t cur_stream = nullptr;     // stream of the next launch (capture stream while capturing)
@@ -510,7 +512,7 @@ class Precond : public PrecondBase {
         return global ? (ClKernel)k_cluster_mg<SI, false, true> : (ClKernel)k_cluster_mg<SI, false, false>;
     }
 
-    bool plan_cluster(int C, int deep, int lean, long long dyn_max, ClCtx<SI>& t, long long& bytes) {
+    bool plan_cluster(int C, int deep, int lean, long long dyn_max, ClCtx<SI>& t, long long& bytes, int& resident) {
         const Geo& g0 = h->g;
         const int T = L - 1;
         constexpr int VN = ClVec<A>::n;
@@ -631,10 +633,11 @@ class Precond : public PrecondBase {
             cudaGetLastError();
             return false;
         }
+        resident = nclusters;
         return true;
     }
 
-    aao_status store_cluster_plan(ClPlan& pl, const ClCtx<SI>& plan, long long bytes) {
+    aao_status store_cluster_plan(ClPlan& pl, const ClCtx<SI>& plan, long long bytes, int resident) {
         ClCtx<SI> t = plan;
         const std::vector<ClOp> prog = cl_program(t);
         ClOp* dprog;
@@ -682,12 +685,13 @@ class Precond : public PrecondBase {
         pl.C = t.C;
         pl.smem = (size_t)bytes;
         pl.kernel = cluster_kernel(t);
+        pl.resident = resident;
         return AAO_OK;
     }
 
     aao_status build_cluster(int optin) {
         cl_C = 0;
-        clp[0].C = clp[1].C = 0;
+        for (ClPlan& pl : clp) pl.C = 0;
         const Geo& g0 = h->g;
         if (g0.d != 2 || L < 2) return AAO_OK;
         long long dyn_max = optin;
@@ -703,6 +707,7 @@ class Precond : public PrecondBase {
         }
         ClCtx<SI> t;
         long long bytes = 0;
+        int resident = 0;
         // FP64 arithmetic is too slow for redundant rows; else the deepest ghost regions that fit, before
         // staging less
         const int deepest = std::is_same<A, double>::value ? 0 : 2;
@@ -710,7 +715,7 @@ class Precond : public PrecondBase {
             for (int lo = 0; lo <= 2; lo += 2)          // lean 0 and 1 for every depth, then 2 and 3
                 for (int deep = deepest; deep >= 0; --deep)
                     for (int lean = lo; lean <= lo + 1; ++lean)
-                        if (plan_cluster(C, deep, lean, dyn_max, t, bytes)) return true;
+                        if (plan_cluster(C, deep, lean, dyn_max, t, bytes, resident)) return true;
             return false;
         };
         if (!find(16) && !find(8)) return AAO_OK;
@@ -723,9 +728,14 @@ class Precond : public PrecondBase {
             }
         }
         AAO_LAUNCH_CHECK();
-        AAO_TRY(store_cluster_plan(clp[0], t, bytes));
+        AAO_TRY(store_cluster_plan(clp[0], t, bytes, resident));
         if (clp[0].C == 8) clp[1] = clp[0];
-        else if (find(8)) AAO_TRY(store_cluster_plan(clp[1], t, bytes));
+        else if (find(8)) AAO_TRY(store_cluster_plan(clp[1], t, bytes, resident));
+        // 16-bit storage keeps to its two plans: its larger batches round intermediates as the level kernels do
+        if constexpr (!PT<SI>::scaled) {
+            if (find(4)) AAO_TRY(store_cluster_plan(clp[2], t, bytes, resident));
+            if (find(2)) AAO_TRY(store_cluster_plan(clp[3], t, bytes, resident));
+        }
         cl_C = clp[0].C;
         return AAO_OK;
     }
@@ -836,7 +846,7 @@ class Precond : public PrecondBase {
             }
         }
         if constexpr (std::is_same<A, float>::value) {
-            if (st27_ok(op)) {
+            if (st27_ok(op, B)) {
                 const int gs = row_group(op.g.n0, 4);
                 const dim3 gr = row_group_grid<SI>(op.g, 4, B);
                 if (x.d) launch(k_st27<SI, 0>, gr, kVecThreads, 0, st(), op, gs, act, x, b, out, om);
@@ -883,7 +893,7 @@ class Precond : public PrecondBase {
             }
         }
         if constexpr (std::is_same<A, float>::value) {
-            if (st27_ok(op) && x.d) {
+            if (st27_ok(op, B) && x.d) {
                 launch(k_st27<SI, 2>, row_group_grid<SI>(op.g, 4, B), kVecThreads, 0, st(), op, row_group(op.g.n0, 4), act, x,
                        b, out, A(0));
                 return;
@@ -1045,10 +1055,46 @@ class Precond : public PrecondBase {
         return AAO_OK;
     }
 
+    // The cluster plan of a batch, or null: the level kernels.  16-bit storage: 8 CTAs per item from kClBatch8
+    // items on, up to kClMaxBatch items.  Else the plan with the least waves of resident clusters times the time
+    // of a launch, unless the level kernels are faster.  Measured (us per three V-cycles with their share of the
+    // Krylov kernels, B items; level kernels / 16 / 8 / 4 / 2 CTAs per item):
+    //   FP32 128^2, B = 1: 275 / 62 / 65 / 71 / 94; B = 64: 574 / 465 / 264 / 143 / 116
+    //   FP32 64^2, B = 64: 209 / 322 / 166 / 83 / 60; 256^2, B = 128: 939 / 1390 / 949 / - / -
+    //   FP64 64^2, B = 32: 615 / 310 / 221 / 122 / 177; 256^2, B = 128: 5431 / 5602 / - / - / -
+    // The model: a launch takes 22 + 14 T us on T distributed levels and 5.5 us per 1000 points of a CTA's rows
+    // beyond 2500 (FP64: 20 + 25 T and 50 us per 1000 beyond 400); the level kernels 0.105 us per 1000 points
+    // (FP64: 0.62) and 150 us per 148 items.  It reproduces the figures above to about 15%; the level kernels are
+    // taken unless a plan is faster by 10%.
+    const ClPlan* pick_cluster(int B) const {
+        if (cl_C == 0) return nullptr;
+        if constexpr (PT<SI>::scaled) {
+            if (B > kClMaxBatch) return nullptr;
+            return B >= kClBatch8 && clp[1].C > 0 ? &clp[1] : &clp[0];
+        }
+        const bool f64 = std::is_same<A, double>::value;
+        const double nx = (double)h->g.nx;
+        const double levels = (f64 ? 0.62e-3 : 0.105e-3) * nx * B + 150.0 * ((B + 147) / 148);
+        const ClPlan* best = nullptr;
+        double cost = B > kClMaxBatch ? 0.9 * levels : 1e300;
+        for (const ClPlan& pl : clp) {
+            if (pl.C == 0) continue;
+            const double per = nx / pl.C;
+            const double t = f64 ? 20.0 + 25.0 * (L - 1) + 50e-3 * std::max(0.0, per - 400.0)
+                                 : 22.0 + 14.0 * (L - 1) + 5.5e-3 * std::max(0.0, per - 2500.0);
+            const double c = t * ((B + pl.resident - 1) / pl.resident);
+            if (c < cost) {
+                cost = c;
+                best = &pl;
+            }
+        }
+        return best;
+    }
+
     aao_status mg_solve(int stage, int B, const int* act, Vec<SI> b, Vec<SI> out) {
-        if (B <= kClMaxBatch && cl_C > 0) {
+        if (const ClPlan* plan = pick_cluster(B)) {
             // one cluster per item: small batches (single time steps, MGRIT's batched steps)
-            const ClPlan& pl = B >= kClBatch8 && clp[1].C > 0 ? clp[1] : clp[0];
+            const ClPlan& pl = *plan;
             bytes_hint(2.0 * nact * h->g.nx * sizeof(SI));
             launch_cluster(pl.kernel, dim3((unsigned)(pl.C * B)), dim3(kClThreads), pl.smem, st(), pl.C,
                            pl.ctx[stage], act, b, out);
@@ -1272,7 +1318,7 @@ class Precond : public PrecondBase {
         const Geo& g = h->g;
         const int s = h->s;
         const H2FF h2{to_ff(g.hx2), to_ff(g.hy2), to_ff(g.hz2)};
-        const ArRed red = ar_red(B, g.nx);
+        const ArRed red = ar_red(B, g.nx / 4 + 1);        // four points per thread: the reduction is the larger part
         with_int(g.d == 3, [&](auto d3) {
             launch(k_schur_start<A, decltype(d3)::value>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g,
                    h2, s, (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
