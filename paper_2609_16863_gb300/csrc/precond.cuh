@@ -856,21 +856,24 @@ class Precond : public PrecondBase {
         }
         launch_smooth_rows(kind, grid, block, op, pm, B, act, x, b, out, om);
     }
-    template <class... Args> void launch_smooth_rows(int kind, dim3 grid, dim3 block, Args... args) {
+    // Large 2D batches take four rows per thread, a column each (grid.y = items), where a block spans the row; wider
+    // rows (more than kPtMaxThreads columns) take the kernels that walk over their columns.
+    static bool rows_ok(dim3 grid, dim3 block, const Geo& g) { return grid.y >= 16 && (int)block.x >= g.n0; }
+    template <class... Args> void launch_smooth_rows(int kind, dim3 grid, dim3 block, const LevelOp<SI>& op,
+                                                          Args... args) {
         if constexpr (!PT<SI>::scaled) {
-            // large 2D batches: four rows per thread (grid.y = items)
             constexpr int kRows = 4;
-            if ((kind == 4 || kind == 2) && grid.y >= 16) {
+            if ((kind == 4 || kind == 2) && rows_ok(grid, block, op.g)) {
                 dim3 gr((grid.x + kRows - 1) / kRows, grid.y);
-                if (kind == 4) launch(k_smooth_rows<SI, 4, kRows>, gr, block, 0, st(), args...);
-                else launch(k_smooth_rows<SI, 2, kRows>, gr, block, 0, st(), args...);
+                if (kind == 4) launch(k_smooth_rows<SI, 4, kRows>, gr, block, 0, st(), op, args...);
+                else launch(k_smooth_rows<SI, 2, kRows>, gr, block, 0, st(), op, args...);
                 return;
             }
         }
-        if (kind == 4) launch(k_smooth<SI, 4>, grid, block, 0, st(), args...);
-        else if (kind == 2) launch(k_smooth<SI, 2>, grid, block, 0, st(), args...);
-        else if (kind == 3) launch(k_smooth<SI, 3>, grid, block, 0, st(), args...);
-        else launch(k_smooth<SI, 0>, grid, block, 0, st(), args...);
+        if (kind == 4) launch(k_smooth<SI, 4>, grid, block, 0, st(), op, args...);
+        else if (kind == 2) launch(k_smooth<SI, 2>, grid, block, 0, st(), op, args...);
+        else if (kind == 3) launch(k_smooth<SI, 3>, grid, block, 0, st(), op, args...);
+        else launch(k_smooth<SI, 0>, grid, block, 0, st(), op, args...);
     }
     void launch_residual(int kind, dim3 grid, dim3 block, const LevelOp<SI>& op, const PtMap& pm, int B,
                          const int* act, Vec<SI> x, Vec<SI> b, Vec<SI> out) {
@@ -921,26 +924,27 @@ class Precond : public PrecondBase {
                        xc, x, out);
                 return;
             }
-        } else if (gf.d == 2 && B >= 16) {
+        } else if (gf.d == 2 && rows_ok(pbl, pth, gf)) {
             launch(k_prolong_add_rows<SI, 4>, dim3((pbl.x + 3) / 4, pbl.y), pth, 0, st(), gf, gc, pm, B, act, xc, x, out);
             return;
         }
         launch(k_prolong_add<SI>, pbl, pth, 0, st(), gf, gc, pm, B, act, xc, x, out);
     }
-    template <class... Args> void launch_residual_rows(int kind, dim3 grid, dim3 block, Args... args) {
+    template <class... Args> void launch_residual_rows(int kind, dim3 grid, dim3 block, const LevelOp<SI>& op,
+                                                            Args... args) {
         if constexpr (!PT<SI>::scaled) {
             constexpr int kRows = 4;
-            if ((kind == 4 || kind == 2) && grid.y >= 16) {
+            if ((kind == 4 || kind == 2) && rows_ok(grid, block, op.g)) {
                 dim3 gr((grid.x + kRows - 1) / kRows, grid.y);
-                if (kind == 4) launch(k_residual_rows<SI, 4, kRows>, gr, block, 0, st(), args...);
-                else launch(k_residual_rows<SI, 2, kRows>, gr, block, 0, st(), args...);
+                if (kind == 4) launch(k_residual_rows<SI, 4, kRows>, gr, block, 0, st(), op, args...);
+                else launch(k_residual_rows<SI, 2, kRows>, gr, block, 0, st(), op, args...);
                 return;
             }
         }
-        if (kind == 4) launch(k_residual<SI, 4>, grid, block, 0, st(), args...);
-        else if (kind == 2) launch(k_residual<SI, 2>, grid, block, 0, st(), args...);
-        else if (kind == 3) launch(k_residual<SI, 3>, grid, block, 0, st(), args...);
-        else launch(k_residual<SI, 0>, grid, block, 0, st(), args...);
+        if (kind == 4) launch(k_residual<SI, 4>, grid, block, 0, st(), op, args...);
+        else if (kind == 2) launch(k_residual<SI, 2>, grid, block, 0, st(), op, args...);
+        else if (kind == 3) launch(k_residual<SI, 3>, grid, block, 0, st(), op, args...);
+        else launch(k_residual<SI, 0>, grid, block, 0, st(), op, args...);
     }
 
     // x_out = V-cycle(l) applied to (x_in, b); x_in.d == nullptr: zero guess.
