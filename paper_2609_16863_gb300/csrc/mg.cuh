@@ -1294,6 +1294,116 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_prolong_add_rows(Geo gf, Geo 
     }
 }
 
+// Transfers of batched 2D levels in unscaled storage, a 16-byte vector of columns per thread; per point the sums of
+// k_prolong_add and k_restrict in their order.  Bound by memory; a point per
+// thread and row spent its time on indices and weights (33 us for the interpolation to 128 items of 256^2, where
+// its traffic takes about 12).  With both, the FP32 solve on 256^2 with 128 items went from 288.8 to 280.4 ms.
+// Interpolation: the fine rows 2J and 2J + 1 share their coarse rows J - 1 and J.
+template <class S>
+__global__ void __launch_bounds__(kVecThreads) k_prolong2d(Geo gf, Geo gc, const int* active, Vec<S> xcv, Vec<S> xin,
+                                                           Vec<S> xout) {
+    pdl_prologue();
+    static_assert(!PT<S>::scaled, "unscaled storage only");
+    using VT = typename Vec16<S>::T;
+    constexpr int V = Vec16<S>::n, C = V / 2;
+    const int b = blockIdx.y;
+    if (active && !active[b]) return;
+    const int n0 = gf.n0, tpr = n0 / V;
+    const int q = blockIdx.x * kVecThreads + threadIdx.x;
+    const int J = q / tpr, c0 = (q - J * tpr) * V, cc = c0 / 2;
+    if (2 * J >= gf.n1) return;
+    const S* Xc = xcv.d + (long long)b * xcv.bs;
+    S lo[C + 2], hi[C + 2];                       // coarse rows J - 1 and J, columns cc - 1 .. cc + C
+#pragma unroll
+    for (int t = 0; t < C + 2; ++t) {
+        const int I = cc - 1 + t;
+        const bool in = I >= 0 && I < gc.n0;
+        lo[t] = in && J > 0 ? Xc[(J - 1) * gc.n0 + I] : S(0);
+        hi[t] = in && J < gc.n1 ? Xc[J * gc.n0 + I] : S(0);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int row = 2 * J + r;
+        if (row >= gf.n1) continue;
+        S x[V];
+        if (xin.d) {
+            const VT v = *reinterpret_cast<const VT*>(xin.d + (long long)b * xin.bs + row * n0 + c0);
+            const S* e = reinterpret_cast<const S*>(&v);
+#pragma unroll
+            for (int t = 0; t < V; ++t) x[t] = e[t];
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; ++t) x[t] = S(0);
+        }
+        const S w = r == 0 ? S(0.5) : S(1), h = S(0.5) * w;
+#pragma unroll
+        for (int t = 0; t < C; ++t) {
+            if (r == 0) {
+                x[2 * t] += h * lo[t];
+                x[2 * t] += h * lo[t + 1];
+                x[2 * t + 1] += w * lo[t + 1];
+            }
+            x[2 * t] += h * hi[t];
+            x[2 * t] += h * hi[t + 1];
+            x[2 * t + 1] += w * hi[t + 1];
+        }
+        VT o;
+        S* e = reinterpret_cast<S*>(&o);
+#pragma unroll
+        for (int t = 0; t < V; ++t) e[t] = x[t];
+        *reinterpret_cast<VT*>(xout.d + (long long)b * xout.bs + row * n0 + c0) = o;
+    }
+}
+
+// Restriction: V / 2 coarse columns per thread (one vector and the column after it of three fine rows).
+template <class S>
+__global__ void __launch_bounds__(kVecThreads) k_restrict2d(Geo gf, Geo gc, const int* active, Vec<S> rv, Vec<S> bcv) {
+    pdl_prologue();
+    static_assert(!PT<S>::scaled, "unscaled storage only");
+    using VT = typename Vec16<S>::T;
+    constexpr int V = Vec16<S>::n, C = V / 2;
+    const int b = blockIdx.y;
+    if (active && !active[b]) return;
+    const int n0 = gf.n0, tpr = n0 / V;
+    const int q = blockIdx.x * kVecThreads + threadIdx.x;
+    const int J = q / tpr, f0 = (q - J * tpr) * V;
+    if (J >= gc.n1) return;
+    const S* R = rv.d + (long long)b * rv.bs;
+    S v[3][V + 1];
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+        const int row = 2 * J + y;
+        const bool in = row < gf.n1;
+        if (in) {
+            const VT u = *reinterpret_cast<const VT*>(R + row * n0 + f0);
+            const S* e = reinterpret_cast<const S*>(&u);
+#pragma unroll
+            for (int t = 0; t < V; ++t) v[y][t] = e[t];
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; ++t) v[y][t] = S(0);
+        }
+        v[y][V] = in && f0 + V < n0 ? R[row * n0 + f0 + V] : S(0);
+    }
+#pragma unroll
+    for (int t = 0; t < C; ++t) {
+        S acc = S(0);
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const S w = y == 1 ? S(1) : S(0.5), h = S(0.5) * w;
+            acc += h * v[y][2 * t];
+            acc += w * v[y][2 * t + 1];
+            acc += h * v[y][2 * t + 2];
+        }
+        bcv.d[(long long)b * bcv.bs + J * gc.n0 + f0 / 2 + t] = acc;
+    }
+}
+// Whether batched 2D transfers take the vector kernels: rows of whole 16-byte vectors (their items then start on
+// 16-byte boundaries too), and items enough to fill the chip with vectors instead of points.
+template <class S> inline bool transfer2d_ok(const Geo& gf, int B) {
+    return !PT<S>::scaled && gf.d == 2 && B >= 16 && gf.n0 % (16 / (int)sizeof(S)) == 0;
+}
+
 // x_out = xp + omega D^{-1} (b - A xp) with xp = x_in + P xc computed on the fly at
 // the point and its stencil neighbours (prolongation fused with one sweep).
 template <class S>

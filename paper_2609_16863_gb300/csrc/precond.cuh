@@ -912,6 +912,14 @@ class Precond : public PrecondBase {
                 return;
             }
         }
+        if constexpr (!PT<SI>::scaled) {
+            if (transfer2d_ok<SI>(gf, B)) {
+                const long long pos = (long long)(gf.n0 / (16 / (int)sizeof(SI))) * gc.n1;
+                launch(k_restrict2d<SI>, dim3((unsigned)((pos + kVecThreads - 1) / kVecThreads), (unsigned)B), kVecThreads, 0,
+                       st(), gf, gc, act, r, bc);
+                return;
+            }
+        }
         const PtMap pmc = ptmap(gc.n0);
         launch(k_restrict<SI>, pt_grid(pmc, gc.R, B), pt_block(pmc), 0, st(), gf, gc, pmc, B, act, r, bc);
     }
@@ -924,6 +932,11 @@ class Precond : public PrecondBase {
                        xc, x, out);
                 return;
             }
+        } else if (transfer2d_ok<SI>(gf, B)) {
+            const long long pos = (long long)(gf.n0 / (16 / (int)sizeof(SI))) * ((gf.n1 + 1) / 2);
+            launch(k_prolong2d<SI>, dim3((unsigned)((pos + kVecThreads - 1) / kVecThreads), (unsigned)B), kVecThreads, 0, st(),
+                   gf, gc, act, xc, x, out);
+            return;
         } else if (gf.d == 2 && rows_ok(pbl, pth, gf)) {
             launch(k_prolong_add_rows<SI, 4>, dim3((pbl.x + 3) / 4, pbl.y), pth, 0, st(), gf, gc, pm, B, act, xc, x, out);
             return;
