@@ -650,11 +650,14 @@ def main():
             short = name
             for tok in ("k_strip2dIfLi0", "k_strip2dIfLi1", "k_strip2dIfLi2", "k_strip2dIdLi0", "k_strip2dIdLi1",
                         "k_strip2dIdLi2", "k_cluster_mg", "k_vcycle_tail", "k_smooth2", "k_smooth_rows", "k_smooth", "k_resid_restrict",
-                        "k_residual_rows", "k_residual", "k_restrict", "k_prolong_smooth", "k_prolong_add_rows",
-                        "k_prolong_add", "k_coarse_solve", "k_rana_rhs", "k_theta", "k_mgs", "k_norm", "k_scale_store",
-                        "k_combine", "k_matvec", "k_givens", "k_hess_solve", "k_schur_update_b", "k_schur_update",
-                        "k_schur_rhs_b", "k_schur_rhs", "k_schurT", "k_schur_g", "k_mgrit_cpoints", "k_inner_init",
-                        "k_count_its", "k_step_add", "k_step_set", "k_outer_init", "k_rhs", "k_load"):
+                        "k_residual_rows", "k_residual", "k_restrict2d", "k_restrict16", "k_restrict", "k_prolong_smooth",
+                        "k_prolong_add_rows",
+                        "k_prolong_add", "k_prolong2d", "k_prolong16", "k_st27",
+                        "k_coarse_solve", "k_rana_vec", "k_rana_pt", "k_rana_rhs", "k_theta_dots", "k_arnoldi_upd",
+                        "k_ar_start", "k_scale_vec", "k_combine_vec", "k_mgs", "k_norm", "k_scale_store",
+                        "k_combine", "k_matvec", "k_givens", "k_hess_solve", "k_schur_start", "k_schur_finish",
+                        "k_schurT", "k_schur_g", "k_mgrit_cpoints", "k_step_add", "k_step_set", "k_outer_init",
+                        "k_rhs", "k_load"):
                 if tok in name:
                     short = tok
                     break
@@ -702,7 +705,7 @@ def main():
                      "achieved": ach_model, "frac": ach_model / peak, "algorithmic_bytes_per_launch": model,
                      "bytes_model": "method-level: 3 V-cycles x (22 + 9/4) n_x b_p per item",
                      "items_per_launch": items,
-                     "limit": "latency: cluster barriers and dependent step chains per V-cycle (16 SMs per item)"})
+                     "limit": "latency: cluster barriers and dependent step chains per V-cycle (2 to 16 SMs per item)"})
         roof["traffic"] = profile_traffic("k_cluster_mg_fd2d_n256", f"{args.prec} per item")
         if roof["traffic"] is not None:
             roof["traffic"] *= items

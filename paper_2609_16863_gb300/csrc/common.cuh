@@ -362,14 +362,6 @@ __device__ __forceinline__ typename PT<S>::A op_K(const View<S>& u, const Geo& g
     return fd_K(u, g, op.faces, row, j, k, c);
 }
 
-template <class S, class T>
-__device__ __forceinline__ typename PT<S>::A op_M(const View<S>& u, const Geo& g, const SpaceOp<T>& op,
-                                                  long long row, int j, int k, int c) {
-    using A = typename PT<S>::A;
-    if (op.q1) return q1_apply(u, g, op.q, row, j, k, c, A(1), A(0));
-    return A(u.at(row, c));
-}
-
 // Diagonal of K at a point.
 template <class A, class T>
 __device__ __forceinline__ A fd_K_diag(const Geo& g, const Faces<T>& f, long long row, int j, int k, int c) {

@@ -1669,7 +1669,7 @@ __global__ void __launch_bounds__(kT3Threads) k_prolong_smooth_tile(LevelOp<S> o
     }
     __syncthreads();
     const T3Rows<A> u{xp, W1, j0 - 1, k0 - 1, n0};
-    A val[(kMaxRowLen + kWarp - 1) / kWarp > 4 ? 4 : 4];
+    A val[4];
     for (int r = wp; r < kT3 * kT3; r += kT3Warps) {
         const int j = j0 + r % kT3, k = k0 + r / kT3;
         const bool in = j < g.n1 && k < g.n2;
