@@ -1297,7 +1297,8 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_prolong_add_rows(Geo gf, Geo 
 // Transfers of batched 2D levels in unscaled storage, a 16-byte vector of columns per thread; per point the sums of
 // k_prolong_add and k_restrict in their order.  Bound by memory; a point per
 // thread and row spent its time on indices and weights (33 us for the interpolation to 128 items of 256^2, where
-// its traffic takes about 12).  With both, the FP32 solve on 256^2 with 128 items went from 288.8 to 280.4 ms.
+// its traffic takes about 12; now 13 us on average over that level and the next, and 10 us for the restriction, both with
+// the events' overhead).  With both, the FP32 solve on 256^2 with 128 items went from 288.8 to 280.4 ms.
 // Interpolation: the fine rows 2J and 2J + 1 share their coarse rows J - 1 and J.
 template <class S>
 __global__ void __launch_bounds__(kVecThreads) k_prolong2d(Geo gf, Geo gc, const int* active, Vec<S> xcv, Vec<S> xin,
