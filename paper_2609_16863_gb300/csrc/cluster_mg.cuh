@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_mg(const __grid_const
             const int r = cl_div(i, t.magicv[0]), c = (i - r * nvp) * VN, row = a + r - H;
             A* d = B + r * ld + c;
             const bool in = row >= 0 && row < n1;
-            if (in && vec) {
+            if (in && vec && c < n0) {      // (rows of n0 = VN columns are padded to two vectors)
                 cp_async16(d, src + (long long)row * n0 + c);
                 continue;
             }
@@ -929,6 +929,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_mg(const __grid_const
             const bool vec = v.n0 % VN == 0;
             for (int i = tid; i < v.nr * v.nvp; i += nthr) {
                 const int r = cl_div(i, v.magicv), c = (i - r * v.nvp) * VN;
+                if (c >= v.n0) continue;              // a vector of padding columns
                 const A* x = sm + v.X + k * v.xs + r * v.ld + c;
                 A* d = reinterpret_cast<A*>(o) + r * v.n0 + c;
                 if (vec) {

@@ -597,7 +597,7 @@ class Precond : public PrecondBase {
             const bool fd = l == 0 && fine0;
             if (!fd) {
                 t.sten_global[l] = l >= 1 && (lean >= 3 || (lean == 2 && l == 1)) ? 1 : 0;
-                if (t.sten_global[l] && lev[l].g.n0 % VN != 0) return false;     // read as whole vectors
+                if (t.sten_global[l] && lev[l].g.n0 != np) return false;     // read as whole vectors of the padded row
                 if (!t.sten_global[l]) t.soff[l] = take(9LL * (t.maxr[l] + 2 * (t.H[l] - 1)) * np);
             }
             if (!fd || faces) t.woff[l] = take((long long)(t.maxr[l] + 2 * t.H[l]) * np);
