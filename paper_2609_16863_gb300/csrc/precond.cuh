@@ -642,7 +642,9 @@ class Precond : public PrecondBase {
         const std::vector<ClOp> prog = cl_program(t);
         ClOp* dprog;
         AAO_TRY(ar.alloc(&dprog, prog.size()));
-        AAO_CUDA_TRY(cudaMemcpy(dprog, prog.data(), sizeof(ClOp) * prog.size(), cudaMemcpyHostToDevice));
+        // on the stream of the images' kernel, which reads it (a copy on the legacy stream from pageable memory may
+        // end after the call, unordered with a non-blocking stream)
+        AAO_CUDA_TRY(cudaMemcpyAsync(dprog, prog.data(), sizeof(ClOp) * prog.size(), cudaMemcpyHostToDevice, st()));
         for (int i = 0; i < h->s; ++i) {
             ClCtx<SI>& q = pl.ctx[i];
             q = t;
@@ -682,6 +684,7 @@ class Precond : public PrecondBase {
             q.img = img;
             if (dpad) q.Dinv = dpad;
         }
+        AAO_CUDA_TRY(cudaStreamSynchronize(st()));       // prog is read until here
         pl.C = t.C;
         pl.smem = (size_t)bytes;
         pl.kernel = cluster_kernel(t);
