@@ -224,10 +224,17 @@ __global__ void __launch_bounds__(kPtMaxThreads) k_resid_restrict(LevelOp<S> op,
     });
 }
 
+// Whether offsets into a 3D level's 27 stencil components fit 32 bits (they pass 2^31 from 79.6 million points on).  The kernels
+// that load every component of a point at once take such levels only: 64-bit offsets cost the 96^3 BF16 solve 2.9% and
+// the 47 x 39 x 43 FP16 one 3.1%.  Larger levels take the kernels whose offsets are 64-bit.
+constexpr bool sten32_ok(long long nx) { return 27 * nx <= 2147483647LL; }
+
 // Level kinds known at compile time (fewer registers than the run-time dispatch of level_apply):
 // 0 any, 1 matrix-free FD level, 2 stored 9-point (2D), 3 stored 27-point (3D),
 // 4: matrix-free FD level in 2D.
-inline int level_kind(int fine, int d) { return fine ? (d == 2 ? 4 : 1) : (d == 2 ? 2 : 3); }
+inline int level_kind(int fine, int d, long long nx) {
+    return fine ? (d == 2 ? 4 : 1) : (d == 2 ? 2 : (sten32_ok(nx) ? 3 : 0));
+}
 
 template <int KIND, class S, class SU>
 __device__ __forceinline__ void level_apply_k(const LevelOp<S>& op, const View<SU>& u, long long row, int j, int k,
@@ -276,8 +283,8 @@ __device__ __forceinline__ void level_apply_k(const LevelOp<S>& op, const View<S
         Au = acc;
         diag = sten_coef(op, 4, p);
     } else if constexpr (KIND == 3) {
-        // stored 27-point stencil: every load is issued before the sum (a point outside the grid adds an exact
-        // zero where level_apply skips it)
+        // stored 27-point stencil, 32-bit offsets (sten32_ok): every load is issued before the sum (a point outside the
+        // grid adds an exact zero where level_apply skips it)
         const unsigned nx = (unsigned)g.nx, p = (unsigned)row * g.n0 + c;
         const bool xm = c > 0, xp = c + 1 < g.n0;
         A v[27];
@@ -938,11 +945,12 @@ __global__ void __launch_bounds__(kVecThreads) k_st27(LevelOp<S> op, int gs, con
         *reinterpret_cast<float4*>(o) = make_float4(res[0], res[1], res[2], res[3]);
     }
 }
-// Whether a level takes k_st27: FP32 arithmetic, rows of whole 4-column vectors with at most 32 of them, and
+// Whether a level takes k_st27: FP32 arithmetic, 32-bit offsets, rows of whole 4-column vectors with at most 32 of them, and
 // enough points to fill the GPU with a quarter of the threads (one sweep in us, k_st27 / point per thread: 48^3 6.7 /
 // 9.3, eight items 13 / 34; 24^3 6.5 / 5.0, eight items 6.3 / 7.2; 12^3 6.6 / 4.8).
 template <class S> inline bool st27_ok(const LevelOp<S>& op, int B) {
-    return (long long)B * op.g.nx >= 1 << 16 && std::is_same<typename PT<S>::A, float>::value && !op.fine && op.g.d == 3 && op.g.n0 % 4 == 0 && op.g.n0 <= 128;
+    return (long long)B * op.g.nx >= 1 << 16 && std::is_same<typename PT<S>::A, float>::value && !op.fine && op.g.d == 3 &&
+           op.g.n0 % 4 == 0 && op.g.n0 <= 128 && sten32_ok(op.g.nx);
 }
 
 // x_out = x_in + P xc (x_in.d == nullptr: 0) for 16-bit storage: a thread owns 8 fine columns; each of the (one,

@@ -1027,7 +1027,7 @@ class Precond : public PrecondBase {
         for (; q < nu1; ++q) {
             Vec<SI> d = dest();
             bytes_hint((cur.d ? 3.0 : 2.0) * nact * g.nx * sizeof(SI));
-            launch_smooth(level_kind(op.fine, g.d), pbl, pth, op, pm, B, act, cur, b, d, om);
+            launch_smooth(level_kind(op.fine, g.d, g.nx), pbl, pth, op, pm, B, act, cur, b, d, om);
             cur = d;
         }
         // residual and restriction
@@ -1042,7 +1042,7 @@ class Precond : public PrecondBase {
             launch_restrict(g, gc, B, act, b, lev[l + 1].Bb);
         } else {
             bytes_hint(3.0 * nact * g.nx * sizeof(SI));
-            launch_residual(level_kind(op.fine, g.d), pbl, pth, op, pm, B, act, cur, b, lev[l].Rr);
+            launch_residual(level_kind(op.fine, g.d, g.nx), pbl, pth, op, pm, B, act, cur, b, lev[l].Rr);
             bytes_hint(1.0 * nact * (g.nx + gc.nx) * sizeof(SI));
             launch_restrict(g, gc, B, act, lev[l].Rr, lev[l + 1].Bb);
         }
@@ -1068,7 +1068,7 @@ class Precond : public PrecondBase {
         for (; q < nu2; ++q) {
             Vec<SI> d = dest();
             bytes_hint(3.0 * nact * g.nx * sizeof(SI));
-            launch_smooth(level_kind(op.fine, g.d), pbl, pth, op, pm, B, act, cur, b, d, om);
+            launch_smooth(level_kind(op.fine, g.d, g.nx), pbl, pth, op, pm, B, act, cur, b, d, om);
             cur = d;
         }
         AAO_LAUNCH_CHECK();
