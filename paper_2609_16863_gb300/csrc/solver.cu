@@ -388,7 +388,10 @@ static aao_status setup_handle(Handle* h, const aao_grid* grid, double tau, int 
         long long nnode = (long long)(g.n0 + 2) * (g.n1 + 2) * (g.d == 3 ? g.n2 + 2 : 1);
         double* kap;
         AAO_TRY(ar.alloc(&kap, nnode));
+        // on the legacy stream, behind the kernels there that made kappa; a copy between device arrays may end after the
+        // call, and nothing orders a non-blocking stream of the handle behind it
         AAO_CUDA_TRY(cudaMemcpy(kap, grid->kappa, sizeof(double) * nnode, cudaMemcpyDefault));
+        AAO_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
         long long nfx = (long long)(g.n0 + 1) * g.R;
         long long nfy = (long long)g.n0 * (g.n1 + 1) * g.n2;
         long long nfz = g.d == 3 ? (long long)g.n0 * g.n1 * (g.n2 + 1) : 0;

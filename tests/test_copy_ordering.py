@@ -20,3 +20,9 @@ def test_preconditioner_copies_run_on_its_stream():
     body = body[:body.index("aao_status build_cluster")]
     copy, image = body.index("cudaMemcpyAsync(dprog"), body.index("k_cluster_image")
     assert copy < image < body.rindex("cudaStreamSynchronize(st())")
+
+
+def test_kappa_has_arrived_before_the_faces_are_formed():
+    text = _source("solver.cu")
+    copy, faces = text.index("cudaMemcpy(kap, grid->kappa"), text.index("launch(k_faces")
+    assert copy < text.index("cudaStreamSynchronize(cudaStreamLegacy)", copy) < faces
