@@ -222,51 +222,59 @@ struct ArRed {
     int nchunk;
 };
 
+// float -> double by integer operations (an FP64 conversion costs as much as an FP64 operation).
+__device__ __forceinline__ double to_fp64(float v) {
+    const unsigned u = __float_as_uint(v), e = u >> 23 & 255u;
+    if (e - 1u >= 254u) return (double)v;                     // zero, subnormal, infinity, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (e + 896u) << 20 | (u >> 3 & 0xfffffu)), (int)(u << 29));
+}
+__device__ __forceinline__ double to_fp64(double v) { return v; }
+
 // Sum the values chosen by `mask` over the blocks of item blockIdx.y: the last block to arrive has the
 // sums in sum[] (shared memory) and gets true.  Partial sums are added in chunk order, so the result does
 // not depend on scheduling.  preload() runs in that block beside the loads of the partial sums (all
 // threads; visible to all on return): the item's state comes in the same trip to L2.
 template <int MV, class A, class F>
 __device__ __forceinline__ bool ar_reduce(const A* v, unsigned mask, const ArRed& red, double* sum, F&& preload) {
-    // FP32 partial sums are added over the block in double-float arithmetic (FP64 adds at two per cycle and SM
-    // would take longer than the sums themselves: 45 us of k_theta_dots on 128 items of 256^2), FP64 beyond it
-    constexpr bool kFF = std::is_same<A, float>::value;
-    using SH = typename std::conditional<kFF, FF, double>::type;
-    __shared__ SH sh[kArWarps][MV];
+    // FP64 adds run at two per cycle and SM, and summing each value by shuffles in every warp would take longer than
+    // the launch's other work (37 us of them in k_theta_dots on 128 items of 256^2): so the threads' FP32 values meet in
+    // shared memory and one warp per value adds four per lane before its shuffles, 8 adds per value instead of 23.
+    constexpr bool kF32 = std::is_same<A, float>::value;
+    __shared__ A sh[MV][kF32 ? kArThreads : kArWarps];
     __shared__ bool last;
     const int w = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
 #pragma unroll
     for (int i = 0; i < MV; ++i)
         if (mask >> i & 1u) {
-            if constexpr (kFF) {
-                FF t{v[i], 0.f};
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-                    t = ff_add(t, FF{__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o)});
-                if (lane == 0) sh[w][i] = t;
+            if constexpr (kF32) {
+                sh[i][threadIdx.x] = v[i];
             } else {
                 const double t = warp_sum(v[i]);
-                if (lane == 0) sh[w][i] = t;
+                if (lane == 0) sh[i][w] = t;
             }
         }
     __syncthreads();
     double* part = red.part + (long long)blockIdx.y * red.nchunk * MV;
-    if (threadIdx.x < MV && (mask >> threadIdx.x & 1u)) {
-        double t;
-        if constexpr (kFF) {
-            FF s = sh[0][threadIdx.x];
-            for (int i = 1; i < kArWarps; ++i) s = ff_add(s, sh[i][threadIdx.x]);
-            t = (double)s.hi + (double)s.lo;
-        } else {
-            t = 0.0;
-            for (int i = 0; i < kArWarps; ++i) t += sh[i][threadIdx.x];
-        }
+    auto put = [&](int i, double t) {
         if (red.nchunk == 1) {
-            sum[threadIdx.x] = t;       // the block is the item's only one
+            sum[i] = t;                 // the block is the item's only one
         } else {
-            part[(long long)blockIdx.x * MV + threadIdx.x] = t;
+            part[(long long)blockIdx.x * MV + i] = t;
             __threadfence();
         }
+    };
+    if constexpr (kF32) {
+        for (int i = w; i < MV; i += kArWarps) {
+            if (!(mask >> i & 1u)) continue;
+            static_assert(kArThreads == 4 * kWarp, "four values per lane");
+            const A* s = sh[i] + lane;
+            const double t = warp_sum((to_fp64(s[0]) + to_fp64(s[kWarp])) + (to_fp64(s[2 * kWarp]) + to_fp64(s[3 * kWarp])));
+            if (lane == 0) put(i, t);
+        }
+    } else if (threadIdx.x < MV && (mask >> threadIdx.x & 1u)) {
+        double t = 0.0;
+        for (int i = 0; i < kArWarps; ++i) t += sh[threadIdx.x][i];
+        put(threadIdx.x, t);
     }
     if (red.nchunk == 1) {
         preload();
@@ -671,12 +679,6 @@ __device__ __forceinline__ float to_arith(double d, float) {
     return exact_float(d, f) ? f : (float)d;
 }
 __device__ __forceinline__ double to_arith(double d, double) { return d; }
-__device__ __forceinline__ double to_fp64(float v) {
-    const unsigned u = __float_as_uint(v), e = u >> 23 & 255u;
-    if (e - 1u >= 254u) return (double)v;                     // zero, subnormal, infinity, NaN
-    return __hiloint2double((int)((u & 0x80000000u) | (e + 896u) << 20 | (u >> 3 & 0xfffffu)), (int)(u << 29));
-}
-__device__ __forceinline__ double to_fp64(double v) { return v; }
 
 struct H2FF {
     FF x, y, z;
