@@ -15,8 +15,8 @@
 //
 // What bounds them: at large batches memory, at one item the launch and the reduction's two trips
 // through L2.  FP64 runs at 1/58 of the FP32 rate on this GPU and conversions between the two share
-// that pipe, so no thread converts or multiplies in FP64 per point: tableau coefficients are
-// rounded once per block, and only the sums of a reduction are FP64.
+// that pipe, so tableau coefficients are rounded once per block instead of per point, and in FP32 only the sums
+// of a reduction and K z of S_tilde's recurrence are FP64.
 #pragma once
 
 #include <type_traits>
@@ -193,28 +193,6 @@ template <class S> struct Basis {
     __device__ __forceinline__ const float* scale(int m, int b) const { return v.sc + m * srows + (long long)b * rows; }
 };
 
-// Double-float values (hi + lo, about 48 bits): error-free sums after Knuth (TAOCP 2, 4.2.2), products by one
-// fused multiply-add.
-struct FF {
-    float hi, lo;
-};
-__device__ __forceinline__ FF ff_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
-    return FF{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
-}
-// 2 P - a - b
-__device__ __forceinline__ FF ff_diff2(float P, float a, float b) {
-    const FF x = ff_sum(P, -a), y = ff_sum(P, -b), s = ff_sum(x.hi, y.hi);
-    return FF{s.hi, s.lo + (x.lo + y.lo)};
-}
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-    const FF s = ff_sum(a.hi, b.hi);
-    return FF{s.hi, s.lo + (a.lo + b.lo)};
-}
-__device__ __forceinline__ FF ff_mul(FF a, FF b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    return FF{p, fmaf(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi)};
-}
 // Reduction scratch of one preconditioner: nchunk blocks per item, up to nv values per block.
 struct ArRed {
     double* part;          // items * nchunk * nv
@@ -680,79 +658,15 @@ __device__ __forceinline__ float to_arith(double d, float) {
 }
 __device__ __forceinline__ double to_arith(double d, double) { return d; }
 
-struct H2FF {
-    FF x, y, z;
-};
-inline FF to_ff(double d) {
-    FF f;
-    f.hi = (float)d;
-    f.lo = (float)(d - (double)f.hi);
-    return f;
-}
-
-// K z at a point in FP64, rounded to A (out of line: FP32's rare path, Q1 and FP64).
-template <class A>
-__device__ __noinline__ A schur_K64(const double* u, const Geo& g, const SpaceOp<A>& op, int row, int j, int k, int c) {
-    const View<double> z{u, nullptr, g.n0};
-    return (A)op_K(z, g, op, row, j, k, c);
-}
-
-// K z at a point from its FP64 values, rounded once to A (FD).  For A = float the sums run in double-float
-// arithmetic, whose error (2^-46 of the largest term) is below the final rounding by as wide a margin as
-// FP64's in practice: K z cancels to 1e-4 of its terms on the finest grids, so the rounded results agree
-// but for ties.  FP64 needs 7 operations per point at two per cycle and SM.  A point whose values are not floats
-// of moderate size takes FP64.  One point per thread and the FP64 code out of line: four points per thread,
-// all inline, were 98 KB of code and 63 us for 14 items of 256^2, most of it instruction fetches.
-template <class A, bool D3>
-__device__ __forceinline__ A schur_K(const double* u, const Geo& g, const H2FF& h, const SpaceOp<A>& op, int row, int j,
-                                     int k, int c) {
-    if constexpr (std::is_same<A, float>::value) {
-        const double* p = u + (long long)row * g.n0 + c;
-        const int pl = g.n0 * g.n1;
-        double d[7];
-        d[0] = p[0];
-        d[1] = c > 0 ? p[-1] : 0.0;
-        d[2] = c + 1 < g.n0 ? p[1] : 0.0;
-        d[3] = j > 0 ? p[-g.n0] : 0.0;
-        d[4] = j + 1 < g.n1 ? p[g.n0] : 0.0;
-        if (D3) {
-            d[5] = k > 0 ? p[-pl] : 0.0;
-            d[6] = k + 1 < g.n2 ? p[pl] : 0.0;
-        }
-        float f[7];
-        bool ok = !op.q1;
-#pragma unroll
-        for (int q = 0; q < (D3 ? 7 : 5); ++q) ok = exact_float(d[q], f[q]) && ok;
-        if (ok) {
-            FF r;
-            if (op.faces.fx == nullptr) {
-                r = ff_add(ff_mul(ff_diff2(f[0], f[1], f[2]), h.x), ff_mul(ff_diff2(f[0], f[3], f[4]), h.y));
-                if (D3) r = ff_add(r, ff_mul(ff_diff2(f[0], f[5], f[6]), h.z));
-            } else {
-                const int fxi = row * (g.n0 + 1) + c, fyi = (k * (g.n1 + 1) + j) * g.n0 + c;
-                auto term = [&](float nb, float face) { return ff_mul(ff_sum(f[0], -nb), FF{face, 0.f}); };
-                r = ff_add(ff_add(term(f[1], op.faces.fx[fxi]), term(f[2], op.faces.fx[fxi + 1])),
-                           ff_add(term(f[3], op.faces.fy[fyi]), term(f[4], op.faces.fy[fyi + g.n0])));
-                if (D3) {
-                    const int fzi = row * g.n0 + c;
-                    r = ff_add(r, ff_add(term(f[5], op.faces.fz[fzi]), term(f[6], op.faces.fz[fzi + pl])));
-                }
-            }
-            return r.hi + r.lo;
-        }
-    }
-    return schur_K64<A>(u, g, op, row, j, k, c);
-}
-
 // t = K z_{v,n} (every stage's right-hand side: one copy) and the start of the step's inner solves with
-// ||r|| = sqrt(s) ||t||.
-template <class A, bool D3>
-__global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, H2FF h, int s, const StepPtrs* sp, int stride, A* t,
+// ||r|| = sqrt(s) ||t||.  K z in FP64, rounded once to A: it cancels to 1e-4 of its terms on the finest grids.
+template <class A>
+__global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, int s, const StepPtrs* sp, int stride, A* t,
                                                             SpaceOp<A> sop, ArRed red, ArItems it) {
     pdl_prologue();
     __shared__ double sum[1];
     const int b = blockIdx.y;
-    const double* z = sp->z + (long long)(sp->n + b * stride) * g.nx;
+    const View<double> z{sp->z + (long long)(sp->n + b * stride) * g.nx, nullptr, g.n0};
     A* tb = t + (long long)b * g.nx;
     A acc = A(0);
 #pragma unroll 1
@@ -760,7 +674,7 @@ __global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, H2FF h, int s
         const int row = (int)(q / (unsigned)g.n0), c = (int)(q - row * g.n0);
         int j, k;
         row_jk(g, row, j, k);
-        const A v = schur_K<A, D3>(z, g, h, sop, row, j, k, c);
+        const A v = (A)op_K(z, g, sop, row, j, k, c);
         tb[q] = v;
         acc += v * v;
     }

@@ -1337,12 +1337,9 @@ class Precond : public PrecondBase {
     aao_status forward_step(int B, int stride, const A* w, A* res) {
         const Geo& g = h->g;
         const int s = h->s;
-        const H2FF h2{to_ff(g.hx2), to_ff(g.hy2), to_ff(g.hz2)};
         const ArRed red = ar_red(B, g.nx / 4 + 1);        // four points per thread: the reduction is the larger part
-        with_int(g.d == 3, [&](auto d3) {
-            launch(k_schur_start<A, decltype(d3)::value>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g,
-                   h2, s, (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
-        });
+        launch(k_schur_start<A>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g, s,
+               (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
         scale_basis<A>(B, tbuf, g.nx, (const double*)betah, 1LL, V0, 1, stepp);
         AAO_LAUNCH_CHECK();
         AAO_TRY(arnoldi(B, 0));
