@@ -29,8 +29,7 @@
 //     inverse) is laid out once per handle as each CTA's shared-memory image, padded rows included, and
 //     copied linearly;
 //   * a thread keeps one 16-byte vector of columns and walks down consecutive rows with the rows around
-//     it in registers; on the finest level (FD, kappa = 1) the sweep's constants are folded, x + w (b - A x)
-//     = k0 P + kx (W + E) + ky (S + N) + w b, six operations per point instead of ten.  Rows are padded
+//     it in registers; on the finest level (FD, kappa = 1) the modes' constants are folded.  Rows are padded
 //     to whole vectors with zeros, so odd widths take the same path.
 //
 // One launch of three V(2,2)-cycles, one item on 16 CTAs (event-timed, before -> now): FP32 256^2 77.9 -> 69.3 us,
@@ -76,8 +75,7 @@ template <class SI> struct ClCtx {
     int fine0, has_faces;                 // level 0 is the FD operator; with faces of a kappa field
     A sigma, c;                           // level 0 (FD): sigma I + c K
     A hx2, hy2;
-    A w0, k0, kx, ky;                     // FD, kappa = 1: omega / a_PP; the folded sweep
-    A d0, ex, ey;                         // FD, kappa = 1: A u = d0 P - ex (W + E) - ey (S + N)
+    A w0, ex, ey;                         // FD, kappa = 1: omega / a_PP; c / hx^2, c / hy^2
     int fuse0;                            // 1: level 0 takes two zero-guess sweeps at once (mode 3)
     int n0[kClMaxLevels], n1[kClMaxLevels];
     int nvp[kClMaxLevels];                // vectors per padded row
@@ -140,8 +138,8 @@ template <class A> struct alignas(16) ClL {
     int S, fx, fy, far;                   // stencil at (own row 0, column 0), row stride nvp * VN; faces likewise (rows
                                           // of ld | of nvp * VN); 1: ghost rows reach beyond the next CTA
     int prev[kClReach], next[kClReach];   // rows of the CTAs before and after, nearest first (0: none)
-    A cf[4][4];                           // kind 1, per mode (cl_fd)
-    A mP[4];                              // kind 1, per mode: factor of P
+    A cf[3][4];                           // kind 1, per mode (cl_fd)
+    A mP[3];                              // kind 1, per mode: factor of P
     A sigma, c, hx2, hy2;                 // kind 2 (and kind 1 in 16-bit storage): sigma I + c K
     const void* Sg;                       // stencil in global memory at (own row 0, column 0), component stride cs,
     const float* Ssc;                     // row stride n0 (16-bit: times Ssc[k])
@@ -270,18 +268,22 @@ __device__ __forceinline__ ClRows cl_rows(const ClL<A>& v, int lo, int hi) {
 }
 
 // One point of a step with the FD operator, kappa = 1 (P, its neighbours and b).
-// FP64 folds the constants: kb b + k0 P + kx (W + E) + ky (S + N), six operations where the rate is two per
-// cycle and SM.  FP32 keeps the differences P - W, ..., which are exact for smooth fields, so the residual's
-// cancellation costs no digits: kw (b - kA (sigma P + ex (...) + ey (...))) + mP P.  16-bit storage takes
+// FP64: kw (b - (P + ex (2 P - W - E) + ey (2 P - S - N))) + (P or 0).  (Folding the constants further, into
+// k0 P + kx (W + E) + ky (S + N) + w b, takes six operations, but makes the residual of a smooth x
+// five to thirteen times and a sweep's result up to three times less accurate; subtracting the terms from b one by
+// one shortens the chain, but rounds three times at b's size.)
+// FP32 takes the differences P - W, ..., which are exact for smooth fields, so the residual's
+// cancellation costs no digits: kw (b - (kP P + ex (...) + ey (...))) + mP P.  16-bit storage takes
 // the level kernels' formula operation by operation: its results are rounded to the storage format, and the
 // roundings are pinned.
 template <bool SCALED>
-__device__ __forceinline__ double cl_fd(const ClL<double>&, const double* cf, double, int, double b, double P, double W,
+__device__ __forceinline__ double cl_fd(const ClL<double>&, const double* cf, double, int mode, double b, double P, double W,
                                         double E, double S, double N) {
-    double s = cf[0] * b;
-    s += cf[1] * P;
-    s += cf[2] * (W + E);
-    return s + cf[3] * (S + N);
+    const double dx = 2.0 * P - W - E, dy = 2.0 * P - S - N;
+    double s = P;                         // sigma = 1
+    s += cf[2] * dx;
+    s += cf[3] * dy;
+    return cf[0] * (b - s) + (mode == 0 ? P : 0.0);
 }
 template <bool SCALED>
 __device__ __forceinline__ float cl_fd(const ClL<float>& v, const float* cf, float mP, int mode, float b, float P, float W,
@@ -343,25 +345,51 @@ __device__ __forceinline__ void cl_step(const ClL<A>& v, int rank, int mode, int
     };
     if (v.kind == 1) {
         A cf[4];
+        const int m = mode == 3 ? 0 : mode;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) cf[i] = v.cf[mode][i];
-        const A mP = v.mP[mode];
+        for (int i = 0; i < 4; ++i) cf[i] = v.cf[m][i];
+        const A mP = v.mP[m];
+        // mode 3: a sweep from w0 b, rounded as the first of the two sweeps would store it (a loop of its own: products
+        // that the other modes skip would still take their turns of the FP64 pipe)
+        auto rows = [&](auto from_b) {
+            constexpr bool kFromB = decltype(from_b)::value;
+            auto times = [&](A* x) {
+#pragma unroll
+                for (int i = 0; i < VN; ++i) x[i] *= cf[0];
+            };
+            if constexpr (kFromB) {
+                times(S);
+                times(P);
+            }
 #pragma unroll 1
-        for (int r = q.r0; r < q.r1; ++r) {
-            A b[VN], out[VN], l = A(0), e = A(0);
-            cl_vload(bm, b);
-            if (ax) {
-                cl_vload(xm + ld, N);
-                l = xm[-1];
-                e = xm[VN];
-            }
+            for (int r = q.r0; r < q.r1; ++r) {
+                A b[VN], out[VN], l = A(0), e = A(0);
+                cl_vload(bm, b);
+                if (ax) {
+                    cl_vload(xm + ld, N);
+                    l = xm[-1];
+                    e = xm[VN];
+                    if constexpr (kFromB) {
+                        times(N);
+                        l *= cf[0];
+                        e *= cf[0];
+                    }
+                }
 #pragma unroll
-            for (int i = 0; i < VN; ++i) {
-                const A W = i == 0 ? l : P[i - 1], E = i == VN - 1 ? e : P[i + 1];
-                out[i] = cl_fd<PT<SI>::scaled>(v, cf, mP, mode, b[i], P[i], W, E, S[i], N[i]);
+                for (int i = 0; i < VN; ++i) {
+                    const A W = i == 0 ? l : P[i - 1], E = i == VN - 1 ? e : P[i + 1];
+                    out[i] = cl_fd<PT<SI>::scaled>(v, cf, mP, m, b[i], P[i], W, E, S[i], N[i]);
+                }
+                finish(r, out);
             }
-            finish(r, out);
+        };
+        if constexpr (!PT<SI>::scaled) {              // (16-bit storage's programs have no mode 3)
+            if (mode == 3) {
+                rows(std::true_type{});
+                return;
+            }
         }
+        rows(std::false_type{});
         return;
     }
     const int wrow = v.nvp * VN;
@@ -781,29 +809,13 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_mg(const __grid_const
             v.Sg = t.sten[l] + (long long)v.a * v.n0;
             v.Ssc = t.sten_sc[l];
         }
-        if constexpr (std::is_same<A, double>::value) {
-            v.cf[0][0] = v.cf[1][0] = v.cf[3][0] = t.w0;
-            v.cf[0][1] = t.k0;
-            v.cf[0][2] = t.kx;
-            v.cf[0][3] = t.ky;
-            v.cf[2][0] = A(1);
-            v.cf[2][1] = -t.d0;
-            v.cf[2][2] = t.ex;
-            v.cf[2][3] = t.ey;
-            for (int q = 1; q < 4; ++q) v.cf[3][q] = t.w0 * v.cf[0][q];
-        } else {
-            for (int q = 0; q < 4; ++q) {
-                const A k = q == 3 ? t.w0 : A(1);          // mode 3: A acts on w0 b
-                v.cf[q][0] = q == 2 ? A(1) : t.w0;
-                v.cf[q][1] = k * t.sigma;
-                v.cf[q][2] = k * t.ex;
-                v.cf[q][3] = k * t.ey;
-            }
+        for (int q = 0; q < 3; ++q) {
+            v.cf[q][0] = q == 2 ? A(1) : t.w0;
+            v.cf[q][1] = q == 1 ? A(0) : t.sigma;
+            v.cf[q][2] = q == 1 ? A(0) : t.ex;
+            v.cf[q][3] = q == 1 ? A(0) : t.ey;
+            v.mP[q] = q == 0 ? A(1) : A(0);
         }
-        v.cf[1][1] = v.cf[1][2] = v.cf[1][3] = A(0);
-        v.mP[0] = A(1);
-        v.mP[1] = v.mP[2] = A(0);
-        v.mP[3] = t.w0;
         v.hx2 = t.hx2;
         v.hy2 = t.hy2;
         v.sigma = t.sigma;

@@ -649,17 +649,12 @@ class Precond : public PrecondBase {
             ClCtx<SI>& q = pl.ctx[i];
             q = t;
             const double c = h->tau * h->D[i], hx2 = h->g.hx2, hy2 = h->g.hy2;
-            const double d0 = 1.0 + c * (2.0 * hx2 + 2.0 * hy2), w = h->opt.mg_omega / d0;
             q.c = (A)c;
             // omega / a_PP by the staged weights' operations
             const A kd = A(2) * (A)hx2 + A(2) * (A)hy2;
             q.w0 = (A)h->opt.mg_omega / std::fma((A)c, kd, A(1));
             q.hx2 = (A)hx2;
             q.hy2 = (A)hy2;
-            q.k0 = (A)(1.0 - h->opt.mg_omega);
-            q.kx = (A)(w * c * hx2);
-            q.ky = (A)(w * c * hy2);
-            q.d0 = (A)d0;
             q.ex = (A)(c * hx2);
             q.ey = (A)(c * hy2);
             for (int l = 0; l < L; ++l) {
