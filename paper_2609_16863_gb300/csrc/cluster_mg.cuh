@@ -394,7 +394,7 @@ __device__ __forceinline__ void cl_step(const ClL<A>& v, int rank, int mode, int
     }
     const int wrow = v.nvp * VN;
     const A* wm = sm + v.W + q.r0 * wrow + c;
-    const A mP = mode == 0 ? A(1) : A(0);
+    const bool addx = mode == 0;
     if (FACES && v.kind == 2) {
         const A sigma = v.sigma, cK = v.c;
         const A* fx = sm + v.fx + q.r0 * ld + c;
@@ -421,7 +421,7 @@ __device__ __forceinline__ void cl_step(const ClL<A>& v, int rank, int mode, int
                 }
             }
 #pragma unroll
-            for (int i = 0; i < VN; ++i) out[i] = (mode == 2 ? A(1) : w[i]) * b[i] + mP * P[i];
+            for (int i = 0; i < VN; ++i) out[i] = (mode == 2 ? A(1) : w[i]) * b[i] + (addx ? P[i] : A(0));
             fx += ld;
             fy += wrow;
             wm += wrow;
@@ -470,38 +470,25 @@ __device__ __forceinline__ void cl_step(const ClL<A>& v, int rank, int mode, int
             }
 #pragma unroll
             for (int i = 0; i < VN; ++i) {
-                if constexpr (PT<SI>::scaled) {
-                    // the level kernels' order (see cl_fd)
-                    A acc = A(0);
-                    acc += K[0][i] * (i == 0 ? sl : S[i - 1]);
-                    acc += K[1][i] * S[i];
-                    acc += K[2][i] * (i == VN - 1 ? sr : S[i + 1]);
-                    acc += K[3][i] * (i == 0 ? pl : P[i - 1]);
-                    acc += K[4][i] * P[i];
-                    acc += K[5][i] * (i == VN - 1 ? pr : P[i + 1]);
-                    acc += K[6][i] * (i == 0 ? nl : N[i - 1]);
-                    acc += K[7][i] * N[i];
-                    acc += K[8][i] * (i == VN - 1 ? nr : N[i + 1]);
-                    b[i] -= acc;
-                    continue;
-                }
-                // three chains, one per row
-                A s0 = K[0][i] * (i == 0 ? sl : S[i - 1]);
-                A s1 = K[3][i] * (i == 0 ? pl : P[i - 1]);
-                A s2 = K[6][i] * (i == 0 ? nl : N[i - 1]);
-                s0 += K[1][i] * S[i];
-                s1 += K[4][i] * P[i];
-                s2 += K[7][i] * N[i];
-                s0 += K[2][i] * (i == VN - 1 ? sr : S[i + 1]);
-                s1 += K[5][i] * (i == VN - 1 ? pr : P[i + 1]);
-                s2 += K[8][i] * (i == VN - 1 ? nr : N[i + 1]);
-                b[i] -= s0 + s1 + s2;
+                // in the level kernels' order: a smooth x cancels late in the sum, where three chains, one per row, would
+                // round larger partial sums (residual off by a third more) and take three operations more
+                A acc = A(0);
+                acc += K[0][i] * (i == 0 ? sl : S[i - 1]);
+                acc += K[1][i] * S[i];
+                acc += K[2][i] * (i == VN - 1 ? sr : S[i + 1]);
+                acc += K[3][i] * (i == 0 ? pl : P[i - 1]);
+                acc += K[4][i] * P[i];
+                acc += K[5][i] * (i == VN - 1 ? pr : P[i + 1]);
+                acc += K[6][i] * (i == 0 ? nl : N[i - 1]);
+                acc += K[7][i] * N[i];
+                acc += K[8][i] * (i == VN - 1 ? nr : N[i + 1]);
+                b[i] -= acc;
             }
         }
         Gm += v.n0;
         Sm += wrow;
 #pragma unroll
-        for (int i = 0; i < VN; ++i) out[i] = (mode == 2 ? A(1) : w[i]) * b[i] + mP * P[i];
+        for (int i = 0; i < VN; ++i) out[i] = (mode == 2 ? A(1) : w[i]) * b[i] + (addx ? P[i] : A(0));
         wm += wrow;
         finish(r, out);
         sl = pl;
