@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "handle.cuh"
+#include "matvec.cuh"
 
 namespace aao {
 
