@@ -22,8 +22,9 @@ namespace aao {
 // its FP32 result, k_relax_decide).
 // Bound by FP64 arithmetic (two operations per cycle and SM): so tau a_ij and tau b_i are formed on the host,
 // K's differences stay as they are (2 P - W - E is exact for smooth fields; merging the stages before K would
-// save five operations of 41 but round those sums) and, where the mesh is square, one factor 1/h^2
-// multiplies each row's sum of differences instead of every difference (36).  Every load of a thread is issued
+// save five operations of 41 but round those sums) and, where the mesh is square, the factor 1/h^2 is part of
+// tau a_ij instead of multiplying every difference (36).  K v, the largest term of a stage's row, is added last, so one
+// rounding of the row's size is left (rms error of the stages 0.89e-16; with K v first 1.21e-16).  Every load of a thread is issued
 // before its arithmetic; a warp per row with its columns in a loop left the FP64 pipe idle for a third of the time.
 // Measured: 256^2, s = 3, 128 steps 905 -> 655 us (36 operations per point and block: 0.46 TFMA/s of 0.60);
 // 49 x 45 x 41 with faces, s = 2, 24 steps, transposed 256 -> 162 us; 32^2, 16 steps 5.5 -> 4.2 us.
@@ -31,7 +32,7 @@ namespace aao {
 constexpr int kMvThreads = 128;
 
 struct MvTab {
-    double A[kMaxS * kMaxS], b[kMaxS];   // tau a_ij (transpose: tau a_ji), tau b_i
+    double A[kMaxS * kMaxS], b[kMaxS];   // tau a_ij (transpose: tau a_ji), on square meshes times 1 / h^2; tau b_i
     double h2;                           // square meshes: 1 / h^2 (the differences are unscaled), else 1
     double hx2, hy2, hz2;                // factors of the differences (square meshes: 1)
 };
@@ -147,12 +148,12 @@ __global__ void __launch_bounds__(kMvThreads) k_matvec(Geo g, int nt, int stages
 #pragma unroll
     for (int i = 0; i < TS; ++i)
         if (i < s) {
-            double a = Kv;
+            double a = TRANS ? V[i][0] - tab.b[i] * v1 : V[i][0];
 #pragma unroll
             for (int q = 0; q < TS; ++q)
                 if (q < s) a += tab.A[i * s + q] * K[q];
-            const double m = TRANS ? V[i][0] - tab.b[i] * v1 : V[i][0];
-            put(voff + ((long long)n * s + i) * nx + p, SQUARE ? m + tab.h2 * a : m + a);
+            if constexpr (!TRANS) a += SQUARE ? tab.h2 * Kv : Kv;
+            put(voff + ((long long)n * s + i) * nx + p, a);
         }
 }
 
@@ -166,6 +167,8 @@ inline void launch_matvec(const Geo& g, int nt, const Tab& tab, double tau, cons
         for (int q = 0; q < s; ++q) t.A[i * s + q] = tau * (transpose ? tab.A[q * s + i] : tab.A[i * s + q]);
     }
     const bool square = faces.fx == nullptr && g.hx2 == g.hy2 && (g.d == 2 || g.hz2 == g.hx2);
+    if (square)
+        for (int i = 0; i < s * s; ++i) t.A[i] *= g.hx2;
     t.h2 = g.hx2;
     t.hx2 = g.hx2;
     t.hy2 = g.hy2;
