@@ -38,22 +38,12 @@
 // Deep ghost regions against single ghost rows on the new kernel: 256^2 68 against 82, 64^2 FP64 60.1 against 60.3.
 #pragma once
 
-#include <algorithm>
 #include <type_traits>
-#include <vector>
 
+#include "cluster_plan.h"
 #include "mg.cuh"
 
 namespace aao {
-
-constexpr int kClMax = 16;            // CTAs per cluster (16 needs the non-portable size)
-constexpr int kClThreads = 512;
-constexpr int kClMaxBatch = 32;       // batches of at most this many items run one cluster per item
-constexpr int kClBatch8 = 8;          // batches of at least this many items take the 8-CTA plan
-constexpr int kClPad = 4;             // columns before a row's first point and after its last vector: rows
-                                      // start 16-byte aligned, the columns beside the grid are zero
-constexpr int kClReach = 3;           // CTAs on either side whose ghost rows may hold a CTA's rows
-constexpr int kClMaxLevels = 10;      // 2D levels of grids that fit a cluster
 
 // Columns per thread: one 16-byte vector in FP32.  FP64 takes single columns: a step's chain of FP64 operations
 // is long, and twice the warps hide twice as much of it.
@@ -68,38 +58,11 @@ template <> struct ClVec<double> {
 };
 
 // Plan of one shift (a kernel parameter: every field is read through the constant bank).
-template <class SI> struct ClCtx {
+template <class SI> struct ClCtx : ClShape {
     using A = typename PT<SI>::A;
-    int C, L, T;                          // cluster size, levels, T = L-1 (the replicated coarsest level)
-    int cycles, nu1, nu2;
-    int fine0, has_faces;                 // level 0 is the FD operator; with faces of a kappa field
     A sigma, c;                           // level 0 (FD): sigma I + c K
     A hx2, hy2;
     A w0, ex, ey;                         // FD, kappa = 1: omega / a_PP; c / hx^2, c / hy^2
-    int fuse0;                            // 1: level 0 takes two zero-guess sweeps at once (mode 3)
-    int n0[kClMaxLevels], n1[kClMaxLevels];
-    int nvp[kClMaxLevels];                // vectors per padded row
-    unsigned magicv[kClMaxLevels];        // ceil(2^32 / nvp): tid / nvp = umulhi(tid, magicv)
-    unsigned magic[kClMaxLevels];         // ceil(2^32 / n0)
-    int per[kClMaxLevels];                // rows per thread
-    int H[kClMaxLevels];                  // ghost rows
-    int ix[kClMaxLevels];                 // rows of the x inbox per side
-    int maxr[kClMaxLevels];               // own rows in the shared-memory layout
-    int rlo[kClMaxLevels][kClMax + 1];    // CTA r owns rows [rlo[l][r], rlo[l][r+1]) (the coarsest: computes them)
-    int off[kClMaxLevels];                // A-element offset of level l's X0 | X1 | B, each (maxr + 2H) x ld
-    int ioff[kClMaxLevels];               // x inbox: 2 ix rows of ld
-    int soff[kClMaxLevels];               // staged stencil, 9 x (maxr + 2(H-1)) x padded row (-1: none)
-    int woff[kClMaxLevels];               // omega / a_PP, (maxr + 2H) x padded row (-1: the scalar w0)
-    int sten_global[kClMaxLevels];        // 1: level l's stencil is read from global memory (L2), not staged
-    int fxoff, fyoff;                     // level 0 faces: rows of ld | rows of the padded width
-    int dinv_global;                      // 1: the rows of A_c^{-1} are read from global memory
-    int dinv_off, boff;                   // this CTA's rows of A_c^{-1}, each padded to ncp; the coarsest b (ncp)
-    int ncp;                              // unknowns of the coarsest level, rounded up to vectors
-    int cs[kClMax + 1];                   // coarsest rows [cs[r], cs[r+1]) of A_c^{-1} b are computed by CTA r
-    int img_off, img_len;                 // the staged constants: A elements [img_off, img_off + img_len)
-    int prog_off;                         // byte offset of the program in shared memory (part of the image)
-    int pc[4];                            // operations of the first cycle, of odd and of even later cycles
-    int kfin;                             // buffer of x_0 after the last cycle
     const A* img;                         // C images
     const A* fx;
     const A* fy;
@@ -108,20 +71,6 @@ template <class SI> struct ClCtx {
     const A* W[kClMaxLevels];             // omega / a_PP of every point (null: w0)
     const A* Dinv;                        // rows of ncp values (dinv_global and the image's source: nc)
 };
-
-// One operation of the cycle's program.
-enum ClKind { kClStep, kClRestrict, kClRestrictLast, kClSolve, kClProlong, kClInbox, kClClear };
-struct ClOp {
-    unsigned char kind, lev;
-    unsigned char mode;                   // step: 0 sweep, 1 sweep of a zero guess, 2 residual, 3 two sweeps of a
-                                          // zero guess at once; restriction: also the first sweep (1)
-    unsigned char kin;                    // buffer read (prolong: x_f's)
-    unsigned char kc;                     // prolong: buffer of x_c; step: buffer written; restriction: of the sweep
-    unsigned char ext;                    // ghost rows computed
-    unsigned char depth;                  // ghost rows stored into the other CTAs (0: none)
-    unsigned char flags;                  // 1: into the x inboxes; 2: cluster barrier
-};
-static_assert(sizeof(ClOp) == 8, "one 8-byte load");
 
 // One distributed level as a step sees it (shared memory, built once per launch).  Positions are indices
 // into the dynamic shared memory: accesses stay in the shared address space with 32-bit arithmetic (as
@@ -943,90 +892,6 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_mg(const __grid_const
             }
         }
     }
-}
-
-// The program of a plan: the operations of the first cycle, of an odd and of an even later one (the
-// buffers alternate with the number of sweeps), and the buffer x_0 ends in.  Every CTA runs the same
-// program, so its barriers match.  A step writes ghost rows of other CTAs' buffers (depth > 0 without
-// the inbox flag) only where a cluster barrier separates it from the last read of those rows: with H = 1 an
-// exchange follows every sweep; on levels with deeper ghost regions (at most two post-sweeps) no sweep but
-// the first post-sweep can be such a step, and the buffer it writes was last read by the restriction.  b and
-// the inboxes are read before the barriers of the steps in between.
-template <class SI> inline std::vector<ClOp> cl_program(ClCtx<SI>& t) {
-    std::vector<ClOp> prog;
-    const int T = t.T, nu1 = t.nu1, nu2 = t.nu2;
-    auto emit = [&](int kind, int l, int mode, int kin, int kc, int ext, int depth, int flags) {
-        prog.push_back(ClOp{(unsigned char)kind, (unsigned char)l, (unsigned char)mode, (unsigned char)kin,
-                            (unsigned char)kc, (unsigned char)ext, (unsigned char)depth,
-                            (unsigned char)(flags | (depth > 0 ? 2 : 0))});
-    };
-    int cur[kClMaxLevels] = {}, reach[kClMaxLevels] = {};     // buffer of x; valid ghost rows of the pre-smoothed x
-    int after[3] = {};
-    for (int part = 0; part < 3; ++part) {
-        t.pc[part] = (int)prog.size();
-        for (int l = 0; l < T; ++l) {
-            const int H = t.H[l];
-            int k = cur[l], v = H;
-            bool zero = part == 0 || l > 0;
-            int sw = 0;
-            if (!zero) {
-                emit(kClInbox, l, 0, k, 0, 0, 0, 0);
-            } else if (l > 0 && nu1 > 0) {
-                sw = 1;                        // the restriction has done the first sweep, into buffer k ^ 1
-                zero = false;
-                k ^= 1;
-            } else if (l == 0 && nu1 > 1 && t.fuse0) {
-                // two sweeps from b at once
-                const int ext = std::min(v - 1, nu1 - 2 + 2), depth = ext == 0 ? H : 0;
-                emit(kClStep, l, 3, 2, k, ext, depth, 0);
-                v = depth > 0 ? H : ext;
-                sw = 2;
-                zero = false;
-            }
-            for (; sw < nu1; ++sw) {
-                // the result is read up to (sweeps left) + 2 rows beyond the own ones
-                const int ext = std::min(zero ? v : v - 1, nu1 - 1 - sw + 2);
-                const int depth = ext == 0 ? H : 0;
-                emit(kClStep, l, zero ? 1 : 0, k, k ^ 1, ext, depth, 0);
-                v = depth > 0 ? H : ext;
-                zero = false;
-                k ^= 1;
-            }
-            int kr = 2;                        // no sweep on a zero guess: the residual is b
-            if (zero) {
-                emit(kClClear, l, 0, k, 0, 0, 0, 0);
-            } else {
-                emit(kClStep, l, 2, k, k ^ 1, v >= 2 ? 1 : 0, v >= 2 ? 0 : 1, 0);
-                kr = k ^ 1;
-            }
-            cur[l] = k;
-            reach[l] = v;
-            emit(l + 1 < T ? kClRestrict : kClRestrictLast, l, nu1 > 0 ? 1 : 0, kr, cur[l + 1] ^ 1, 0, 0, 2);
-        }
-        emit(kClSolve, T, 0, 0, 0, 0, 0, 2);
-        for (int l = T - 1; l >= 0; --l) {
-            int k = cur[l];
-            // interpolate on up to nu2 ghost rows: e of them need (e + 2) / 2 rows of x_c beyond the own ones
-            int v = std::min(reach[l], nu2);
-            if (l + 1 < T) v = std::min(v, 2 * t.ix[l + 1] - 1);
-            emit(kClProlong, l, 0, k, l + 1 < T ? cur[l + 1] : 0, v, nu2 == 0 ? t.ix[l] : 0, 0);
-            for (int sw = 0; sw < nu2; ++sw) {
-                const bool fin = sw == nu2 - 1;
-                const int e = std::min(v - 1, nu2 - 1 - sw);
-                const int depth = fin ? t.ix[l] : (e == 0 ? t.H[l] : 0);
-                emit(kClStep, l, 0, k, k ^ 1, e, depth, fin ? 1 : 0);
-                v = depth > 0 ? t.H[l] : e;
-                k ^= 1;
-            }
-            cur[l] = k;
-        }
-        after[part] = cur[0];
-    }
-    t.pc[3] = (int)prog.size();
-    prog.push_back(ClOp{});
-    const int last = t.cycles - 1;
-    t.kfin = after[last == 0 ? 0 : 2 - (last & 1)];
-    return prog;
 }
 
 // omega / a_PP of every point of a level, from its stored stencil or the FD diagonal.

@@ -513,110 +513,30 @@ class Precond : public PrecondBase {
     }
 
     bool plan_cluster(int C, int deep, int lean, long long dyn_max, ClCtx<SI>& t, long long& bytes, int& resident) {
-        const Geo& g0 = h->g;
-        const int T = L - 1;
-        constexpr int VN = ClVec<A>::n;
-        if (g0.n1 < C || L > kClMaxLevels) return false;
-        const bool fine0 = !h->q1;
-        const bool faces = fine0 && h->has_kappa;
-        const int nu1 = h->opt.mg_pre, nu2 = h->opt.mg_post;
-        // ghost rows for a whole phase leave no exchange between two sweeps that would write ghost rows a
-        // neighbour still reads; that covers at most two post-sweeps
-        if (deep > 0 && (nu2 > 2 || nu1 > 3)) return false;
-        std::memset(&t, 0, sizeof(t));
-        t.C = C;
-        t.L = L;
-        t.T = T;
-        t.cycles = h->opt.mg_cycles;
-        t.nu1 = nu1;
-        t.nu2 = nu2;
+        if (L > kClMaxLevels) return false;
+        ClSpec spec{};
+        spec.C = C;
+        spec.deep = deep;
+        spec.lean = lean;
+        spec.L = L;
+        for (int l = 0; l < L; ++l) {
+            spec.n0[l] = lev[l].g.n0;
+            spec.n1[l] = lev[l].g.n1;
+        }
+        spec.fine0 = h->q1 ? 0 : 1;
+        spec.faces = spec.fine0 && h->has_kappa ? 1 : 0;
+        spec.fuse0 = spec.fine0 && !spec.faces && !PT<SI>::scaled ? 1 : 0;
+        spec.cycles = h->opt.mg_cycles;
+        spec.nu1 = h->opt.mg_pre;
+        spec.nu2 = h->opt.mg_post;
+        spec.vn = ClVec<A>::n;
+        spec.size = (int)sizeof(A);
+        t = ClCtx<SI>{};
+        bytes = cl_layout(t, spec);
+        if (bytes < 0 || bytes > dyn_max) return false;
         t.sigma = A(1);
-        t.fine0 = fine0 ? 1 : 0;
-        t.has_faces = faces ? 1 : 0;
-        t.fuse0 = fine0 && !faces && !PT<SI>::scaled ? 1 : 0;
         t.fx = facesA.fx;
         t.fy = facesA.fy;
-        t.dinv_global = lean >= 1 ? 1 : 0;
-        auto magic = [](long long d) { return (unsigned)((4294967296ULL + (unsigned long long)d - 1) / (unsigned long long)d); };
-
-        long long o = 0;
-        auto take = [&](long long n) {
-            long long at = o;
-            o += (n + 3) / 4 * 4;
-            return (int)at;
-        };
-        for (int l = 0; l < L; ++l) {
-            const Geo& gl = lev[l].g;
-            const int nvp = std::max((gl.n0 + VN - 1) / VN, 2);
-            if (nvp > kClThreads) return false;
-            t.n0[l] = gl.n0;
-            t.n1[l] = gl.n1;
-            t.nvp[l] = nvp;
-            t.magicv[l] = magic(nvp);
-            t.magic[l] = magic(std::max(gl.n0, 2));
-            for (int r = 0; r <= C; ++r)
-                t.rlo[l][r] = l == 0 ? (int)((long long)r * gl.n1 / C) : t.rlo[l - 1][r] / 2;
-            // Every CTA must own at least one row of every distributed level (neighbours store edge rows
-            // into the CTAs that own the rows beside theirs; grids with few rows for their width fail
-            // this), and its ghost rows must belong to the kClReach CTAs on either side.
-            int mr = 1;
-            auto covered = [&](int need) {
-                for (int r = 0; r < C; ++r) {
-                    if (std::max(t.rlo[l][r] - need, 0) < t.rlo[l][std::max(r - kClReach, 0)]) return false;
-                    const int top = r + 1 + kClReach >= C ? gl.n1 : t.rlo[l][r + 1 + kClReach];
-                    if (std::min(t.rlo[l][r + 1] + need, gl.n1) > top) return false;
-                }
-                return true;
-            };
-            for (int r = 0; r < C; ++r) {
-                const int own = t.rlo[l][r + 1] - t.rlo[l][r];
-                mr = std::max(mr, own);
-                if (l < T && own < 1) return false;
-            }
-            const int deepH = std::max(l == 0 ? nu1 + 2 : nu1 + 1, 2);
-            const bool dl = deep >= (l == 0 ? 2 : 1) && l < T && covered(deepH);
-            if (deep == 2 && l == 0 && !dl) return false;
-            t.H[l] = dl ? deepH : 1;
-            t.ix[l] = l >= T ? 0 : (l == 0 ? t.H[0] : (deep > 0 && covered(2) ? 2 : 1));
-            t.maxr[l] = l < T ? mr : gl.n1;
-            const int groups = kClThreads / nvp;
-            t.per[l] = (t.maxr[l] + 2 * t.H[l] + groups - 1) / groups;
-            const long long ld = (long long)nvp * VN + 2 * kClPad;
-            t.off[l] = take(3LL * (t.maxr[l] + 2 * t.H[l]) * ld);
-            t.ioff[l] = take(2LL * t.ix[l] * ld);
-        }
-        const long long ncst = lev[T].g.nx;
-        t.ncp = (int)((ncst + VN - 1) / VN * VN);
-        t.boff = take(t.ncp);
-        // the image of constants, the program at its end
-        t.img_off = (int)o;
-        for (int l = 0; l < L; ++l) {
-            t.soff[l] = t.woff[l] = -1;
-            if (l >= T) continue;
-            const long long np = (long long)t.nvp[l] * VN;
-            const bool fd = l == 0 && fine0;
-            if (!fd) {
-                t.sten_global[l] = l >= 1 && (lean >= 3 || (lean == 2 && l == 1)) ? 1 : 0;
-                if (t.sten_global[l] && lev[l].g.n0 != np) return false;     // read as whole vectors of the padded row
-                if (!t.sten_global[l]) t.soff[l] = take(9LL * (t.maxr[l] + 2 * (t.H[l] - 1)) * np);
-            }
-            if (!fd || faces) t.woff[l] = take((long long)(t.maxr[l] + 2 * t.H[l]) * np);
-        }
-        if (faces) {
-            const long long np = (long long)t.nvp[0] * VN, rows = t.maxr[0] + 2 * (t.H[0] - 1);
-            t.fxoff = take(rows * (np + 2 * kClPad));
-            t.fyoff = take((rows + 1) * np);
-        }
-        int msl = 0;
-        for (int r = 0; r <= C; ++r) t.cs[r] = (int)((long long)r * ncst / C);
-        for (int r = 0; r < C; ++r) msl = std::max(msl, t.cs[r + 1] - t.cs[r]);
-        t.dinv_off = t.dinv_global ? -1 : take((long long)msl * t.ncp);
-        const long long nprog = (long long)cl_program(t).size();
-        t.prog_off = (int)(o * (long long)sizeof(A));
-        take((nprog * (long long)sizeof(ClOp) + (long long)sizeof(A) - 1) / (long long)sizeof(A));
-        t.img_len = (int)(o - t.img_off);
-        bytes = o * (long long)sizeof(A);
-        if (bytes > dyn_max) return false;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(C);
         cfg.blockDim = dim3(kClThreads);
