@@ -62,16 +62,19 @@ struct ClOp {
 };
 static_assert(sizeof(ClOp) == 8, "one 8-byte load");
 
+// Ghost rows of the pre-smoothed x that are read: two by the residual of a ghost row, nu2 by the post-sweeps.
+inline int cl_reach_after(int nu2) { return nu2 > 2 ? nu2 : 2; }
+
 // The program of a plan: the operations of the first cycle, of an odd and of an even later one (the
 // buffers alternate with the number of sweeps), and the buffer x_0 ends in.  Every CTA runs the same
 // program, so its barriers match.  A step writes ghost rows of other CTAs' buffers (depth > 0 without
 // the inbox flag) only where a cluster barrier separates it from the last read of those rows: with H = 1 an
-// exchange follows every sweep; on levels with deeper ghost regions (at most two post-sweeps) no sweep but
-// the first post-sweep can be such a step, and the buffer it writes was last read by the restriction.  b and
-// the inboxes are read before the barriers of the steps in between.
+// exchange follows every sweep; on levels with deeper ghost regions no sweep but the first post-sweep can be such a
+// step (the interpolation covers all the post-sweeps' ghost rows, or one), and the buffer it writes was last read
+// by the restriction.  b and the inboxes are read before the barriers of the steps in between.
 inline std::vector<ClOp> cl_program(ClShape& t) {
     std::vector<ClOp> prog;
-    const int T = t.T, nu1 = t.nu1, nu2 = t.nu2;
+    const int T = t.T, nu1 = t.nu1, nu2 = t.nu2, left = cl_reach_after(nu2);
     auto emit = [&](int kind, int l, int mode, int kin, int kc, int ext, int depth, int flags) {
         prog.push_back(ClOp{(unsigned char)kind, (unsigned char)l, (unsigned char)mode, (unsigned char)kin,
                             (unsigned char)kc, (unsigned char)ext, (unsigned char)depth,
@@ -94,15 +97,15 @@ inline std::vector<ClOp> cl_program(ClShape& t) {
                 k ^= 1;
             } else if (l == 0 && nu1 > 1 && t.fuse0) {
                 // two sweeps from b at once
-                const int ext = std::min(v - 1, nu1 - 2 + 2), depth = ext == 0 ? H : 0;
+                const int ext = std::min(v - 1, nu1 - 2 + left), depth = ext == 0 ? H : 0;
                 emit(kClStep, l, 3, 2, k, ext, depth, 0);
                 v = depth > 0 ? H : ext;
                 sw = 2;
                 zero = false;
             }
             for (; sw < nu1; ++sw) {
-                // the result is read up to (sweeps left) + 2 rows beyond the own ones
-                const int ext = std::min(zero ? v : v - 1, nu1 - 1 - sw + 2);
+                // the result is read up to (sweeps left) + left rows beyond the own ones
+                const int ext = std::min(zero ? v : v - 1, nu1 - 1 - sw + left);
                 const int depth = ext == 0 ? H : 0;
                 emit(kClStep, l, zero ? 1 : 0, k, k ^ 1, ext, depth, 0);
                 v = depth > 0 ? H : ext;
@@ -126,6 +129,7 @@ inline std::vector<ClOp> cl_program(ClShape& t) {
             // interpolate on up to nu2 ghost rows: e of them need (e + 2) / 2 rows of x_c beyond the own ones
             int v = std::min(reach[l], nu2);
             if (l + 1 < T) v = std::min(v, 2 * t.ix[l + 1] - 1);
+            if (v < nu2) v = std::min(v, 1);       // an exchange among the sweeps: after the first one
             emit(kClProlong, l, 0, k, l + 1 < T ? cur[l + 1] : 0, v, nu2 == 0 ? t.ix[l] : 0, 0);
             for (int sw = 0; sw < nu2; ++sw) {
                 const bool fin = sw == nu2 - 1;
@@ -163,9 +167,8 @@ struct ClSpec {
 // Lay out a plan; its bytes of shared memory, or -1 where the grid does not take it.
 inline long long cl_layout(ClShape& t, const ClSpec& s) {
     if (s.n1[0] < s.C || s.L > kClMaxLevels) return -1;
-    // ghost rows for a whole phase leave no exchange between two sweeps that would write ghost rows a
-    // neighbour still reads; that covers at most two post-sweeps
-    if (s.deep > 0 && (s.nu2 > 2 || s.nu1 > 3)) return -1;
+    // ghost rows for up to three sweeps (an inbox of two rows of x_c serves three of the interpolation's ghost rows)
+    if (s.deep > 0 && (s.nu2 > 3 || s.nu1 > 3)) return -1;
     const int C = s.C, L = s.L, T = L - 1, VN = s.vn, nu1 = s.nu1, nu2 = s.nu2, deep = s.deep, lean = s.lean;
     t = ClShape{};
     t.C = C;
@@ -213,7 +216,7 @@ inline long long cl_layout(ClShape& t, const ClSpec& s) {
             mr = std::max(mr, own);
             if (l < T && own < 1) return -1;
         }
-        const int deepH = std::max(l == 0 ? nu1 + 2 : nu1 + 1, 2);
+        const int deepH = std::max((l == 0 ? nu1 : nu1 - 1) + cl_reach_after(nu2), 2);
         const bool dl = deep >= (l == 0 ? 2 : 1) && l < T && covered(deepH);
         if (deep == 2 && l == 0 && !dl) return -1;
         t.H[l] = dl ? deepH : 1;
