@@ -1888,32 +1888,43 @@ static __global__ void k_dense_level(FineDesc fd, double* Adense) {
 }
 
 // Gauss--Jordan inverses (SPD input, no pivoting needed) of the coarsest level's matrices, one cluster
-// of kGjCtas CTAs per matrix.  Bound by FP64 arithmetic: n^3 multiply-adds at about two per cycle and
+// of up to kGjCtas CTAs per matrix.  Bound by FP64 arithmetic: n^3 multiply-adds at about two per cycle and
 // SM, so one CTA needs 9.0 ms for n = 256 while the rest of the chip idles.  Here CTA r keeps rows
-// r, r + kGjCtas, ... in shared memory (in place: column k of the inverse replaces column k of A, half
+// r, r + ctas, ... in shared memory (in place: column k of the inverse replaces column k of A, half
 // the arithmetic of an augmented matrix); the owner of pivot row k + 1 updates and scales that row
 // first and stores it into every CTA's buffer, then all CTAs eliminate their rows with pivot row k,
 // so one cluster barrier per pivot is left.  The same pivots and products as elimination of [A | I].
+// Where no such cluster fits (a device shared out in small parts), smaller ones take its place, at last one CTA
+// whose rows are in the result's memory.
 constexpr int kGjCtas = 16;
 constexpr int kGjThreads = 512;
 
-inline size_t gj_smem(int n) {
-    return ((size_t)((n + kGjCtas - 1) / kGjCtas) * n + 2 * (size_t)n) * sizeof(double);
+// Shared memory: two pivot rows and (staged) a CTA's rows.
+inline size_t gj_smem(int n, int ctas, bool staged) {
+    return ((staged ? (size_t)((n + ctas - 1) / ctas) * n : 0) + 2 * (size_t)n) * sizeof(double);
+}
+// CTAs per cluster: the most whose cluster fits, 0 for one CTA without staged rows.
+template <class Fits> inline int gj_ctas(Fits&& fits) {
+    for (int c = kGjCtas; c >= 1; c /= 2)
+        if (fits(c)) return c;
+    return 0;
 }
 
-static __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan(const double* Ain, double* Inv, int n, int* fail) {
+static __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan(const double* Ain, double* Inv, int n, int ctas,
+                                                                    int staged, int* fail) {
     pdl_prologue();
     extern __shared__ __align__(16) double gj_sm[];
     unsigned rank, mat;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(mat));
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = kGjThreads / 32;
-    const int nr = n > (int)rank ? (n - (int)rank + kGjCtas - 1) / kGjCtas : 0;   // own rows
-    double* prow = gj_sm;                       // two pivot rows, scaled by 1 / pivot
-    double* R = gj_sm + 2 * n;
+    const int nr = n > (int)rank ? (n - (int)rank + ctas - 1) / ctas : 0;   // own rows
     const double* A = Ain + (long long)mat * n * n;
+    double* O = Inv + (long long)mat * n * n;
+    double* prow = gj_sm;                       // two pivot rows, scaled by 1 / pivot
+    double* R = staged ? gj_sm + 2 * n : O;     // (not staged: one CTA, which owns every row)
     for (int i = w; i < nr; i += nw)
-        for (int j = lane; j < n; j += 32) R[i * n + j] = A[(long long)(rank + i * kGjCtas) * n + j];
+        for (int j = lane; j < n; j += 32) R[i * n + j] = A[(long long)(rank + i * ctas) * n + j];
     __syncthreads();
     // row i minus its column k times pivot row k; the pivot's own entry becomes 1 / pivot there, so
     // column k of every other row becomes -f / pivot
@@ -1923,7 +1934,7 @@ static __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan(const double
         for (int j = lane; j < n; j += 32) row[j] = j == k ? -f * pr[j] : row[j] - f * pr[j];
     };
     auto publish = [&](int k) {                 // the owner: scale row k, store it into every CTA
-        double* row = R + (k / kGjCtas) * n;
+        double* row = R + (k / ctas) * n;
         const double piv = row[k];
         if (tid == 0 && !(piv > 0.0)) *fail = 1;
         const double pinv = 1.0 / piv;
@@ -1932,7 +1943,7 @@ static __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan(const double
             const double v = j == k ? pinv : row[j] * pinv;
             row[j] = v;
             double* dst = prow + (k & 1) * n + j;
-            for (unsigned c = 0; c < kGjCtas; ++c) {
+            for (int c = 0; c < ctas; ++c) {
                 unsigned long long q;
                 asm volatile("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"(dst), "r"(c));
                 *reinterpret_cast<double*>(q) = v;
@@ -1948,30 +1959,52 @@ static __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan(const double
     cluster_barrier();
     for (int k = 0; k < n; ++k) {
         const double* pr = prow + (k & 1) * n;
-        const bool ahead = k + 1 < n && (k + 1) % kGjCtas == (int)rank;
-        const int ia = (k + 1) / kGjCtas;
+        const bool ahead = k + 1 < n && (k + 1) % ctas == (int)rank;
+        const int ia = (k + 1) / ctas;
         if (ahead) {
             if (w == 0) eliminate(R + ia * n, pr, k);
             __syncthreads();
             publish(k + 1);                     // buffer (k + 1) & 1: last read before the previous barrier
         }
         for (int i = w; i < nr; i += nw) {
-            if ((int)rank + i * kGjCtas == k || (ahead && i == ia)) continue;
+            if ((int)rank + i * ctas == k || (ahead && i == ia)) continue;
             eliminate(R + i * n, pr, k);
         }
         cluster_barrier();
     }
-    double* O = Inv + (long long)mat * n * n;
+    if (!staged) return;
     for (int i = w; i < nr; i += nw)
-        for (int j = lane; j < n; j += 32) O[(long long)(rank + i * kGjCtas) * n + j] = R[i * n + j];
+        for (int j = lane; j < n; j += 32) O[(long long)(rank + i * ctas) * n + j] = R[i * n + j];
 }
 
 // Invert nmat consecutive n x n matrices; *fail is set when a pivot is not positive.
 inline aao_status launch_gauss_jordan(const double* A, double* Inv, int n, int nmat, int* fail, cudaStream_t st) {
-    AAO_CUDA_TRY(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)gj_smem(kMaxCoarsest)));
+    int dev = 0, optin = 0;
+    AAO_CUDA_TRY(cudaGetDevice(&dev));
+    AAO_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    AAO_CUDA_TRY(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     AAO_CUDA_TRY(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    launch_cluster(k_gauss_jordan, dim3(kGjCtas * nmat), dim3(kGjThreads), gj_smem(n), st, kGjCtas, A, Inv, n, fail);
+    const int c = gj_ctas([&](int ctas) {
+        if (gj_smem(n, ctas, true) > (size_t)optin) return false;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3(kGjThreads);
+        cfg.dynamicSmemBytes = gj_smem(n, ctas, true);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)ctas;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_gauss_jordan, &cfg) == cudaSuccess && fit > 0) return true;
+        cudaGetLastError();
+        return false;
+    });
+    const int ctas = c > 0 ? c : 1;
+    launch_cluster(k_gauss_jordan, dim3((unsigned)(ctas * nmat)), dim3(kGjThreads), gj_smem(n, ctas, c > 0), st, ctas, A, Inv,
+                   n, ctas, c > 0 ? 1 : 0, fail);
     AAO_LAUNCH_CHECK();
     return AAO_OK;
 }
