@@ -133,8 +133,7 @@ struct Handle {
     double* beta = nullptr;        // [0] beta, [1] bnorm
     int* flags = nullptr;          // [0] active, [1] its, [2] nonfinite, [3] breakdown
     double* resid = nullptr;       // 1
-    Red red;                       // reduction scratch
-    int red_cap_items = 0, red_cap_chunks = 0;
+    Red red;                       // scratch of the outer vectors' reductions (kRedChunks partial sums)
 
     // pinned host mirror of the small per-iteration results
     struct Small {
@@ -146,20 +145,17 @@ struct Handle {
     PrecondBase* P = nullptr;
     cudaEvent_t ev[4];
     int ev_ok = 0;
-
-    // reduction blocks per item: about 8 blocks per SM over the whole batch, at
-    // most one 32-column segment per warp
-    int nchunk_for(int B, long long segments) const {
-        // a single small item (the Schur sweep's inner solves): one block per SM, so fewer
-        // partials and atomics on the item's counter; otherwise about eight blocks per SM in total
-        // (enough loads in flight for the long outer vectors)
-        const bool small_single = B == 1 && segments < 152LL * kWarpsPerBlock * 32;
-        long long target = small_single ? 152LL : (152LL * 8 + B - 1) / B;
-        long long maxc = (segments + kWarpsPerBlock - 1) / kWarpsPerBlock;
-        long long c = target < maxc ? target : maxc;
-        if (c > red_cap_chunks) c = red_cap_chunks;
-        return (int)(c < 1 ? 1 : c);
-    }
 };
+
+// Blocks of a reduction over an outer vector of `segments` 32-column segments: about eight per SM (enough loads in flight
+// for the long vectors) or, for small ones, one per SM (fewer partial sums and atomics), at most one segment per
+// warp.
+constexpr int kRedChunks = 152 * 8;
+inline int nchunk_for(long long segments) {
+    const long long target = segments < 152LL * kWarpsPerBlock * 32 ? 152LL : (long long)kRedChunks;
+    const long long maxc = (segments + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    const long long c = target < maxc ? target : maxc;
+    return (int)(c < 1 ? 1 : c);
+}
 
 }  // namespace aao

@@ -417,11 +417,7 @@ class Precond : public PrecondBase {
                 q->nst = q->nv + (long long)s * g0.nx;
                 q->opt.mgrit_m = 0;
                 q->stream = wst[w];
-                // a worker's reductions run concurrently with the others': its own scratch
-                q->red_cap_items = 1;
-                AAO_TRY(ar.alloc(&q->red.partials, (size_t)(q->red_cap_chunks + 1 + 16)));
-                AAO_TRY(ar.alloc(&q->red.count, 1));
-                AAO_CUDA_TRY(cudaMemsetAsync(q->red.count, 0, sizeof(unsigned int), st()));
+                q->red = Red{};        // (a worker's own reductions have its preconditioner's scratch)
                 work[w] = new Precond(q);
                 AAO_TRY(work[w]->setup());
                 work[w]->wsrc = wbuf;

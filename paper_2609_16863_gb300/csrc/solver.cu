@@ -428,11 +428,9 @@ static aao_status setup_handle(Handle* h, const aao_grid* grid, double tau, int 
     AAO_TRY(ar.alloc(&h->flags, 4));
     AAO_TRY(ar.alloc(&h->resid, 1));
     AAO_CUDA_TRY(cudaMemset(h->flags, 0, 4 * sizeof(int)));
-    h->red_cap_chunks = 152 * 8;
-    h->red_cap_items = nt > 1 ? nt : 1;
-    AAO_TRY(ar.alloc(&h->red.partials, (size_t)(h->red_cap_chunks + h->red_cap_items + 16)));
-    AAO_TRY(ar.alloc(&h->red.count, (size_t)h->red_cap_items));
-    AAO_CUDA_TRY(cudaMemset(h->red.count, 0, sizeof(unsigned int) * h->red_cap_items));
+    AAO_TRY(ar.alloc(&h->red.partials, (size_t)kRedChunks));
+    AAO_TRY(ar.alloc(&h->red.count, 1));
+    AAO_CUDA_TRY(cudaMemset(h->red.count, 0, sizeof(unsigned int)));
     AAO_CUDA_TRY(cudaMallocHost((void**)&h->hsmall, sizeof(SmallDev)));
     h->P = make_precond(h, h->opt.prec_P, h->opt.prec_Pint);
     if (!h->P) {
@@ -496,7 +494,7 @@ static aao_status rhs_dev(Handle* h, const double* f, int f_time_dep, const doub
 
 static aao_status norm_dev(Handle* h, const double* v, double* out) {
     const long long rows = h->nst / h->g.n0;
-    dim3 grid(h->nchunk_for(1, rows * ((h->g.n0 + kWarp - 1) / kWarp)), 1);
+    dim3 grid(nchunk_for(rows * ((h->g.n0 + kWarp - 1) / kWarp)), 1);
     Red red = h->red;
     red.nchunk = grid.x;
     launch(k_norm<double>, grid, kBlock, 0, h->stream, h->g.n0, rows, 1, nullptr, v, h->nst, red, out, 1);
@@ -550,7 +548,7 @@ static aao_status fgmres(Handle* h, const double* b, double* x, int x0_given, in
         int total = 0;
         const double tol = h->opt.tol;
         Red red = h->red;
-        red.nchunk = h->nchunk_for(1, rows * ((n0 + kWarp - 1) / kWarp));
+        red.nchunk = nchunk_for(rows * ((n0 + kWarp - 1) / kWarp));
         dim3 rgrid(red.nchunk, 1);
         const PtMap pmo = ptmap(n0);
         const dim3 nbp = pt_grid(pmo, rows, 1), ntp = pt_block(pmo);
@@ -680,7 +678,7 @@ static aao_status fgmres_left(Handle* h, const double* b, double* x, int x0_give
         int total = 0;
         const double tol = h->opt.tol;
         Red red = h->red;
-        red.nchunk = h->nchunk_for(1, rows * ((n0 + kWarp - 1) / kWarp));
+        red.nchunk = nchunk_for(rows * ((n0 + kWarp - 1) / kWarp));
         dim3 rgrid(red.nchunk, 1);
         const PtMap pmo = ptmap(n0);
         const dim3 nbp = pt_grid(pmo, rows, 1), ntp = pt_block(pmo);
