@@ -94,12 +94,6 @@ __device__ __forceinline__ Field<S> field_of(const Vec<S>& v, int b, long long r
     return f;
 }
 
-// 1 / h^2 per axis in the arithmetic type (rounded on the host: no FP64 conversion per thread).
-template <class A> struct InvH2 {
-    A x, y, z;
-};
-template <class A> inline InvH2<A> inv_h2(const Geo& g) { return InvH2<A>{(A)g.hx2, (A)g.hy2, (A)g.hz2}; }
-
 // (K u) at N consecutive columns of row (j, k), FD; P receives u there.  The arithmetic of fd_K.
 template <int N, class S, class A>
 __device__ __forceinline__ void fd_K_n(const Field<S>& u, const Geo& g, const InvH2<A>& h, const Faces<A>& f, int row,

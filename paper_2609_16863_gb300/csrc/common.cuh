@@ -239,6 +239,12 @@ struct Geo {
     double hx2, hy2, hz2;   // 1/h^2 per axis
 };
 
+// 1 / h^2 per axis in the arithmetic type (rounded on the host: no FP64 conversion per thread).
+template <class A> struct InvH2 {
+    A x, y, z;
+};
+template <class A> inline InvH2<A> inv_h2(const Geo& g) { return InvH2<A>{(A)g.hx2, (A)g.hy2, (A)g.hz2}; }
+
 // (j, k) of a grid row without 64-bit division (2D: k = 0).
 __device__ __forceinline__ void row_jk(const Geo& g, long long row, int& j, int& k) {
     if (g.d == 2) {

@@ -26,7 +26,6 @@ template <class S> struct LevelOp {
     const S* sten = nullptr; // coarse: ncoef*nx, component-major
     const float* sten_sc = nullptr;  // coarse, scaled types: one scale per component
     int ncoef = 9;
-    A hx2 = A(0), hy2 = A(0), hz2 = A(0);   // 1 / h^2 of g in the arithmetic type (matrix-free 3D tiles)
 };
 
 template <class S>
@@ -1483,9 +1482,11 @@ template <class A> struct T3Rows {
     __device__ __forceinline__ A operator()(int j, int k, int c) const { return d[((k - k0) * w + j - j0) * n0 + c]; }
 };
 
-// (A u)_P and a_PP of the matrix-free 3D level from u(j, k, c) in shared memory.
+// (A u)_P and a_PP of the matrix-free 3D level from u(j, k, c) in shared memory.  (1 / h^2 comes beside the level: as fields
+// of LevelOp its values would change the register allocation of every kernel that takes one: 96 instead of 118 for
+// k_smooth2<double>, 10% slower.)
 template <class S, class A>
-__device__ __forceinline__ void t3_apply(const LevelOp<S>& op, const T3Rows<A>& u, int j, int k, int c, A& Au, A& diag) {
+__device__ __forceinline__ void t3_apply(const LevelOp<S>& op, const InvH2<A>& h, const T3Rows<A>& u, int j, int k, int c, A& Au, A& diag) {
     const Geo& g = op.g;
     const A uP = u(j, k, c);
     const A uW = c > 0 ? u(j, k, c - 1) : A(0), uE = c + 1 < g.n0 ? u(j, k, c + 1) : A(0);
@@ -1494,10 +1495,10 @@ __device__ __forceinline__ void t3_apply(const LevelOp<S>& op, const T3Rows<A>& 
     const Faces<A>& f = op.faces;
     A Ku, kd;
     if (f.fx == nullptr) {
-        Ku = op.hx2 * (A(2) * uP - uW - uE) + op.hy2 * (A(2) * uP - uS - uN);
-        Ku += op.hz2 * (A(2) * uP - uD - uU);
-        kd = A(2) * op.hx2 + A(2) * op.hy2;
-        kd += A(2) * op.hz2;
+        Ku = h.x * (A(2) * uP - uW - uE) + h.y * (A(2) * uP - uS - uN);
+        Ku += h.z * (A(2) * uP - uD - uU);
+        kd = A(2) * h.x + A(2) * h.y;
+        kd += A(2) * h.z;
     } else {
         const int row = j + g.n1 * k, fxi = row * (g.n0 + 1) + c, fyi = (k * (g.n1 + 1) + j) * g.n0 + c;
         const int fzi = row * g.n0 + c, pl = g.n1 * g.n0;
@@ -1524,8 +1525,8 @@ __device__ __forceinline__ void t3_load(const Geo& g, const View<S>& v, int w, i
 }
 
 template <class S>
-__global__ void __launch_bounds__(kT3Threads) k_smooth2_tile(LevelOp<S> op, const int* active, Vec<S> xin, Vec<S> bv,
-                                                             Vec<S> xout, typename PT<S>::A omega) {
+__global__ void __launch_bounds__(kT3Threads) k_smooth2_tile(LevelOp<S> op, InvH2<typename PT<S>::A> h, const int* active,
+                                                             Vec<S> xin, Vec<S> bv, Vec<S> xout, typename PT<S>::A omega) {
     pdl_prologue();
     using A = typename PT<S>::A;
     extern __shared__ __align__(16) unsigned char t3_smem[];
@@ -1549,7 +1550,7 @@ __global__ void __launch_bounds__(kT3Threads) k_smooth2_tile(LevelOp<S> op, cons
             const A bp = bb.at(j + g.n1 * k, c);
             if (has) {
                 A Au, dg;
-                t3_apply(op, u0, j, k, c, Au, dg);
+                t3_apply(op, h, u0, j, k, c, Au, dg);
                 x1[r * n0 + c] = u0(j, k, c) + omega * (bp - Au) / dg;
             } else {
                 x1[r * n0 + c] = omega * bp / level_diag(op, j + g.n1 * k, j, k, c);
@@ -1564,7 +1565,7 @@ __global__ void __launch_bounds__(kT3Threads) k_smooth2_tile(LevelOp<S> op, cons
         A* x2 = x0 + r * n0;                      // x_in is not read again
         for (int c = lane; c < n0; c += kWarp) {
             A Au, dg;
-            t3_apply(op, u1, j, k, c, Au, dg);
+            t3_apply(op, h, u1, j, k, c, Au, dg);
             x2[c] = u1(j, k, c) + omega * (bb.at(j + g.n1 * k, c) - Au) / dg;
         }
         S* out; float* osc;
@@ -1574,8 +1575,8 @@ __global__ void __launch_bounds__(kT3Threads) k_smooth2_tile(LevelOp<S> op, cons
 }
 
 template <class S>
-__global__ void __launch_bounds__(kT3Threads) k_resid_restrict_tile(LevelOp<S> op, Geo gc, const int* active, Vec<S> xv,
-                                                                    Vec<S> bv, Vec<S> bcv) {
+__global__ void __launch_bounds__(kT3Threads) k_resid_restrict_tile(LevelOp<S> op, InvH2<typename PT<S>::A> h, Geo gc,
+                                                                    const int* active, Vec<S> xv, Vec<S> bv, Vec<S> bcv) {
     pdl_prologue();
     using A = typename PT<S>::A;
     extern __shared__ __align__(16) unsigned char t3_smem[];
@@ -1601,7 +1602,7 @@ __global__ void __launch_bounds__(kT3Threads) k_resid_restrict_tile(LevelOp<S> o
                 res = bb.at(j + g.n1 * k, c);
                 if (has) {
                     A Au, dg;
-                    t3_apply(op, u, j, k, c, Au, dg);
+                    t3_apply(op, h, u, j, k, c, Au, dg);
                     res -= Au;
                 }
             }
@@ -1634,9 +1635,9 @@ __global__ void __launch_bounds__(kT3Threads) k_resid_restrict_tile(LevelOp<S> o
 }
 
 template <class S>
-__global__ void __launch_bounds__(kT3Threads) k_prolong_smooth_tile(LevelOp<S> op, Geo gc, const int* active, Vec<S> xcv,
-                                                                    Vec<S> xin, Vec<S> bv, Vec<S> xout,
-                                                                    typename PT<S>::A omega) {
+__global__ void __launch_bounds__(kT3Threads) k_prolong_smooth_tile(LevelOp<S> op, InvH2<typename PT<S>::A> h, Geo gc,
+                                                                    const int* active, Vec<S> xcv, Vec<S> xin, Vec<S> bv,
+                                                                    Vec<S> xout, typename PT<S>::A omega) {
     pdl_prologue();
     using A = typename PT<S>::A;
     extern __shared__ __align__(16) unsigned char t3_smem[];
@@ -1689,7 +1690,7 @@ __global__ void __launch_bounds__(kT3Threads) k_prolong_smooth_tile(LevelOp<S> o
             val[q] = A(0);
             if (in && c < n0) {
                 A Au, dg;
-                t3_apply(op, u, j, k, c, Au, dg);
+                t3_apply(op, h, u, j, k, c, Au, dg);
                 val[q] = u(j, k, c) + omega * (bb.at(j + g.n1 * k, c) - Au) / dg;
             }
         }

@@ -712,9 +712,6 @@ class Precond : public PrecondBase {
         LevelOp<SI> op;
         op.g = lev[l].g;
         op.ncoef = op.g.d == 3 ? 27 : 9;
-        op.hx2 = (A)op.g.hx2;
-        op.hy2 = (A)op.g.hy2;
-        op.hz2 = (A)op.g.hz2;
         if (l == 0 && !h->q1) {
             op.fine = 1;
             op.sigma = A(1);
@@ -930,7 +927,7 @@ class Precond : public PrecondBase {
             bytes_hint((cur.d ? 3.0 : 2.0) * nact * g.nx * sizeof(SI));
             if (tiles)
                 launch(k_smooth2_tile<SI>, t3_grid(g.n1, g.n2, kT3, B), kT3Threads, t3_smem_smooth2(g.n0, sizeof(A)), st(),
-                       op, act, cur, b, d, om);
+                       op, inv_h2<A>(g), act, cur, b, d, om);
             else launch(k_smooth2<SI>, pbl, pth, 0, st(), op, pm, B, act, cur, b, d, om);
             cur = d;
             q = 2;
@@ -946,7 +943,7 @@ class Precond : public PrecondBase {
             bytes_hint(((cur.d ? 2.0 : 1.0) * g.nx + gc.nx) * nact * sizeof(SI));
             if (tiles)
                 launch(k_resid_restrict_tile<SI>, t3_grid(gc.n1, gc.n2, kT3 / 2, B), kT3Threads,
-                       t3_smem_restrict(g.n0, sizeof(A)), st(), op, gc, act, cur, b, lev[l + 1].Bb);
+                       t3_smem_restrict(g.n0, sizeof(A)), st(), op, inv_h2<A>(g), gc, act, cur, b, lev[l + 1].Bb);
             else launch(k_resid_restrict<SI>, cbl, cth, 0, st(), op, gc, pmc, B, act, cur, b, lev[l + 1].Bb);
         } else if (cur.d == nullptr) {
             bytes_hint(1.0 * nact * (g.nx + gc.nx) * sizeof(SI));
@@ -966,7 +963,7 @@ class Precond : public PrecondBase {
             bytes_hint(1.0 * nact * (gc.nx + (cur.d ? 3.0 : 2.0) * g.nx) * sizeof(SI));
             if (tiles)
                 launch(k_prolong_smooth_tile<SI>, t3_grid(g.n1, g.n2, kT3, B), kT3Threads, t3_smem_prolong(g.n0, sizeof(A)),
-                       st(), op, gc, act, lev[l + 1].X, cur, b, d, om);
+                       st(), op, inv_h2<A>(g), gc, act, lev[l + 1].X, cur, b, d, om);
             else launch(k_prolong_smooth<SI>, pbl, pth, 0, st(), op, gc, pm, B, act, lev[l + 1].X, cur, b, d, om);
             cur = d;
             q = 1;
