@@ -2,7 +2,7 @@
 // three V-cycles per stage solve).
 //
 // The V-cycles of one shifted solve are a chain of about 30 dependent grid-wide steps per cycle.  One
-// thread-block cluster per item (16 CTAs for single items, 8 for batches) runs the chain on chip:
+// thread-block cluster per item (16 CTAs for single items, 8, 4 or 2 for batches) runs the chain on chip:
 //   * every level above the coarsest is split by grid rows over the CTAs; a CTA keeps its rows of x (two
 //     ping-pong buffers), b, the stored stencil and the Jacobi weights in shared memory, with H ghost
 //     rows on each side and zero columns beside the grid (the Dirichlet boundary);

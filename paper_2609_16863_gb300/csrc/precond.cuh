@@ -492,9 +492,9 @@ class Precond : public PrecondBase {
 
     // Plan the cluster-resident shifted solve: 2D, at least one level above the coarsest, every
     // CTA owning rows of every distributed level, its share within shared memory, and the cluster
-    // co-resident on the device.  Two plans: one for single items (16 CTAs where a layout
-    // fits, else 8) and one for batches (8 CTAs, so that about twice as many items run at once:
-    // at 256^2 only 7 clusters of 16 are resident).  deep: ghost rows for whole smoothing phases (1: on
+    // co-resident on the device.  Up to four plans: one for single items (16 CTAs where a layout
+    // fits, else 8) and others for batches (8, 4 and 2 CTAs, so that more items run at once: 7 clusters of 16 are
+    // resident, 15 of 8, 36 of 4, 76 of 2).  deep: ghost rows for whole smoothing phases (1: on
     // the coarse levels, 2: on the finest too), else one ghost row.  lean: what is read from global
     // memory (L2) instead of being staged: 1: the rows of A_c^{-1}, 2: the first coarse stencil, 3: every
     // coarse stencil.  All give the same values.
@@ -983,34 +983,56 @@ class Precond : public PrecondBase {
         return AAO_OK;
     }
 
+    // us of three cycles of B items on the clusters of a plan: waves of resident clusters times a launch, whose
+    // steps cost 14 us per distributed level and 5.5 us per 1000 points of a CTA beyond 2500, 15% more where every sweep on
+    // the finest level is followed by an exchange (FP64: 22 and 55 per 1000 points); per sweep, relative to V(2,2)-cycles.
+    double cluster_cost(const ClPlan& pl, int B) const {
+        const double per = (double)h->g.nx / pl.C, sweeps = h->opt.mg_pre + h->opt.mg_post;
+        const double launch = std::is_same<A, double>::value
+                                  ? (22.0 * (L - 1) + 55e-3 * per) * (0.42 + 0.145 * sweeps)
+                                  : (14.0 * (L - 1) + 5.5e-3 * std::max(0.0, per - 2500.0)) * (0.66 + 0.085 * sweeps) *
+                                        (pl.ctx[0].H[0] > 1 ? 1.0 : 1.15);
+        return launch * ((B + pl.resident - 1) / pl.resident);
+    }
+    // The same on the level kernels: the tail, an SM per item, and each level above it by its points, less where whole batches
+    // stream (kFuseMaxPoints), least on the finest level with kappa = 1 and rows of whole vectors.
+    double levels_cost(int B) const {
+        const bool f64 = std::is_same<A, double>::value;
+        const int lc = tails[B > 1 ? 1 : 0].lc, sweeps = h->opt.mg_pre + h->opt.mg_post;
+        const double tail = (f64 ? 93.0 + 121e-3 * lev[lc].g.nx : 113.0 + 17.5e-3 * lev[lc].g.nx) * ((B + 151) / 152);
+        double above = 0.0;
+        for (int l = 0; l < lc; ++l) {
+            const long long points = (long long)B * lev[l].g.nx;
+            const bool vectors = lev[l].g.n0 % kVN == 0 && (l > 0 || (!h->q1 && !h->has_kappa));
+            const double us = points <= kFuseMaxPoints ? (f64 ? 1.7e-3 : 0.36e-3)
+                              : vectors                ? (f64 ? 0.45e-3 : 0.061e-3)
+                                                       : (f64 ? 0.68e-3 : 0.12e-3);
+            above += us * (double)points;
+        }
+        return (tail + above) * (f64 ? 0.28 + 0.18 * sweeps : 0.56 + 0.11 * sweeps);
+    }
     // The cluster plan of a batch, or null: the level kernels.  16-bit storage: 8 CTAs per item from kClBatch8
-    // items on, up to kClMaxBatch items.  Else the plan with the least waves of resident clusters times the time
-    // of a launch, unless the level kernels are faster.  Measured (us per three V-cycles with their share of the
-    // Krylov kernels, B items; level kernels / 16 / 8 / 4 / 2 CTAs per item):
-    //   FP32 128^2, B = 1: 275 / 62 / 65 / 71 / 94; B = 64: 574 / 465 / 264 / 143 / 116
-    //   FP32 64^2, B = 64: 209 / 322 / 166 / 83 / 60; 256^2, B = 128: 939 / 1390 / 949 / - / -
-    //   FP64 64^2, B = 32: 615 / 310 / 221 / 122 / 177; 256^2, B = 128: 5431 / 5602 / - / - / -
-    // The model: a launch takes 22 + 14 T us on T distributed levels and 5.5 us per 1000 points of a CTA's rows
-    // beyond 2500 (FP64: 20 + 25 T and 50 us per 1000 beyond 400); the level kernels 0.105 us per 1000 points
-    // (FP64: 0.62) and 150 us per 148 items.  It reproduces the figures above to about 15%; the level kernels are
-    // taken unless a plan is faster by 10%.
+    // items on, up to kClMaxBatch items.  Else the plan of the least cost if that is below 0.8 of the level kernels'.  The
+    // costs are fitted to inner solves of one step (two shifted solves; us, level kernels / 16 / 8 / 4 / 2 CTAs per item):
+    //   FP32 64^2, B = 64: 455 / 674 / 372 / 202 / 157; 127 x 95, B = 24: 583 / 451 / 285 / 204 / 228;
+    //   256^2, B = 64: 1873 / 1549 / 1119 / - / -, B = 128: 1726 / 2876 / 1969 / - / -
+    //   FP64 64^2, B = 40: 1271 / 803 / 524 / 504 / 433; 127 x 95, B = 40: 2667 / 1441 / 1030 / 1070 / -;
+    //   128^2, B = 256: 5618 / 9094 / 6599 / 5200 / -; 256^2, B = 40: 5842 / 4099 / - / - / -,
+    //   B = 128: 9936 / 12708 / - / - / -
+    // with about 70 us of Krylov kernels in each.  Over kappa, Q1, 1 and 3 cycles, one to six sweeps, 32^2 to 256^2 and 1 to 256
+    // items the choice costs 17% more than the best one at most, 0.6% on average.
     const ClPlan* pick_cluster(int B) const {
         if (cl_C == 0) return nullptr;
         if constexpr (PT<SI>::scaled) {
             if (B > kClMaxBatch) return nullptr;
             return B >= kClBatch8 && clp[1].C > 0 ? &clp[1] : &clp[0];
         }
-        const bool f64 = std::is_same<A, double>::value;
-        const double nx = (double)h->g.nx;
-        const double levels = (f64 ? 0.62e-3 : 0.105e-3) * nx * B + 150.0 * ((B + 147) / 148);
         const ClPlan* best = nullptr;
-        double cost = B > kClMaxBatch ? 0.9 * levels : 1e300;
+        // (a batch of one wave of the largest clusters: the level kernels are launch-bound there)
+        double cost = B <= clp[0].resident ? 1e300 : 0.8 * levels_cost(B);
         for (const ClPlan& pl : clp) {
             if (pl.C == 0) continue;
-            const double per = nx / pl.C;
-            const double t = f64 ? 20.0 + 25.0 * (L - 1) + 50e-3 * std::max(0.0, per - 400.0)
-                                 : 22.0 + 14.0 * (L - 1) + 5.5e-3 * std::max(0.0, per - 2500.0);
-            const double c = t * ((B + pl.resident - 1) / pl.resident);
+            const double c = cluster_cost(pl, B);
             if (c < cost) {
                 cost = c;
                 best = &pl;
@@ -1087,7 +1109,7 @@ class Precond : public PrecondBase {
     static bool aligned16(const void* p) { return (reinterpret_cast<unsigned long long>(p) & 15ULL) == 0; }
 
     // Blocks per item of the Arnoldi kernels: one position per thread while that gives fewer than kArBlocks
-    // blocks (eight per SM) over the batch, else the blocks stride over the item.
+    // blocks (48 per SM) over the batch, else the blocks stride over the item.
     ArRed ar_red(int B, long long positions) const {
         const long long full = (positions + kArThreads - 1) / kArThreads, cap = (kArBlocks + B - 1) / B;
         ArRed r;
