@@ -209,7 +209,7 @@ __device__ __forceinline__ double to_fp64(double v) { return v; }
 template <int MV, class A, class F>
 __device__ __forceinline__ bool ar_reduce(const A* v, unsigned mask, const ArRed& red, double* sum, F&& preload) {
     // FP64 adds run at two per cycle and SM, and summing each value by shuffles in every warp would take longer than
-    // the launch's other work (37 us of them in k_theta_dots on 128 items of 256^2): so the threads' FP32 values meet in
+    // the launch's other work (45 us of k_theta_dots on 128 items of 256^2): so the threads' FP32 values meet in
     // shared memory and one warp per value adds four per lane before its shuffles, 8 adds per value instead of 23.
     constexpr bool kF32 = std::is_same<A, float>::value;
     __shared__ A sh[MV][kF32 ? kArThreads : kArWarps];
@@ -653,8 +653,9 @@ __device__ __forceinline__ float to_arith(double d, float) {
 __device__ __forceinline__ double to_arith(double d, double) { return d; }
 
 // t = K z_{v,n} (every stage's right-hand side: one copy) and the start of the step's inner solves with
-// ||r|| = sqrt(s) ||t||.  K z in FP64, rounded once to A: it cancels to 1e-4 of its terms on the finest grids.
-template <class A>
+// ||r|| = sqrt(s) ||t||.  K z in FP64, rounded once to A: it cancels to 1e-4 of its terms on the finest grids.  (Q1 and FD
+// apart: with both in one kernel 14 items of 256^2 took 48 us instead of 25; double-float sums took 18.)
+template <class A, bool Q1M>
 __global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, int s, const StepPtrs* sp, int stride, A* t,
                                                             SpaceOp<A> sop, ArRed red, ArItems it) {
     pdl_prologue();
@@ -668,7 +669,9 @@ __global__ void __launch_bounds__(kArThreads) k_schur_start(Geo g, int s, const 
         const int row = (int)(q / (unsigned)g.n0), c = (int)(q - row * g.n0);
         int j, k;
         row_jk(g, row, j, k);
-        const A v = (A)op_K(z, g, sop, row, j, k, c);
+        A v;
+        if constexpr (Q1M) v = (A)op_K(z, g, sop, row, j, k, c);
+        else v = (A)fd_K(z, g, sop.faces, row, j, k, c);
         tb[q] = v;
         acc += v * v;
     }

@@ -10,8 +10,8 @@ namespace aao {
 
 constexpr int kClMax = 16;            // CTAs per cluster (16 needs the non-portable size)
 constexpr int kClThreads = 512;
-constexpr int kClMaxBatch = 32;       // batches of at most this many items run one cluster per item
-constexpr int kClBatch8 = 8;          // batches of at least this many items take the 8-CTA plan
+constexpr int kClMaxBatch = 32;       // 16-bit storage: batches of at most this many items run one cluster per item
+constexpr int kClBatch8 = 8;          // 16-bit storage: batches of at least this many items take the 8-CTA plan
 constexpr int kClPad = 4;             // columns before a row's first point and after its last vector: rows
                                       // start 16-byte aligned, the columns beside the grid are zero
 constexpr int kClReach = 3;           // CTAs on either side whose ghost rows may hold a CTA's rows

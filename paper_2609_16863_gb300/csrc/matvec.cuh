@@ -27,7 +27,7 @@ namespace aao {
 // rounding of the row's size is left (rms error of the stages 0.89e-16; with K v first 1.21e-16).  Every load of a thread is issued
 // before its arithmetic; a warp per row with its columns in a loop left the FP64 pipe idle for a third of the time.
 // Measured: 256^2, s = 3, 128 steps 905 -> 655 us (36 operations per point and block: 0.46 TFMA/s of 0.60);
-// 49 x 45 x 41 with faces, s = 2, 24 steps, transposed 256 -> 162 us; 32^2, 16 steps 5.5 -> 4.2 us.
+// 49 x 45 x 41 with faces, s = 2, 24 steps, transposed 256 -> 141 us; 32^2, 16 steps 5.5 -> 4.2 us.
 // ---------------------------------------------------------------------------
 constexpr int kMvThreads = 128;
 

@@ -1268,8 +1268,10 @@ class Precond : public PrecondBase {
         const Geo& g = h->g;
         const int s = h->s;
         const ArRed red = ar_red(B, g.nx / 4 + 1);        // four points per thread: the reduction is the larger part
-        launch(k_schur_start<A>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g, s,
-               (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
+        with_int(h->q1 != 0, [&](auto q1) {
+            launch(k_schur_start<A, decltype(q1)::value>, dim3((unsigned)red.nchunk, (unsigned)B), kArThreads, 0, st(), g, s,
+                   (const StepPtrs*)stepp, stride, tbuf, sopA, red, ar_items());
+        });
         scale_basis<A>(B, tbuf, g.nx, (const double*)betah, 1LL, V0, 1, stepp);
         AAO_LAUNCH_CHECK();
         AAO_TRY(arnoldi(B, 0));
