@@ -32,7 +32,7 @@
 //     it in registers; on the finest level (FD, kappa = 1) the modes' constants are folded.  Rows are padded
 //     to whole vectors with zeros, so odd widths take the same path.
 //
-// One launch of three V(2,2)-cycles, one item on 16 CTAs (event-timed, with a step per exchange and two-sided index work ->
+// One launch of three V(2,2)-cycles, one item on 16 CTAs (event-timed; with one ghost row and an exchange after every step ->
 // now): FP32 256^2 77.3 -> 69.2 us, 128^2 52.8 -> 46.7, 127 x 95 56.9 -> 46.7, 64^2 38.5 -> 32.9, Q1 80 x 72 51.9 -> 48.7;
 // FP64 256^2 331 -> 308 (FP64-bound), 128^2 129 -> 118, 64^2 67.2 -> 62.1, 32^2 44.6 -> 37.5; eight to fifteen items of 256^2
 // on 8 CTAs each 97 -> 93.  Deep ghost regions against single ghost rows on this kernel: 256^2 68 against 82, 64^2 FP64
