@@ -1890,9 +1890,9 @@ static __global__ void k_dense_level(FineDesc fd, double* Adense) {
 
 // Gauss--Jordan inverses (SPD input, no pivoting needed) of the coarsest level's matrices, one cluster
 // of up to kGjCtas CTAs per matrix.  Bound by FP64 arithmetic: n^3 multiply-adds at about two per cycle and
-// SM, so one CTA needs 9.0 ms for n = 256 while the rest of the chip idles (16 CTAs: 1.2 ms, three matrices at once).  Here CTA r keeps rows
-// r, r + ctas, ... in shared memory (in place: column k of the inverse replaces column k of A, half
-// the arithmetic of an augmented matrix); the owner of pivot row k + 1 updates and scales that row
+// SM, so one CTA needs 9.0 ms for n = 256 while the rest of the chip idles (16 CTAs: 1.2 ms, three matrices at once).
+// Here CTA r keeps rows r, r + ctas, ... in shared memory (in place: column k of the inverse replaces column k of A,
+// half the arithmetic of an augmented matrix); the owner of pivot row k + 1 updates and scales that row
 // first and stores it into every CTA's buffer, then all CTAs eliminate their rows with pivot row k,
 // so one cluster barrier per pivot is left.  The same pivots and products as elimination of [A | I].
 // Where no such cluster fits (a device shared out in small parts), smaller ones take its place, at last one CTA
